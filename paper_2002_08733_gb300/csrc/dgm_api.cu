@@ -175,6 +175,7 @@ struct dgm_plan {
     int64_t n_facets = 0;            // interior facets
     size_t off_sfid = 0;             // [4][K] int32: (facet << 1) | owner, or -1
     size_t off_fcp = 0;              // [FC_ROWS][K] precomputed face constants (plan precision)
+    size_t off_fct = 0;              // [TG_ROWS][K] tangential face constants (plan precision)
     std::vector<int32_t> sfid_host;
     void* hs[2] = {nullptr, nullptr};
     void* hs_res = nullptr;
@@ -422,6 +423,8 @@ static int plan_create(dgm_plan** out, int64_t nv, const double* xyz, int64_t nt
     off = align256(off + sizeof(int32_t) * 4 * K);
     P->off_fcp = off;    // precomputed face constants of the stage kernels
     off = align256(off + size_t(kt->real_size) * FC_ROWS * K);
+    P->off_fct = off;    // constants of the tangential-trace kernels
+    off = align256(off + size_t(kt->real_size) * TG_ROWS * K);
     P->off_tmap = off;   // tensor maps of the phase-1 bulk copies
     off = align256(off + size_t(TMAP_SETS) * TMAP_COUNT * TMAP_BYTES);
     P->bytes_geom = off;
@@ -511,21 +514,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder() {
     return fn;
 }
 
-// Tensor maps of the stage kernels' phase-1 bulk copies (TmapIndex), for the
-// bound field buffers, the element constants and the face-constant table.
-// Built when each element has one column (S = 1: a tile's columns are
-// consecutive elements in every table) and every row starts on a 16-byte
-// boundary; otherwise, or when the driver has no encoder, the kernels keep
-// their per-thread loads.  The maps hold addresses only, so they stay valid
-// until the next bind.
 static_assert(sizeof(CUtensorMap) == TMAP_BYTES, "tensor-map slot size");
-
-// tile width of a tensor-map set: rows of 128 bytes (set 0), 16 FP32 columns
-// (set 1, FP32 plans only); 0 when the set does not exist for the plan
-static cuuint32_t tmap_tile(const dgm_plan* P, int set) {
-    const int rs = P->kt->real_size;
-    return set == 0 ? cuuint32_t(128 / rs) : (rs == 4 ? 16u : 0u);
-}
 
 static bool tmap_encode(const dgm_plan* P, CUtensorMap* out, void* base, cuuint32_t rank,
                         const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
@@ -539,17 +528,16 @@ static bool tmap_encode(const dgm_plan* P, CUtensorMap* out, void* base, cuuint3
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// the field-shaped buffer `base` ([6][N][C], C = K) into map `slot` of every
+// the field-shaped buffer `base` ([6][N][C], C = K S) into map `slot` of every
 // set of the host copy; false if a buffer is misaligned or the encoder refuses
 static bool tmap_fields(dgm_plan* P, void* base, int slot) {
     if (reinterpret_cast<uintptr_t>(base) % 16 != 0) return false;
-    const cuuint64_t row = cuuint64_t(P->mesh.K) * cuuint64_t(P->kt->real_size);
-    const cuuint64_t dims[3] = {cuuint64_t(P->mesh.K), cuuint64_t(P->N), 6};
+    const cuuint64_t C = cuuint64_t(P->mesh.K) * cuuint64_t(P->opt.n_columns);
+    const cuuint64_t row = C * cuuint64_t(P->kt->real_size);
+    const cuuint64_t dims[3] = {C, cuuint64_t(P->N), 6};
     const cuuint64_t str[2] = {row, row * cuuint64_t(P->N)};
     for (int set = 0; set < TMAP_SETS; ++set) {
-        const cuuint32_t te = tmap_tile(P, set);
-        if (te == 0) continue;
-        const cuuint32_t box[3] = {te, cuuint32_t(P->N), 6};
+        const cuuint32_t box[3] = {cuuint32_t(tmap_columns(set)), cuuint32_t(P->N), 6};
         if (!tmap_encode(P, &P->tmap_host[size_t(set) * TMAP_COUNT + slot], base, 3, dims, str, box))
             return false;
     }
@@ -565,30 +553,30 @@ static int tmap_upload(dgm_plan* P) {
     return e == cudaSuccess ? DGM_OK : cuda_fail(e, "upload tensor maps");
 }
 
-// Tensor maps of the stage kernels' phase-1 bulk copies (TmapIndex), for the
-// bound field buffers, the element constants and the face-constant table.
-// Built when each element has one column (S = 1: a tile's columns are
-// consecutive elements in every table) and every row starts on a 16-byte
-// boundary; otherwise, or when the driver has no encoder, the kernels keep
-// their per-thread loads.  The maps hold addresses only, so they stay valid
-// until the next bind.
+// Tensor maps of the stage kernels' tile copies (TmapIndex): the bound field
+// buffers, and for stage_kernel (FP32, one column per element) the element
+// constants and the face-constant table.  Built when every row starts on a
+// 16-byte boundary (a tile then does too) and, with several columns per element,
+// an element's columns fill whole 16-byte units; otherwise, or when the driver
+// has no encoder, the kernels keep their per-thread loads.  The maps hold
+// addresses only, so they stay valid until the next bind.
 static int build_tmaps(dgm_plan* P) {
     P->tmaps_ok = false;
     const int rs = P->kt->real_size;
-    const int64_t K = P->mesh.K;
+    const int64_t K = P->mesh.K, S = P->opt.n_columns;
     // (mixed-order plans run their own kernel on fields of 3 (N + N_H) rows)
-    if (P->mixed || P->opt.n_columns != 1 || K <= 0 || (K * rs) % 16 != 0 || K >= (int64_t(1) << 31))
+    if (P->mixed || K <= 0 || (K * S * rs) % 16 != 0 || (S > 1 && (S * rs) % 16 != 0) ||
+        K * S >= (int64_t(1) << 31))
         return DGM_OK;
     if (tmap_encoder() == nullptr) return DGM_OK;
     P->tmap_host.assign(size_t(TMAP_SETS) * TMAP_COUNT, CUtensorMap{});
     for (int b = 0; b < 2; ++b)
         if (P->fields[b] != nullptr && !tmap_fields(P, P->fields[b], TM_U0 + b)) return DGM_OK;
     const cuuint64_t Ke = cuuint64_t(K), row = cuuint64_t(K) * cuuint64_t(rs);   // row stride in bytes
-    unsigned char* geo = P->geom + (rs == 8 ? P->off_geo : P->off_geo32);
+    unsigned char* geo = P->geom + P->off_geo32;
     unsigned char* fcp = P->geom + P->off_fcp;
-    for (int set = 0; set < TMAP_SETS; ++set) {
-        const cuuint32_t te = tmap_tile(P, set);
-        if (te == 0) continue;
+    for (int set = 0; set < TMAP_SETS && rs == 4 && S == 1; ++set) {
+        const cuuint32_t te = cuuint32_t(tmap_columns(set));
         CUtensorMap* m = P->tmap_host.data() + size_t(set) * TMAP_COUNT;
         bool ok = true;
         {   // element constants [G_COUNT][K]
@@ -633,7 +621,8 @@ static int build_face_table(dgm_plan* P) {
     stage_params(P, prm);
     const bool sip = P->sip_alpha > 0.0;
     prm.sfid = sip ? reinterpret_cast<const int32_t*>(P->geom + P->off_sfid) : nullptr;
-    const int rc = launch_face_consts(prm, P->kt->real_size, sip, P->geom + P->off_fcp, P->stream);
+    int rc = launch_face_consts(prm, P->kt->real_size, false, P->geom + P->off_fcp, P->stream);
+    if (!rc) rc = launch_tang_consts(prm, P->kt->real_size, sip, P->geom + P->off_fct, P->stream);
     return rc ? fail(rc, "face constants") : DGM_OK;
 }
 
@@ -741,6 +730,8 @@ static void stage_params(dgm_plan* P, StageParams& prm) {
     prm.sip_alpha = P->sip_alpha;
     prm.n_facets = P->n_facets;
     prm.fcp = P->geom + P->off_fcp;
+    prm.fct = P->geom + P->off_fct;
+    prm.recorded = P->kt->real_size == 4 && P->n_rec > 0;
     if (P->tmaps_ok && P->tile_loads == 0) {   // phase-1 bulk copies (the launchers pick the map)
         prm.tmaps = P->geom + P->off_tmap;
         prm.tm_f0 = P->fields[0];

@@ -104,6 +104,7 @@ struct StageParams {
     void* raw;            // MODE_RAW: right-hand side before the mass inverse [6][N][K][S]
     void* jumps;          // MODE_RAW: physical face jumps dE, dH [4][6][NF][K][S]
     int32_t variant;      // tile-shape variant of the LSRK stage kernel (autotuner)
+    int32_t recorded;     // FP32 plan with receivers: stage_kernel (its rounding), not tang_kernel
     int32_t force_index64;// 1: 64-bit index arithmetic even where 32 bits suffice
     int32_t tile_groups;  // tile visiting order: G interleaved segments (1: in order)
     const void* tc_b;     // tensor-core variant: B operand image (TcShape<P>::B_BYTES), or null
@@ -122,6 +123,7 @@ struct StageParams {
     double sip_alpha;
     int64_t n_facets;
     const void* fcp;      // precomputed face constants [FC_ROWS][K] (R), see face_consts_kernel
+    const void* fct;      // tangential face and element constants [TG_ROWS][K] (R), see tang_consts_kernel
     // Tiled bulk copies of the stage kernel's phase 1 (null: per-thread loads).
     // tmaps: the plan's tensor maps in device memory, TMAP_SETS sets of TMAP_COUNT
     // (one set per tile width; see TmapIndex); tm_f0 / tm_f1: the field buffers
@@ -150,14 +152,18 @@ constexpr int TMAP_BYTES = 128;
 // face constants per face (15, or 16 with the penalty) of the 16 per face of
 // the table, metric, A^T
 constexpr int TM_ROWS_EG = 16, TM_ROWS_FC = 15, TM_ROWS_FACE = 16, TM_ROWS_GM = 6, TM_ROWS_GA = 9;
-// set 0: tiles of 128 bytes per row (32 FP32 or 16 FP64 columns); set 1: 16 FP32 columns
-constexpr int TMAP_SETS = 2;
+constexpr int TMAP_SETS = 2;   // set 0: 32 columns, set 1: 16 columns
+constexpr int tmap_columns(int set) { return set == 0 ? 32 : 16; }
 
 // Rows per element of the precomputed face constants: 4 faces x 16, the
 // metric A^T A (6), A^T (9).
 constexpr int FC_ROWS = 4 * 16 + 6 + 9;
 // Computes them for a plan (dgm_facec.cu); real_size 4 or 8.
 int launch_face_consts(const StageParams& prm, int real_size, bool sip, void* out, void* stream);
+// Rows per element of the tangential face-constant table (dgm_tang.cuh): per face
+// 8, the metric A^T A (6), two mass factors, the penalty's 4 x 7; and its launcher.
+constexpr int TG_ROWS = 4 * 8 + 6 + 2 + 4 * 7;
+int launch_tang_consts(const StageParams& prm, int real_size, bool sip, void* out, void* stream);
 
 // One adjoint stage: lu += dt F_u^T lr, and the material-gradient terms
 // dt lr . (dF/d eps_T, dF/d mu_T) u at the stage input u (per column).

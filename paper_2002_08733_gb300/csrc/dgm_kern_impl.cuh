@@ -114,18 +114,11 @@ int launch_mode(const StageParams& prm, cudaStream_t st) {
                                                : launch_pair_ix<int64_t>(q, grid, st);
 }
 #else
-// the interior penalty's kernels: LSRK and right-hand-side modes, default tile shape
-#if !defined(DGM_TE) && !defined(DGM_TC)
-constexpr bool kSIP = (DGM_MODE == MODE_LSRK || DGM_MODE == MODE_RHS);
-#else
-constexpr bool kSIP = false;
-#endif
-
-template <typename IX, bool SIP>
+template <typename IX>
 int launch_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
-    constexpr size_t smem = stage_smem_bytes<kP, Real, kTE, kTC, SIP>();
+    constexpr size_t smem = stage_smem_bytes<kP, Real, kTE, kTC>();
     static bool configured = false;
-    auto k = stage_kernel<kP, Real, kTE, kNT, DGM_MODE, IX, kTC, SIP>;
+    auto k = stage_kernel<kP, Real, kTE, kNT, DGM_MODE, IX, kTC>;
     if (kTC && q.tc_b == nullptr) return DGM_EUNSUP;   // no operator image for this plan
     if (!configured) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
@@ -160,21 +153,15 @@ int launch_mode(const StageParams& prm, cudaStream_t st) {
     // phase-1 bulk copies: the plan's tensor-map set of this tile width (rows
     // of 128 bytes, or 16 FP32 columns) and the map of this stage's input
     q.tm_u = -1;
-    constexpr int kSet = kTC ? -1 : (kTE * int(sizeof(Real)) == 128 ? 0 : (sizeof(Real) == 4 && kTE == 16 ? 1 : -1));
+    constexpr int kSet = kTC || sizeof(Real) == 8 ? -1 : kTE == tmap_columns(0) ? 0 : kTE == tmap_columns(1) ? 1 : -1;
     if (kSet >= 0 && q.tmaps != nullptr && q.S == 1) {
         q.tmaps = static_cast<const char*>(q.tmaps) + size_t(kSet) * TMAP_COUNT * TMAP_BYTES;
         q.tm_u = q.u == q.tm_f0 ? TM_U0
                  : q.u == q.tm_f1 ? TM_U1
                  : (q.tm_fw != nullptr && q.u == q.tm_fw) ? TM_UW : -1;
     }
-    if (q.hs != nullptr) {   // interior penalty
-        if constexpr (kSIP) {
-            return i32 ? launch_ix<uint32_t, true>(q, grid, st) : launch_ix<int64_t, true>(q, grid, st);
-        } else {
-            return DGM_EUNSUP;
-        }
-    }
-    return i32 ? launch_ix<uint32_t, false>(q, grid, st) : launch_ix<int64_t, false>(q, grid, st);
+    if (q.hs != nullptr) return DGM_EUNSUP;   // the interior penalty: tang_kernel only
+    return i32 ? launch_ix<uint32_t>(q, grid, st) : launch_ix<int64_t>(q, grid, st);
 }
 #endif
 

@@ -1,103 +1,141 @@
 // Dispatch tables over the per-(degree, precision, mode) kernel modules.
-// FP32 LSRK stage variants for the autotuner: 0 = 32 columns x 384 threads,
-// 1 = 32 x 192, 2 = 16 x 192, and up to p = 3 (where 64 columns of pairs fit
-// in shared memory) 3 = paired kernel with packed FP32x2 arithmetic,
-// 4 = paired kernel with scalar arithmetic; at p >= 4 (one CTA per SM)
-// 3 = 32 x 512; at p = 2, 3 also 5 = tensor-core variant (64 columns x 512
-// threads, curl and lift on tcgen05).
+//
+// tang_kernel (dgm_tang.cuh) is the default; FP32 LSRK variants for the
+// autotuner: 0 = the shape measured best, 1 = 32 columns x 8 threads per column
+// (p >= 4: x 4), 2 = 16 columns x 8, p >= 4: 3 = 32 x 8 with more registers; up to
+// p = 3 (where 64 columns of pairs fit in shared memory) 3 = paired kernel with
+// packed FP32x2 arithmetic, 4 = paired kernel with scalar arithmetic; at p = 2, 3
+// also 5 = tensor-core variant (64 columns x 512 threads, curl and lift on tcgen05).
+//
+// FP32 plans with receivers (prm.recorded) run stage_kernel (dgm_stage.cuh) in
+// the LSRK and leapfrog modes: receiver records and the adjoint's gradients are
+// FP64 results formed from FP32 fields, and what was recorded before stays
+// reproducible to FP64 accuracy only if the fields keep their rounding.  Its
+// variants: 0 = 32 columns x 384 threads, 1 = 32 x 192, 2 = 16 x 192, p >= 4:
+// 3 = 32 x 512.
 #include "dgm_internal.h"
 #include "dgmax.h"
 
 namespace dgm {
 
-int launch_p1_f32_rhs(const StageParams&, void*);
+int launch_t_p1_f32_lsrk(const StageParams&, void*);
+int launch_t_p1_f32_rhs(const StageParams&, void*);
+int launch_t_p1_f32_lf(const StageParams&, void*);
+int launch_t_p1_f32_lfh(const StageParams&, void*);
+int launch_p1_f32_raw(const StageParams&, void*);
+int launch_t_p1_f32_lsrk_v1(const StageParams&, void*);
+int launch_t_p1_f32_lsrk_v2(const StageParams&, void*);
 int launch_p1_f32_lsrk(const StageParams&, void*);
 int launch_p1_f32_lfe(const StageParams&, void*);
 int launch_p1_f32_lfh(const StageParams&, void*);
-int launch_p1_f32_raw(const StageParams&, void*);
-int launch_p1_f32_adj(const AdjParams&, void*);
 int launch_p1_f32_lsrk_v1(const StageParams&, void*);
 int launch_p1_f32_lsrk_v2(const StageParams&, void*);
 int launch_p1_f32_lsrk_v3(const StageParams&, void*);
 int launch_p1_f32_lsrk_v4(const StageParams&, void*);
-int launch_p1_f64_rhs(const StageParams&, void*);
-int launch_p1_f64_lsrk(const StageParams&, void*);
-int launch_p1_f64_lfe(const StageParams&, void*);
-int launch_p1_f64_lfh(const StageParams&, void*);
+int launch_p1_f32_adj(const AdjParams&, void*);
+int launch_t_p1_f64_lsrk(const StageParams&, void*);
+int launch_t_p1_f64_rhs(const StageParams&, void*);
+int launch_t_p1_f64_lf(const StageParams&, void*);
+int launch_t_p1_f64_lfh(const StageParams&, void*);
 int launch_p1_f64_raw(const StageParams&, void*);
 int launch_p1_f64_adj(const AdjParams&, void*);
-int launch_p2_f32_rhs(const StageParams&, void*);
+int launch_t_p2_f32_lsrk(const StageParams&, void*);
+int launch_t_p2_f32_rhs(const StageParams&, void*);
+int launch_t_p2_f32_lf(const StageParams&, void*);
+int launch_t_p2_f32_lfh(const StageParams&, void*);
+int launch_p2_f32_raw(const StageParams&, void*);
+int launch_t_p2_f32_lsrk_v1(const StageParams&, void*);
+int launch_t_p2_f32_lsrk_v2(const StageParams&, void*);
 int launch_p2_f32_lsrk(const StageParams&, void*);
 int launch_p2_f32_lfe(const StageParams&, void*);
 int launch_p2_f32_lfh(const StageParams&, void*);
-int launch_p2_f32_raw(const StageParams&, void*);
-int launch_p2_f32_adj(const AdjParams&, void*);
 int launch_p2_f32_lsrk_v1(const StageParams&, void*);
 int launch_p2_f32_lsrk_v2(const StageParams&, void*);
 int launch_p2_f32_lsrk_v3(const StageParams&, void*);
 int launch_p2_f32_lsrk_v4(const StageParams&, void*);
 int launch_p2_f32_lsrk_v5(const StageParams&, void*);
-int launch_p2_f64_rhs(const StageParams&, void*);
-int launch_p2_f64_lsrk(const StageParams&, void*);
-int launch_p2_f64_lfe(const StageParams&, void*);
-int launch_p2_f64_lfh(const StageParams&, void*);
+int launch_p2_f32_adj(const AdjParams&, void*);
+int launch_t_p2_f64_lsrk(const StageParams&, void*);
+int launch_t_p2_f64_rhs(const StageParams&, void*);
+int launch_t_p2_f64_lf(const StageParams&, void*);
+int launch_t_p2_f64_lfh(const StageParams&, void*);
 int launch_p2_f64_raw(const StageParams&, void*);
 int launch_p2_f64_adj(const AdjParams&, void*);
-int launch_p3_f32_rhs(const StageParams&, void*);
+int launch_t_p3_f32_lsrk(const StageParams&, void*);
+int launch_t_p3_f32_rhs(const StageParams&, void*);
+int launch_t_p3_f32_lf(const StageParams&, void*);
+int launch_t_p3_f32_lfh(const StageParams&, void*);
+int launch_p3_f32_raw(const StageParams&, void*);
+int launch_t_p3_f32_lsrk_v1(const StageParams&, void*);
+int launch_t_p3_f32_lsrk_v2(const StageParams&, void*);
 int launch_p3_f32_lsrk(const StageParams&, void*);
 int launch_p3_f32_lfe(const StageParams&, void*);
 int launch_p3_f32_lfh(const StageParams&, void*);
-int launch_p3_f32_raw(const StageParams&, void*);
-int launch_p3_f32_adj(const AdjParams&, void*);
 int launch_p3_f32_lsrk_v1(const StageParams&, void*);
 int launch_p3_f32_lsrk_v2(const StageParams&, void*);
 int launch_p3_f32_lsrk_v3(const StageParams&, void*);
 int launch_p3_f32_lsrk_v4(const StageParams&, void*);
 int launch_p3_f32_lsrk_v5(const StageParams&, void*);
-int launch_p3_f64_rhs(const StageParams&, void*);
-int launch_p3_f64_lsrk(const StageParams&, void*);
-int launch_p3_f64_lfe(const StageParams&, void*);
-int launch_p3_f64_lfh(const StageParams&, void*);
+int launch_p3_f32_adj(const AdjParams&, void*);
+int launch_t_p3_f64_lsrk(const StageParams&, void*);
+int launch_t_p3_f64_rhs(const StageParams&, void*);
+int launch_t_p3_f64_lf(const StageParams&, void*);
+int launch_t_p3_f64_lfh(const StageParams&, void*);
 int launch_p3_f64_raw(const StageParams&, void*);
 int launch_p3_f64_adj(const AdjParams&, void*);
-int launch_p4_f32_rhs(const StageParams&, void*);
+int launch_t_p4_f32_lsrk(const StageParams&, void*);
+int launch_t_p4_f32_rhs(const StageParams&, void*);
+int launch_t_p4_f32_lf(const StageParams&, void*);
+int launch_t_p4_f32_lfh(const StageParams&, void*);
+int launch_p4_f32_raw(const StageParams&, void*);
+int launch_t_p4_f32_lsrk_v1(const StageParams&, void*);
+int launch_t_p4_f32_lsrk_v2(const StageParams&, void*);
+int launch_t_p4_f32_lsrk_v3(const StageParams&, void*);
 int launch_p4_f32_lsrk(const StageParams&, void*);
 int launch_p4_f32_lfe(const StageParams&, void*);
 int launch_p4_f32_lfh(const StageParams&, void*);
-int launch_p4_f32_raw(const StageParams&, void*);
-int launch_p4_f32_adj(const AdjParams&, void*);
 int launch_p4_f32_lsrk_v1(const StageParams&, void*);
 int launch_p4_f32_lsrk_v2(const StageParams&, void*);
 int launch_p4_f32_lsrk_v3(const StageParams&, void*);
-int launch_p4_f64_rhs(const StageParams&, void*);
-int launch_p4_f64_lsrk(const StageParams&, void*);
-int launch_p4_f64_lfe(const StageParams&, void*);
-int launch_p4_f64_lfh(const StageParams&, void*);
+int launch_p4_f32_adj(const AdjParams&, void*);
+int launch_t_p4_f64_lsrk(const StageParams&, void*);
+int launch_t_p4_f64_rhs(const StageParams&, void*);
+int launch_t_p4_f64_lf(const StageParams&, void*);
+int launch_t_p4_f64_lfh(const StageParams&, void*);
 int launch_p4_f64_raw(const StageParams&, void*);
 int launch_p4_f64_adj(const AdjParams&, void*);
-int launch_p5_f32_rhs(const StageParams&, void*);
+int launch_t_p5_f32_lsrk(const StageParams&, void*);
+int launch_t_p5_f32_rhs(const StageParams&, void*);
+int launch_t_p5_f32_lf(const StageParams&, void*);
+int launch_t_p5_f32_lfh(const StageParams&, void*);
+int launch_p5_f32_raw(const StageParams&, void*);
+int launch_t_p5_f32_lsrk_v1(const StageParams&, void*);
+int launch_t_p5_f32_lsrk_v2(const StageParams&, void*);
+int launch_t_p5_f32_lsrk_v3(const StageParams&, void*);
 int launch_p5_f32_lsrk(const StageParams&, void*);
 int launch_p5_f32_lfe(const StageParams&, void*);
 int launch_p5_f32_lfh(const StageParams&, void*);
-int launch_p5_f32_raw(const StageParams&, void*);
-int launch_p5_f32_adj(const AdjParams&, void*);
 int launch_p5_f32_lsrk_v1(const StageParams&, void*);
 int launch_p5_f32_lsrk_v2(const StageParams&, void*);
 int launch_p5_f32_lsrk_v3(const StageParams&, void*);
+int launch_p5_f32_adj(const AdjParams&, void*);
 
 namespace {
 
 int launch_p1_f32(const StageParams& prm, int mode, void* st) {
+    const bool rec = prm.recorded != 0;
     switch (mode) {
-        case MODE_RHS: return launch_p1_f32_rhs(prm, st);
+        case MODE_RHS: return launch_t_p1_f32_rhs(prm, st);
         case MODE_LSRK:
-            if (prm.variant == 1) return launch_p1_f32_lsrk_v1(prm, st);
-            if (prm.variant == 2) return launch_p1_f32_lsrk_v2(prm, st);
-            if (prm.variant == 3) return launch_p1_f32_lsrk_v3(prm, st);
-            if (prm.variant == 4) return launch_p1_f32_lsrk_v4(prm, st);
-            return launch_p1_f32_lsrk(prm, st);
-        case MODE_LF_E: return launch_p1_f32_lfe(prm, st);
-        case MODE_LF_H: return launch_p1_f32_lfh(prm, st);
+            switch (prm.variant) {
+                case 1: return rec ? launch_p1_f32_lsrk_v1(prm, st) : launch_t_p1_f32_lsrk_v1(prm, st);
+                case 2: return rec ? launch_p1_f32_lsrk_v2(prm, st) : launch_t_p1_f32_lsrk_v2(prm, st);
+                case 3: return launch_p1_f32_lsrk_v3(prm, st);
+                case 4: return launch_p1_f32_lsrk_v4(prm, st);
+                default: return rec ? launch_p1_f32_lsrk(prm, st) : launch_t_p1_f32_lsrk(prm, st);
+            }
+        case MODE_LF_E: return rec ? launch_p1_f32_lfe(prm, st) : launch_t_p1_f32_lf(prm, st);
+        case MODE_LF_H: return rec ? launch_p1_f32_lfh(prm, st) : launch_t_p1_f32_lfh(prm, st);
         case MODE_RAW: return launch_p1_f32_raw(prm, st);
         default: return DGM_EINVAL;
     }
@@ -105,27 +143,30 @@ int launch_p1_f32(const StageParams& prm, int mode, void* st) {
 
 int launch_p1_f64(const StageParams& prm, int mode, void* st) {
     switch (mode) {
-        case MODE_RHS: return launch_p1_f64_rhs(prm, st);
-        case MODE_LSRK: return launch_p1_f64_lsrk(prm, st);
-        case MODE_LF_E: return launch_p1_f64_lfe(prm, st);
-        case MODE_LF_H: return launch_p1_f64_lfh(prm, st);
+        case MODE_RHS: return launch_t_p1_f64_rhs(prm, st);
+        case MODE_LSRK: return launch_t_p1_f64_lsrk(prm, st);
+        case MODE_LF_E: return launch_t_p1_f64_lf(prm, st);
+        case MODE_LF_H: return launch_t_p1_f64_lfh(prm, st);
         case MODE_RAW: return launch_p1_f64_raw(prm, st);
         default: return DGM_EINVAL;
     }
 }
 
 int launch_p2_f32(const StageParams& prm, int mode, void* st) {
+    const bool rec = prm.recorded != 0;
     switch (mode) {
-        case MODE_RHS: return launch_p2_f32_rhs(prm, st);
+        case MODE_RHS: return launch_t_p2_f32_rhs(prm, st);
         case MODE_LSRK:
-            if (prm.variant == 1) return launch_p2_f32_lsrk_v1(prm, st);
-            if (prm.variant == 2) return launch_p2_f32_lsrk_v2(prm, st);
-            if (prm.variant == 3) return launch_p2_f32_lsrk_v3(prm, st);
-            if (prm.variant == 4) return launch_p2_f32_lsrk_v4(prm, st);
-            if (prm.variant == 5) return launch_p2_f32_lsrk_v5(prm, st);
-            return launch_p2_f32_lsrk(prm, st);
-        case MODE_LF_E: return launch_p2_f32_lfe(prm, st);
-        case MODE_LF_H: return launch_p2_f32_lfh(prm, st);
+            switch (prm.variant) {
+                case 1: return rec ? launch_p2_f32_lsrk_v1(prm, st) : launch_t_p2_f32_lsrk_v1(prm, st);
+                case 2: return rec ? launch_p2_f32_lsrk_v2(prm, st) : launch_t_p2_f32_lsrk_v2(prm, st);
+                case 3: return launch_p2_f32_lsrk_v3(prm, st);
+                case 4: return launch_p2_f32_lsrk_v4(prm, st);
+                case 5: return launch_p2_f32_lsrk_v5(prm, st);
+                default: return rec ? launch_p2_f32_lsrk(prm, st) : launch_t_p2_f32_lsrk(prm, st);
+            }
+        case MODE_LF_E: return rec ? launch_p2_f32_lfe(prm, st) : launch_t_p2_f32_lf(prm, st);
+        case MODE_LF_H: return rec ? launch_p2_f32_lfh(prm, st) : launch_t_p2_f32_lfh(prm, st);
         case MODE_RAW: return launch_p2_f32_raw(prm, st);
         default: return DGM_EINVAL;
     }
@@ -133,27 +174,30 @@ int launch_p2_f32(const StageParams& prm, int mode, void* st) {
 
 int launch_p2_f64(const StageParams& prm, int mode, void* st) {
     switch (mode) {
-        case MODE_RHS: return launch_p2_f64_rhs(prm, st);
-        case MODE_LSRK: return launch_p2_f64_lsrk(prm, st);
-        case MODE_LF_E: return launch_p2_f64_lfe(prm, st);
-        case MODE_LF_H: return launch_p2_f64_lfh(prm, st);
+        case MODE_RHS: return launch_t_p2_f64_rhs(prm, st);
+        case MODE_LSRK: return launch_t_p2_f64_lsrk(prm, st);
+        case MODE_LF_E: return launch_t_p2_f64_lf(prm, st);
+        case MODE_LF_H: return launch_t_p2_f64_lfh(prm, st);
         case MODE_RAW: return launch_p2_f64_raw(prm, st);
         default: return DGM_EINVAL;
     }
 }
 
 int launch_p3_f32(const StageParams& prm, int mode, void* st) {
+    const bool rec = prm.recorded != 0;
     switch (mode) {
-        case MODE_RHS: return launch_p3_f32_rhs(prm, st);
+        case MODE_RHS: return launch_t_p3_f32_rhs(prm, st);
         case MODE_LSRK:
-            if (prm.variant == 1) return launch_p3_f32_lsrk_v1(prm, st);
-            if (prm.variant == 2) return launch_p3_f32_lsrk_v2(prm, st);
-            if (prm.variant == 3) return launch_p3_f32_lsrk_v3(prm, st);
-            if (prm.variant == 4) return launch_p3_f32_lsrk_v4(prm, st);
-            if (prm.variant == 5) return launch_p3_f32_lsrk_v5(prm, st);
-            return launch_p3_f32_lsrk(prm, st);
-        case MODE_LF_E: return launch_p3_f32_lfe(prm, st);
-        case MODE_LF_H: return launch_p3_f32_lfh(prm, st);
+            switch (prm.variant) {
+                case 1: return rec ? launch_p3_f32_lsrk_v1(prm, st) : launch_t_p3_f32_lsrk_v1(prm, st);
+                case 2: return rec ? launch_p3_f32_lsrk_v2(prm, st) : launch_t_p3_f32_lsrk_v2(prm, st);
+                case 3: return launch_p3_f32_lsrk_v3(prm, st);
+                case 4: return launch_p3_f32_lsrk_v4(prm, st);
+                case 5: return launch_p3_f32_lsrk_v5(prm, st);
+                default: return rec ? launch_p3_f32_lsrk(prm, st) : launch_t_p3_f32_lsrk(prm, st);
+            }
+        case MODE_LF_E: return rec ? launch_p3_f32_lfe(prm, st) : launch_t_p3_f32_lf(prm, st);
+        case MODE_LF_H: return rec ? launch_p3_f32_lfh(prm, st) : launch_t_p3_f32_lfh(prm, st);
         case MODE_RAW: return launch_p3_f32_raw(prm, st);
         default: return DGM_EINVAL;
     }
@@ -161,25 +205,28 @@ int launch_p3_f32(const StageParams& prm, int mode, void* st) {
 
 int launch_p3_f64(const StageParams& prm, int mode, void* st) {
     switch (mode) {
-        case MODE_RHS: return launch_p3_f64_rhs(prm, st);
-        case MODE_LSRK: return launch_p3_f64_lsrk(prm, st);
-        case MODE_LF_E: return launch_p3_f64_lfe(prm, st);
-        case MODE_LF_H: return launch_p3_f64_lfh(prm, st);
+        case MODE_RHS: return launch_t_p3_f64_rhs(prm, st);
+        case MODE_LSRK: return launch_t_p3_f64_lsrk(prm, st);
+        case MODE_LF_E: return launch_t_p3_f64_lf(prm, st);
+        case MODE_LF_H: return launch_t_p3_f64_lfh(prm, st);
         case MODE_RAW: return launch_p3_f64_raw(prm, st);
         default: return DGM_EINVAL;
     }
 }
 
 int launch_p4_f32(const StageParams& prm, int mode, void* st) {
+    const bool rec = prm.recorded != 0;
     switch (mode) {
-        case MODE_RHS: return launch_p4_f32_rhs(prm, st);
+        case MODE_RHS: return launch_t_p4_f32_rhs(prm, st);
         case MODE_LSRK:
-            if (prm.variant == 1) return launch_p4_f32_lsrk_v1(prm, st);
-            if (prm.variant == 2) return launch_p4_f32_lsrk_v2(prm, st);
-            if (prm.variant == 3) return launch_p4_f32_lsrk_v3(prm, st);
-            return launch_p4_f32_lsrk(prm, st);
-        case MODE_LF_E: return launch_p4_f32_lfe(prm, st);
-        case MODE_LF_H: return launch_p4_f32_lfh(prm, st);
+            switch (prm.variant) {
+                case 1: return rec ? launch_p4_f32_lsrk_v1(prm, st) : launch_t_p4_f32_lsrk_v1(prm, st);
+                case 2: return rec ? launch_p4_f32_lsrk_v2(prm, st) : launch_t_p4_f32_lsrk_v2(prm, st);
+                case 3: return rec ? launch_p4_f32_lsrk_v3(prm, st) : launch_t_p4_f32_lsrk_v3(prm, st);
+                default: return rec ? launch_p4_f32_lsrk(prm, st) : launch_t_p4_f32_lsrk(prm, st);
+            }
+        case MODE_LF_E: return rec ? launch_p4_f32_lfe(prm, st) : launch_t_p4_f32_lf(prm, st);
+        case MODE_LF_H: return rec ? launch_p4_f32_lfh(prm, st) : launch_t_p4_f32_lfh(prm, st);
         case MODE_RAW: return launch_p4_f32_raw(prm, st);
         default: return DGM_EINVAL;
     }
@@ -187,25 +234,28 @@ int launch_p4_f32(const StageParams& prm, int mode, void* st) {
 
 int launch_p4_f64(const StageParams& prm, int mode, void* st) {
     switch (mode) {
-        case MODE_RHS: return launch_p4_f64_rhs(prm, st);
-        case MODE_LSRK: return launch_p4_f64_lsrk(prm, st);
-        case MODE_LF_E: return launch_p4_f64_lfe(prm, st);
-        case MODE_LF_H: return launch_p4_f64_lfh(prm, st);
+        case MODE_RHS: return launch_t_p4_f64_rhs(prm, st);
+        case MODE_LSRK: return launch_t_p4_f64_lsrk(prm, st);
+        case MODE_LF_E: return launch_t_p4_f64_lf(prm, st);
+        case MODE_LF_H: return launch_t_p4_f64_lfh(prm, st);
         case MODE_RAW: return launch_p4_f64_raw(prm, st);
         default: return DGM_EINVAL;
     }
 }
 
 int launch_p5_f32(const StageParams& prm, int mode, void* st) {
+    const bool rec = prm.recorded != 0;
     switch (mode) {
-        case MODE_RHS: return launch_p5_f32_rhs(prm, st);
+        case MODE_RHS: return launch_t_p5_f32_rhs(prm, st);
         case MODE_LSRK:
-            if (prm.variant == 1) return launch_p5_f32_lsrk_v1(prm, st);
-            if (prm.variant == 2) return launch_p5_f32_lsrk_v2(prm, st);
-            if (prm.variant == 3) return launch_p5_f32_lsrk_v3(prm, st);
-            return launch_p5_f32_lsrk(prm, st);
-        case MODE_LF_E: return launch_p5_f32_lfe(prm, st);
-        case MODE_LF_H: return launch_p5_f32_lfh(prm, st);
+            switch (prm.variant) {
+                case 1: return rec ? launch_p5_f32_lsrk_v1(prm, st) : launch_t_p5_f32_lsrk_v1(prm, st);
+                case 2: return rec ? launch_p5_f32_lsrk_v2(prm, st) : launch_t_p5_f32_lsrk_v2(prm, st);
+                case 3: return rec ? launch_p5_f32_lsrk_v3(prm, st) : launch_t_p5_f32_lsrk_v3(prm, st);
+                default: return rec ? launch_p5_f32_lsrk(prm, st) : launch_t_p5_f32_lsrk(prm, st);
+            }
+        case MODE_LF_E: return rec ? launch_p5_f32_lfe(prm, st) : launch_t_p5_f32_lf(prm, st);
+        case MODE_LF_H: return rec ? launch_p5_f32_lfh(prm, st) : launch_t_p5_f32_lfh(prm, st);
         case MODE_RAW: return launch_p5_f32_raw(prm, st);
         default: return DGM_EINVAL;
     }

@@ -1,0 +1,750 @@
+// Fused DG right-hand-side / stage-update kernel on tangential traces (SIMT,
+// FP64 or FP32).  It evaluates the semi-discrete system stated at the head of
+// dgm_stage.cuh; this file's form of it has no geometry in the jumps.
+//
+// Tangential traces.  Only n x X of a trace enters a flux, and for covariant
+// coefficients x (X = A^-T x) the tangential part of X on a face is carried by
+// the two numbers tau_i = x . t_i, t_i the reference tangents of the face:
+//   face 0 (x + y + z = 1): t_1 = e_1 - e_0, t_2 = e_2 - e_0;
+//   face a + 1 (x_a = 0):   t_1 = e_b, t_2 = e_c, {b < c} the other two axes.
+// A t_i are the face's edges from its lowest vertex, and both elements of a
+// face keep their vertices in ascending global id: the edges, their order and
+// the parametrisation of the face modes are the same seen from either side.
+// So the jump of a face mode is tau_i(+) - tau_i(-), with no matrix between
+// the two elements' frames, and a trace costs two components instead of three.
+// With sigma_f = -1, +1, -1, +1 for f = 0..3 the identity (M a) x (M b) =
+// det M M^-T (a x b), M = A^-T, turns the pulled-back fluxes into two numbers
+// per field as well, g = gamma_1 e_b + gamma_2 e_c (face 0: component 0 of g is
+// -(gamma_1 + gamma_2)), the same on every face:
+//   s_T gE: gamma_1 =  cE dh_2 + e22 de_1 - e12 de_2,  gamma_2 = -cE dh_1 + e11 de_2 - e12 de_1
+//  -s_T gH: gamma_1 =  cH de_2 - h22 dh_1 + h12 dh_2,  gamma_2 = -cH de_1 - h11 dh_2 + h12 dh_1
+// (de, dh: jumps of tau; cE = sigma c_E, cH = sigma c_H;
+// e_ij = s_T b_E (A t_i . A t_j) / (|det A| |M m_f|), h_ij with b_H).  The
+// signs s_T are moved into the mass block:
+//   du_E = A^T A / (eps det) [curl u_H + lift(s_T gE)]
+//   du_H = -A^T A / (mu det) [curl u_E + lift(-s_T gH)].
+//
+// One CTA owns TE consecutive columns with NG threads per column.
+//   phase A: a thread takes one face (NG = 4) or one face and field (NG = 8) of
+//     its column: own trace from the tile in shared memory, neighbour trace
+//     from its gathered coefficients, both into the same sums; then the flux,
+//     written to shared memory.
+//   phase B: a thread takes one field and one part of the rows: curl and lift
+//     of all three components in registers, then the mass block, the PML terms
+//     and the stage update, so the right-hand side never leaves the registers.
+// One barrier between the two (and one before phase A for the tile).
+//
+// What bounds it.  FP64: the FP64 pipe (88 % of its rate at 48,000 elements,
+// p = 3); the tangential form needs 6.1 k operations per element-stage instead of
+// about 10 k, and with full warps of 32 columns no warp runs two row parts in
+// turn: 22.8 -> 11.9 ms per LSRK4 step of the 32^3 grid.  FP32: instruction issue
+// and latency (IPC 0.47 per SM quarter at 14 warps; long-scoreboard, instruction
+// fetch and barrier stalls); 372 warp instructions per 32 element-stages against
+// 669: 0.882 -> 0.598 ms per step of the 32^3 grid at p = 3 (0.285 ms at the
+// measured HBM rate), 6.64 -> 4.63 ms on the 40^3 grid at p = 4 with a PML.
+// Two columns per thread in packed FP32x2 instructions (half the instructions) was
+// slower, 0.673 ms: twice the registers per thread left half the columns in
+// flight.
+#pragma once
+
+#include <cstdint>
+
+#include "dgm_internal.h"
+#include "dgm_ops_gen.cuh"
+#include "dgm_bulk.cuh"
+#include "dgm_stage.cuh"
+
+namespace dgm {
+
+// Face and element constants of this kernel, one row per constant, [TG_ROWS][K]
+// in the plan's precision (tang_consts_kernel).
+enum TangConst {
+    TG_CE = 0, TG_CH = 1, TG_E11 = 2, TG_NE12 = 3, TG_E22 = 4, TG_NH11 = 5, TG_H12 = 6, TG_NH22 = 7,
+    TG_FACE = 8,                  // rows per face
+    TG_METRIC = 4 * TG_FACE,      // A^T A: 00, 01, 02, 11, 12, 22
+    TG_IE = TG_METRIC + 6,        // 1 / (eps det A)
+    TG_IH = TG_METRIC + 7,        // -1 / (mu det A)
+    TG_SIP = TG_METRIC + 8,       // interior penalty, per face: KS, A t_1 (3), A t_2 (3)
+    TG_SIPF = 7
+};
+static_assert(TG_SIP + 4 * TG_SIPF == TG_ROWS, "rows of the tangential face-constant table");
+
+// component of tangent i of face f (face 0: minus component 0)
+__host__ __device__ constexpr int tang_comp(int f, int i) { return f == 2 ? 2 * i : (f == 3 ? i : 1 + i); }
+
+// One thread per element, from the FP64 geometry (once per plan, again when the
+// materials or the boundary codes change); rounded to the plan's precision last.
+template <typename R>
+__global__ void tang_consts_kernel(const StageParams prm, bool sip, R* __restrict__ out) {
+    const int64_t K = prm.K;
+    const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (e >= K) return;
+    double M[9], at[9];
+    for (int k = 0; k < 9; ++k) M[k] = prm.geo[int64_t(G_AIT + k) * K + e];
+    const double det = prm.geo[int64_t(G_DET) * K + e];
+    const double eps = prm.geo[int64_t(G_EPS) * K + e], mu = prm.geo[int64_t(G_MU) * K + e];
+    // A^T = det A adj(A^-T), row major: row j is the edge A e_j
+    at[0] = M[4] * M[8] - M[5] * M[7];
+    at[1] = M[2] * M[7] - M[1] * M[8];
+    at[2] = M[1] * M[5] - M[2] * M[4];
+    at[3] = M[5] * M[6] - M[3] * M[8];
+    at[4] = M[0] * M[8] - M[2] * M[6];
+    at[5] = M[2] * M[3] - M[0] * M[5];
+    at[6] = M[3] * M[7] - M[4] * M[6];
+    at[7] = M[1] * M[6] - M[0] * M[7];
+    at[8] = M[0] * M[4] - M[1] * M[3];
+    for (int k = 0; k < 9; ++k) at[k] *= det;
+    const double zm = sqrt(mu / eps);
+    for (int f = 0; f < 4; ++f) {
+        double T[2][3], vn[3];
+        for (int i = 0; i < 2; ++i)
+            for (int r = 0; r < 3; ++r)
+                T[i][r] = at[3 * tang_comp(f, i) + r] - (f == 0 ? at[r] : 0.0);
+        const double m[3] = {f == 0 ? 1.0 : (f == 1 ? -1.0 : 0.0), f == 0 ? 1.0 : (f == 2 ? -1.0 : 0.0),
+                             f == 0 ? 1.0 : (f == 3 ? -1.0 : 0.0)};
+        for (int r = 0; r < 3; ++r) vn[r] = M[3 * r] * m[0] + M[3 * r + 1] * m[1] + M[3 * r + 2] * m[2];
+        const double kb = 1.0 / (det * sqrt(vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2]));   // s_T / (|det| |M m|)
+        const int32_t code = prm.nbr[int64_t(f) * K + e];
+        const bool has = code >= 0 && (code >> 2) < K;
+        const int64_t en = has ? int64_t(code >> 2) : e;
+        const double mun = prm.geo[int64_t(G_MU) * K + en];
+        const double zp = has ? sqrt(mun / prm.geo[int64_t(G_EPS) * K + en]) : zm;
+        double ce = 0.5, ch = 0.5, be = 0.0, bh = 0.0;
+        if (prm.upwind) {
+            ce = zp / (zm + zp);
+            be = 1.0 / (zm + zp);
+            ch = zm / (zm + zp);
+            bh = zm * zp / (zm + zp);
+        }
+        const double sg = (f & 1) ? 1.0 : -1.0;
+        const double t11 = T[0][0] * T[0][0] + T[0][1] * T[0][1] + T[0][2] * T[0][2];
+        const double t12 = T[0][0] * T[1][0] + T[0][1] * T[1][1] + T[0][2] * T[1][2];
+        const double t22 = T[1][0] * T[1][0] + T[1][1] * T[1][1] + T[1][2] * T[1][2];
+        const double v[TG_FACE] = {sg * ce, sg * ch, kb * be * t11, -kb * be * t12, kb * be * t22,
+                                   -kb * bh * t11, kb * bh * t12, -kb * bh * t22};
+        for (int k = 0; k < TG_FACE; ++k) out[int64_t(f * TG_FACE + k) * K + e] = R(v[k]);
+        if (sip) {
+            const int32_t sf = prm.sfid[int64_t(f) * K + e];
+            const double ks = (sf >= 0 && (sf & 1)) ? prm.sip_alpha / (0.5 * (mu + mun)) * kb : 0.0;
+            R* o = out + int64_t(TG_SIP + f * TG_SIPF) * K + e;
+            o[0] = R(ks);
+            for (int i = 0; i < 2; ++i)
+                for (int r = 0; r < 3; ++r) o[int64_t(1 + 3 * i + r) * K] = R(T[i][r]);
+        }
+    }
+    int k = TG_METRIC;
+    for (int i = 0; i < 3; ++i)
+        for (int j = i; j < 3; ++j, ++k)
+            out[int64_t(k) * K + e] = R(at[3 * i] * at[3 * j] + at[3 * i + 1] * at[3 * j + 1] + at[3 * i + 2] * at[3 * j + 2]);
+    out[int64_t(TG_IE) * K + e] = R(1.0 / (eps * det));
+    out[int64_t(TG_IH) * K + e] = R(-1.0 / (mu * det));
+}
+
+// shared memory: the tile's coefficients [6N][TE], the face quantities
+// [face][field][tangent][NF][TE] (jumps, then fluxes), an mbarrier
+template <int P, typename R, int TE>
+__host__ __device__ constexpr size_t tang_smem_bytes() {
+    return sizeof(R) * size_t(TE) * (6 * nmodes(P) + 16 * nfmodes(P)) + 16;
+}
+
+// minus the own trace of face f of the row block at v (row stride TE), less that at v0 on face 0
+template <int P, typename R, int TE>
+__device__ __forceinline__ void own_trace(int f, const R* v, const R* v0, R (&acc)[nfmodes(P)]) {
+    switch (f) {
+        case 0: TraceOp<P, 0>::template own<true>(v, v0, TE, acc); break;
+        case 1: TraceOp<P, 1>::template own<false>(v, v0, TE, acc); break;
+        case 2: TraceOp<P, 2>::template own<false>(v, v0, TE, acc); break;
+        default: TraceOp<P, 3>::template own<false>(v, v0, TE, acc); break;
+    }
+}
+
+// acc += trace of v on face f
+template <int P, typename R>
+__device__ __forceinline__ void jump_trace(int f, const R (&v)[nmodes(P)], R (&acc)[nfmodes(P)]) {
+    switch (f) {
+        case 0: TraceOp<P, 0>::jump(v, acc); break;
+        case 1: TraceOp<P, 1>::jump(v, acc); break;
+        case 2: TraceOp<P, 2>::jump(v, acc); break;
+        default: TraceOp<P, 3>::jump(v, acc); break;
+    }
+}
+
+// Tuning of the two phases; FP32 figures are ms per LSRK4 step of the 32^3 (p = 3)
+// and 24^3 grids, the alternatives measured on the same box.
+//
+// NG = 4: the larger row part of phase B goes to the threads of faces 1 and 2,
+// whose phase A is the shortest (20 and 50 trace entries at p = 3 against 142
+// and 125), so that the four warps of a CTA, one per SM quarter, have the same
+// amount to do: p = 3 0.602 with rows [0, 13) | [13, 20), 0.631 with equal parts in
+// group order.  With a PML phase B outweighs phase A, and equal parts are as good.
+template <int P, typename R, bool PML>
+__host__ __device__ constexpr bool tang_balance() { return sizeof(R) == 4 && !PML && (P == 3 || P == 4); }
+template <int P, typename R, bool PML>
+__host__ __device__ constexpr int tang_split(int np, int k) {
+    if (np == 2 && tang_balance<P, R, PML>() && P == 3) return k == 0 ? 0 : k == 1 ? 13 : nmodes(P);
+    return row_split(P, np, k);
+}
+// Residual rows held in registers from before the curl and lift on, in bytes per
+// thread: hides their latency where it fits (p = 3 0.602 against 0.673), spills
+// where it does not (p = 4 with a PML 0.99 against 1.15).
+template <int P, typename R, bool PML>
+__host__ __device__ constexpr int tang_early_bytes() {
+    return sizeof(R) == 8 ? 144 : P >= 4 && PML ? 0 : P == 5 ? 0 : PML ? 144 : 180;
+}
+
+// A thread's column: id, element, source; active: updated by this launch.
+template <typename IX>
+struct Column {
+    IX C, col, e;
+    int s;
+    bool active;
+};
+
+// Phase B of one thread: rows [LO, HI) of the three components of field F
+// (0: E, 1: H).  us, gs: shared memory at this thread's columns.
+template <int P, typename R, int TE, int MODE, typename IX, bool PML, int LO, int HI>
+__device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R* us, const R* gs,
+                                          const Column<IX>& id) {
+    constexpr int N = nmodes(P), NF = nfmodes(P), NR = HI - LO;
+    constexpr bool LF = MODE == MODE_LF_E || MODE == MODE_LF_H;
+    // residual rows requested before the arithmetic where the registers allow it
+    constexpr bool EARLY = MODE == MODE_LSRK && 3 * NR * int(sizeof(R)) <= tang_early_bytes<P, R, PML>();
+    auto coef = [&](double d, float f) { return sizeof(R) == 4 ? R(f) : R(d); };
+    const IX K = prm.K, C = id.C;
+    const bool active = id.active;
+    const R ca = coef(prm.a, prm.a_f), cb = coef(prm.b, prm.b_f), dt = coef(prm.dt, prm.dt_f);
+    const int fb = 3 * F;
+    const IX gb = IX(fb * N + LO) * C + id.col;
+    const R* __restrict__ resi = static_cast<const R*>(prm.res);
+    const bool ld = active && ca != R(0);
+    R rv[EARLY ? NR : 1][3];
+    if constexpr (EARLY) {
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) rv[i][k] = ld ? resi[gb + IX(k * N + i) * C] : R(0);
+    }
+    // a row of a per-element table at the thread's elements
+    auto table = [&](const void* base, int row) -> R {
+        const R* b = static_cast<const R*>(base) + IX(row) * K;
+        return b[id.e];
+    };
+    const R g00 = table(prm.fct, TG_METRIC), g01 = table(prm.fct, TG_METRIC + 1), g02 = table(prm.fct, TG_METRIC + 2);
+    const R g11 = table(prm.fct, TG_METRIC + 3), g12 = table(prm.fct, TG_METRIC + 4), g22 = table(prm.fct, TG_METRIC + 5);
+    const R im = table(prm.fct, TG_IE + F);   // 1 / (eps det) or -1 / (mu det)
+
+    R a0[N], a1[N], a2[N];
+#pragma unroll
+    for (int l = LO; l < HI; ++l) a1[l] = a2[l] = R(0);
+    const R* g = gs + 2 * F * NF * TE;    // this field's gamma_1 of face 0; face f at + 4 f NF TE
+    LiftOp<P, 0>::template apply<R, LO, HI>(g, TE, a1);
+    LiftOp<P, 0>::template apply<R, LO, HI>(g + NF * TE, TE, a2);
+#pragma unroll
+    for (int l = LO; l < HI; ++l) a0[l] = (a1[l] + a2[l]) * R(-1);
+    CurlOp<P>::template apply<R, LO, HI>(us + (3 - fb) * N * TE, N * TE, TE, a0, a1, a2);
+    LiftOp<P, 1>::template apply<R, LO, HI>(g + 4 * NF * TE, TE, a1);
+    LiftOp<P, 1>::template apply<R, LO, HI>(g + 5 * NF * TE, TE, a2);
+    LiftOp<P, 2>::template apply<R, LO, HI>(g + 8 * NF * TE, TE, a0);
+    LiftOp<P, 2>::template apply<R, LO, HI>(g + 9 * NF * TE, TE, a2);
+    LiftOp<P, 3>::template apply<R, LO, HI>(g + 12 * NF * TE, TE, a0);
+    LiftOp<P, 3>::template apply<R, LO, HI>(g + 13 * NF * TE, TE, a1);
+    if (!active) return;
+
+    if (F == 0 && prm.src != nullptr) {
+        const double* rec = prm.src + IX(id.s) * (SRC_HDR + 3 * N);
+        if (rec[0] >= 0.0 && IX(rec[0]) == id.e) {   // -1 marks a column without a source
+            const double tt = prm.tdev ? *prm.tdev + prm.t : prm.t;
+            // the rows carry the factor s_T = sign of det A
+            const R gt = (im < R(0) ? R(1) : R(-1)) * R(source_time(tt, rec[1], rec[2], rec[3]));
+#pragma unroll
+            for (int l = LO; l < HI; ++l) {
+                a0[l] = fmaa(gt, R(rec[SRC_HDR + l]), a0[l]);
+                a1[l] = fmaa(gt, R(rec[SRC_HDR + N + l]), a1[l]);
+                a2[l] = fmaa(gt, R(rec[SRC_HDR + 2 * N + l]), a2[l]);
+            }
+        }
+    }
+    R* __restrict__ res = static_cast<R*>(prm.res);
+    R* uo = static_cast<R*>(prm.u_out);
+    // the mass block; outside the right-hand-side mode scaled by the step
+    const R sc = MODE == MODE_RHS ? im : im * dt;
+    const R b00 = sc * g00, b01 = sc * g01, b02 = sc * g02, b11 = sc * g11, b12 = sc * g12, b22 = sc * g22;
+#pragma unroll
+    for (int l = LO; l < HI; ++l) {
+        const R r0 = a0[l], r1 = a1[l], r2 = a2[l];
+        a0[l] = fmaa(b02, r2, fmaa(b01, r1, b00 * r0));
+        a1[l] = fmaa(b12, r2, fmaa(b11, r1, b01 * r0));
+        a2[l] = fmaa(b22, r2, fmaa(b12, r1, b02 * r0));
+    }
+    if constexpr (PML) {
+        const int32_t pi = prm.pml[id.e];
+        if (pi >= 0) {
+            // PML: D -> A^T D A^-T for D = eta, Sigma, xi ; leapfrog works
+            // per Cartesian component in the physical frame
+            R M[9], AT[3][3];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) M[k] = table(prm.geo_r, G_AIT + k);
+            const R det = table(prm.geo_r, G_DET);
+            const R mat = table(prm.geo_r, G_EPS + F);
+            const R imat = R(1) / mat;
+            const R sx = table(prm.geo_r, G_SIG), sy = table(prm.geo_r, G_SIG + 1), sz = table(prm.geo_r, G_SIG + 2);
+            AT[0][0] = det * (M[4] * M[8] - M[5] * M[7]);
+            AT[0][1] = det * (M[2] * M[7] - M[1] * M[8]);
+            AT[0][2] = det * (M[1] * M[5] - M[2] * M[4]);
+            AT[1][0] = det * (M[5] * M[6] - M[3] * M[8]);
+            AT[1][1] = det * (M[0] * M[8] - M[2] * M[6]);
+            AT[1][2] = det * (M[2] * M[3] - M[0] * M[5]);
+            AT[2][0] = det * (M[3] * M[7] - M[4] * M[6]);
+            AT[2][1] = det * (M[1] * M[6] - M[0] * M[7]);
+            AT[2][2] = det * (M[0] * M[4] - M[1] * M[3]);
+            const R sg[3] = {sx, sy, sz};
+            const R et[3] = {sy + sz - sx, sz + sx - sy, sx + sy - sz};
+            const R xi[3] = {(sx - sy) * (sx - sz), (sy - sz) * (sy - sx), (sz - sx) * (sz - sy)};
+            const IX C2 = IX(prm.npml) * IX(prm.S);
+            const IX acol = IX(pi) * IX(prm.S) + id.s;
+            auto load_aux = [&](const R* p, IX row) -> R { return p[row * C2 + acol]; };
+            auto store_aux = [&](R* p, IX row, R v) { p[row * C2 + acol] = v; };
+            const IX ab = IX(fb * N + LO);
+            if constexpr (LF) {
+                // Leapfrog with the PML terms by the trapezoid rule (Sec. V), X = A^-T x:
+                //   X_new = ((1 - dt eta/2) X + dt (A^-T du - A^-T aux / mat)) / (1 + dt eta/2)
+                // then the other field's auxiliary, Y = A^-T (other field), mat' its material:
+                //   Z_new = ((1 - dt sigma/2) Z + dt mat' xi Y) / (1 + dt sigma/2)
+                const R omat = table(prm.geo_r, G_EPS + 1 - F);
+                const IX abo = IX((3 - fb) * N + LO);
+                R* auxl = static_cast<R*>(prm.aux_out);   // in place: aux_out == aux
+                R xx[3], xy[3], za[3], zb[3];
+                const R ndi = imat * -dt;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const R hd = R(0.5) * dt * et[a], hs = R(0.5) * dt * sg[a];
+                    const R nx = R(1) + hd, nz = R(1) + hs;
+                    xy[a] = R(1) / nx;
+                    xx[a] = (R(1) - hd) * xy[a];
+                    const R iz = R(1) / nz;
+                    za[a] = (R(1) - hs) * iz;
+                    zb[a] = iz * dt * omat * xi[a];
+                }
+                // rows in chunks whose loads are all requested before their arithmetic
+                constexpr int CH = sizeof(R) == 8 ? 2 : 4;
+#pragma unroll
+                for (int i0 = 0; i0 < NR; i0 += CH) {
+                    R av[CH][3], oa[CH][3];
+#pragma unroll
+                    for (int i = 0; i < CH; ++i) {
+                        if (i0 + i >= NR) break;
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            av[i][k] = load_aux(auxl, ab + IX(k * N + i0 + i));
+                            oa[i][k] = load_aux(auxl, abo + IX(k * N + i0 + i));
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < CH; ++i) {
+                        if (i0 + i >= NR) break;
+                        const int l = LO + i0 + i;
+                        R ov[3], uv[3], Xn[3], Zn[3];
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            uv[k] = us[((fb + k) * N + l) * TE];
+                            ov[k] = us[((3 - fb + k) * N + l) * TE];
+                        }
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            auto phys = [&](R p, R q, R r) {
+                                return fmaa(M[3 * a + 2], r, fmaa(M[3 * a + 1], q, M[3 * a] * p));
+                            };
+                            const R y = fmaa(ndi, phys(av[i][0], av[i][1], av[i][2]), phys(a0[l], a1[l], a2[l]));
+                            Xn[a] = fmaa(xx[a], phys(uv[0], uv[1], uv[2]), xy[a] * y);
+                            Zn[a] = fmaa(za[a], phys(oa[i][0], oa[i][1], oa[i][2]), zb[a] * phys(ov[0], ov[1], ov[2]));
+                        }
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            uo[gb + IX(k * N + i0 + i) * C] =
+                                fmaa(AT[k][2], Xn[2], fmaa(AT[k][1], Xn[1], AT[k][0] * Xn[0]));
+                            store_aux(auxl, abo + IX(k * N + i0 + i),
+                                      fmaa(AT[k][2], Zn[2], fmaa(AT[k][1], Zn[1], AT[k][0] * Zn[0])));
+                        }
+                    }
+                }
+                return;
+            } else {
+                // (an auxiliary residual row is read before it is written, by the same thread)
+                const R* __restrict__ aux = static_cast<const R*>(prm.aux);
+                const R* __restrict__ auxi = static_cast<const R*>(prm.aux_res);
+                R* auxo = static_cast<R*>(prm.aux_out);
+                R* auxr = static_cast<R*>(prm.aux_res);
+                // -eta, -Sigma, mat xi and -1/mat, times the step outside the right-hand-side mode
+                const R st = MODE == MODE_RHS ? R(1) : dt;
+                const R nst = R(-1) * st, ni = nst * imat;
+                R ETA[3][3], SIG[3][3], XI[3][3];
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const R w0 = AT[j][0] * M[k], w1 = AT[j][1] * M[3 + k], w2 = AT[j][2] * M[6 + k];
+                        ETA[j][k] = nst * fmaa(w2, et[2], fmaa(w1, et[1], w0 * et[0]));
+                        SIG[j][k] = nst * fmaa(w2, sg[2], fmaa(w1, sg[1], w0 * sg[0]));
+                        XI[j][k] = st * mat * fmaa(w2, xi[2], fmaa(w1, xi[1], w0 * xi[0]));
+                    }
+                // rows in chunks whose loads are all requested before their arithmetic
+                constexpr int CH = sizeof(R) == 8 ? 2 : 3;
+#pragma unroll
+                for (int i0 = 0; i0 < NR; i0 += CH) {
+                    R av[CH][3], ar[CH][3];
+#pragma unroll
+                    for (int i = 0; i < CH; ++i) {
+                        if (i0 + i >= NR) break;
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            av[i][k] = load_aux(aux, ab + IX(k * N + i0 + i));
+                            ar[i][k] = (MODE == MODE_LSRK && ca != R(0)) ? load_aux(auxi, ab + IX(k * N + i0 + i)) : R(0);
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < CH; ++i) {
+                        if (i0 + i >= NR) break;
+                        const int l = LO + i0 + i;
+                        R uv[3], d[3];
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) uv[k] = us[((fb + k) * N + l) * TE];
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            d[k] = fmaa(ni, av[i][k], fmaa(ETA[k][2], uv[2], fmaa(ETA[k][1], uv[1], ETA[k][0] * uv[0])));
+                            const R da = fmaa(SIG[k][2], av[i][2], fmaa(SIG[k][1], av[i][1], fmaa(SIG[k][0], av[i][0],
+                                         fmaa(XI[k][2], uv[2], fmaa(XI[k][1], uv[1], XI[k][0] * uv[0])))));
+                            const IX row = ab + IX(k * N + i0 + i);
+                            if (MODE == MODE_RHS) {
+                                store_aux(auxo, row, da);
+                            } else {
+                                const R rr = fmaa(ca, ar[i][k], da);
+                                store_aux(auxr, row, rr);
+                                store_aux(auxo, row, fmaa(cb, rr, av[i][k]));
+                            }
+                        }
+                        a0[l] += d[0];
+                        a1[l] += d[1];
+                        a2[l] += d[2];
+                    }
+                }
+            }
+        }
+    }
+    // update; residual rows in chunks when they were not requested early
+    constexpr int CH = EARLY ? NR : int(32 / sizeof(R));
+#pragma unroll
+    for (int i0 = 0; i0 < NR; i0 += CH) {
+        R rc[CH][3];
+        if constexpr (MODE == MODE_LSRK) {
+#pragma unroll
+            for (int i = 0; i < CH; ++i) {
+                if (i0 + i >= NR) break;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    if constexpr (EARLY) rc[i][k] = rv[i][k];
+                    else rc[i][k] = ld ? resi[gb + IX(k * N + i0 + i) * C] : R(0);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < CH; ++i) {
+            if (i0 + i >= NR) break;
+            const int l = LO + i0 + i;
+            const R du[3] = {a0[l], a1[l], a2[l]};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const IX gi = gb + IX(k * N + i0 + i) * C;
+                if (MODE == MODE_RHS) {
+                    uo[gi] = du[k];
+                } else if (MODE == MODE_LSRK) {
+                    const R rr = fmaa(ca, rc[i][k], du[k]);
+                    res[gi] = rr;
+                    uo[gi] = fmaa(cb, rr, us[((fb + k) * N + l) * TE]);
+                } else {
+                    uo[gi] = us[((fb + k) * N + l) * TE] + du[k];
+                }
+            }
+        }
+    }
+}
+
+template <int P, typename R, int TE, int MODE, typename IX, bool PML, int NPART>
+__device__ __forceinline__ void tang_part(const StageParams& prm, int F, int part, const R* us, const R* gs,
+                                          const Column<IX>& id) {
+    static_assert(NPART == 2 || NPART == 4, "row parts");
+#define DGM_ROWS(K_) \
+    tang_rows<P, R, TE, MODE, IX, PML, tang_split<P, R, PML>(NPART, K_), tang_split<P, R, PML>(NPART, K_ + 1)>(prm, F, us, gs, id)
+    if constexpr (NPART == 2) {
+        if (part == 0) DGM_ROWS(0);
+        else DGM_ROWS(1);
+    } else {
+        switch (part) {
+            case 0: DGM_ROWS(0); break;
+            case 1: DGM_ROWS(1); break;
+            case 2: DGM_ROWS(2); break;
+            default: DGM_ROWS(3); break;
+        }
+    }
+#undef DGM_ROWS
+}
+
+// IX: type of the element/column/row index arithmetic (uint32_t when every
+// index of the plan fits, else int64_t).  MINB: resident CTAs per SM asked of
+// the register allocator.  NG = 4: thread groups = faces (both fields), then
+// (field, half of the rows); NG = 8: (face, field), then (field, quarter of the
+// rows), the two fields of a face in the two halves of a warp (TE = 16) or in
+// two neighbouring warps (TE = 32).
+template <int P, typename R, int TE, int NG, int MODE, typename IX, bool SIP, bool PML, int MINB>
+__global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams prm) {
+    static_assert((TE == 32 && (NG == 4 || NG == 8)) || (TE == 16 && NG == 8), "tile shape");
+    static_assert(!SIP || MODE == MODE_LSRK || MODE == MODE_RHS, "interior penalty modes");
+    constexpr int N = nmodes(P), NF = nfmodes(P);
+    constexpr bool LF = MODE == MODE_LF_E || MODE == MODE_LF_H;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    R* us = reinterpret_cast<R*>(smem_raw);   // [6N][TE]
+    R* gs = us + 6 * N * TE;                  // [4][2][2][NF][TE]
+    uint64_t* bar = reinterpret_cast<uint64_t*>(gs + 16 * NF * TE);
+
+    const int c = threadIdx.x % TE;
+    const int grp = threadIdx.x / TE;
+    const IX K = prm.K;
+    const int S = prm.S;
+    const IX x0 = IX(tile_index(prm.tile_groups)) * TE;
+    Column<IX> id;
+    id.C = K * S;
+    id.col = x0 + c;
+    // only the first K_active elements are updated; the others (halo copies of
+    // another partition's elements) are read as neighbours
+    id.active = id.col < IX(prm.K_active) * IX(S);
+    id.e = id.active ? id.col / S : 0;
+    id.s = id.active ? int(id.col - id.e * S) : 0;
+    const IX C = id.C;
+    const bool active = id.active;
+    const R* u = static_cast<const R*>(prm.u);   // may alias u_out (leapfrog)
+    auto coef = [&](double d, float f) { return sizeof(R) == 4 ? R(f) : R(d); };
+
+    // The tile: one bulk tensor copy of the box [6][N][TE] where the plan has a
+    // map of u (aligned rows), issued first and waited for by thread 0; columns
+    // past the end arrive as zeros.  Otherwise every thread loads its rows.
+    const bool bulk = prm.tm_u >= 0 && (tc::smem_addr(smem_raw) & 127u) == 0;
+    if (bulk && threadIdx.x == 0) {
+        static_assert(sizeof(R) * TE * 6 * N < (1u << 20), "bytes of an mbarrier phase");
+        tc::mbar_init(bar, 1);
+        bulk::arrive_expect_tx(bar, uint32_t(sizeof(R)) * TE * 6 * N);
+        bulk::load_3d(us, static_cast<const char*>(prm.tmaps) + prm.tm_u * TMAP_BYTES, int(x0), 0, 0, bar);
+    }
+
+    // ---- phase A: jumps and fluxes of one face -----------------------------------
+    const int f = NG == 4 ? grp : grp >> 1;
+    const int half = NG == 4 ? 0 : grp & 1;      // field (leapfrog: tangent) of this thread when NG = 8
+    const int32_t code = active ? prm.nbr[IX(f) * K + id.e] : -1;
+    const bool bad = code >= 0 && IX(code >> 2) >= K;
+    if (bad) atomicOr(prm.status, int32_t(ST_BAD_NEIGHBOUR));
+    const bool has = code >= 0 && !bad;
+    const int nf = code & 3;                                    // the neighbour's local face
+    const IX nc = has ? IX(code >> 2) * S + id.s : 0;           // the neighbour's column
+    // items q = 2 field + tangent of this thread
+    constexpr int QF = MODE == MODE_LF_E ? 2 : 0;              // leapfrog: only the other field's jumps
+    constexpr int QN = LF ? (NG == 4 ? 2 : 1) : (NG == 4 ? 4 : 2);
+    const int q0 = QF + (NG == 4 ? 0 : half * QN);
+    constexpr bool AHEAD = P <= 3 || (P == 4 && PML);   // gathers of a slanted neighbour face in two register sets
+    R vn[N], vm[AHEAD ? N : 1];
+    auto fetch = [&](int comp, R* v) {   // the neighbour's coefficients of one component
+        const R* p = u + (IX(comp * N) * C + nc);
+#pragma unroll
+        for (int l = 0; l < N; ++l) v[l] = p[IX(l) * C];
+    };
+    auto gather = [&](int q) {
+        if (!has) return;
+        fetch((q >> 1) * 3 + tang_comp(nf, q & 1), vn);
+        if constexpr (AHEAD) {
+            if (nf == 0) fetch((q >> 1) * 3, vm);
+        }
+    };
+    gather(q0);
+    auto table = [&](int row) -> R {
+        const R* b = static_cast<const R*>(prm.fct) + IX(row) * K;
+        return b[id.e];
+    };
+    const R cE = table(f * TG_FACE + TG_CE), cH = table(f * TG_FACE + TG_CH);
+    if (bulk) {
+        bool ok = true;
+        if (threadIdx.x == 0) ok = tc::mbar_wait(bar, 0, 500000000ull);
+        if (!__syncthreads_and(ok)) {
+            // the copy did not complete in time: latch the status, give it a
+            // second bounded wait (the shared memory stays this CTA's until its
+            // last thread exits) and leave the tile untouched
+            if (threadIdx.x == 0) {
+                atomicOr(prm.status, int32_t(ST_TIMEOUT));
+                tc::mbar_wait(bar, 0, 500000000ull);
+            }
+            return;
+        }
+    } else {
+        constexpr int UR = (6 * N + NG - 1) / NG, BATCH = UR < 16 ? UR : 16;
+#pragma unroll 1
+        for (int i0 = 0; i0 < UR; i0 += BATCH) {
+            R tmp[BATCH];
+#pragma unroll
+            for (int i = 0; i < BATCH; ++i) {
+                const int q = grp + (i0 + i) * NG;
+                tmp[i] = (active && q < 6 * N) ? u[IX(q) * C + id.col] : R(0);
+            }
+#pragma unroll
+            for (int i = 0; i < BATCH; ++i) {
+                const int q = grp + (i0 + i) * NG;
+                if (q < 6 * N) us[q * TE + c] = tmp[i];
+            }
+        }
+        __syncthreads();
+    }
+    R* gf = gs + f * 4 * NF * TE + c;   // this face's rows: [field][tangent][NF]
+    const bool inc = code <= -2 && prm.inc != nullptr;
+#pragma unroll 1
+    for (int k = 0; k < QN; ++k) {
+        const int q = q0 + k, fld = q >> 1, i = q & 1;
+        const R* v0 = us + fld * 3 * N * TE + c;
+        R acc[NF];
+        own_trace<P, R, TE>(f, v0 + tang_comp(f, i) * N * TE, v0, acc);
+        if (has) {
+            if (nf == 0) {   // slanted neighbour face: less component 0
+                if constexpr (AHEAD) {
+#pragma unroll
+                    for (int l = 0; l < N; ++l) vn[l] -= vm[l];
+                } else {
+                    const R* p0 = u + (IX(fld * 3 * N) * C + nc);
+#pragma unroll
+                    for (int l = 0; l < N; ++l) vn[l] -= p0[IX(l) * C];
+                }
+            }
+            jump_trace<P, R>(nf, vn, acc);
+        } else {
+            // boundary face, acc = -own: PEC (e+ = -e-, h+ = h-) or incident
+            // (e+ = e- + 2 E_inc, h+ = -h-; the E_inc part is added with the flux)
+            const R al = ((fld == 0) != inc) ? R(2) : R(0);
+#pragma unroll
+            for (int m = 0; m < NF; ++m) acc[m] *= al;
+        }
+        // central flux of the leapfrog: gamma_1 = c tau_2, gamma_2 = -c tau_1 of the other field
+        const R cc = LF ? (MODE == MODE_LF_E ? cE : cH) * R(i ? 1 : -1) : R(1);
+        R* o = gf + (LF ? 2 * (1 - fld) + 1 - i : q) * NF * TE;
+#pragma unroll
+        for (int m = 0; m < NF; ++m) o[m * TE] = LF ? cc * acc[m] : acc[m];
+        if (k + 1 < QN) gather(q + 1);
+    }
+    if constexpr (!LF) {
+        // fluxes in place; with NG = 8 the face's two threads split the modes
+        // and first wait for each other's jumps
+        if (NG == 8) {
+            if (TE == 16) __syncwarp();
+            else asm volatile("bar.sync %0, 64;" :: "r"(1 + f) : "memory");
+        }
+        constexpr int MH = NG == 8 ? NF / 2 : NF;
+        const int m0 = half * MH, m1 = (NG == 8 && half == 0) ? MH : NF;
+        const R e11 = table(f * TG_FACE + TG_E11), ne12 = table(f * TG_FACE + TG_NE12), e22 = table(f * TG_FACE + TG_E22);
+        const R nh11 = table(f * TG_FACE + TG_NH11), h12 = table(f * TG_FACE + TG_H12), nh22 = table(f * TG_FACE + TG_NH22);
+        const R ncE = cE * R(-1), ncH = cH * R(-1);
+        // incident jump terms of this face: covariant components [NF][3]
+        const R* ic = inc ? static_cast<const R*>(prm.inc) + IX(-code - 2) * NF * 3 : nullptr;
+        // interior penalty: this column's facet field on face f (and, on the
+        // owner side, its output and residual), [3][NF][facet][S]
+        const R* hsv = nullptr;
+        R *hso = nullptr, *hsr = nullptr;
+        R T1[3], T2[3], ks = R(0);
+        const int64_t fs = int64_t(prm.n_facets) * S;
+        const R ca = coef(prm.a, prm.a_f), cb = coef(prm.b, prm.b_f), dt = coef(prm.dt, prm.dt_f);
+        const R sig = (f & 1) ? R(1) : R(-1);
+        if constexpr (SIP) {
+            const int32_t sf = active ? prm.sfid[IX(f) * K + id.e] : -1;
+            if (sf >= 0) {
+                const int64_t off = int64_t(sf >> 1) * S + id.s;
+                hsv = static_cast<const R*>(prm.hs) + off;
+                if (sf & 1) {
+                    hso = static_cast<R*>(prm.hs_out) + off;
+                    hsr = MODE == MODE_LSRK ? static_cast<R*>(prm.hs_res) + off : nullptr;
+                }
+            }
+            const R* ts = static_cast<const R*>(prm.fct) + IX(TG_SIP + f * TG_SIPF) * K + id.e;
+            ks = ts[0];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                T1[r] = ts[IX(1 + r) * K];
+                T2[r] = ts[IX(4 + r) * K];
+            }
+        }
+        // the modes in chunks, so that a chunk's facet values arrive together
+        constexpr int MC = SIP ? (NF + 3) / 4 : 1;
+#pragma unroll(SIP ? 1 : (P <= 3 ? 10 : 3))
+        for (int mb = m0; mb < m1; mb += MC) {
+            R hv[SIP ? MC : 1][3], hr[SIP ? MC : 1][3];
+            if constexpr (SIP) {
+#pragma unroll
+                for (int j = 0; j < MC; ++j)
+#pragma unroll
+                    for (int r = 0; r < 3; ++r) {
+                        const int64_t o = int64_t(r * NF + mb + j) * fs;
+                        hv[j][r] = (hsv != nullptr && mb + j < m1) ? hsv[o] : R(0);
+                        hr[j][r] = (MODE == MODE_LSRK && hsr != nullptr && mb + j < m1) ? hsr[o] : R(0);
+                    }
+            }
+#pragma unroll
+            for (int j = 0; j < MC; ++j) {
+                const int m = mb + j;
+                if (SIP && m >= m1) break;
+                R* o = gf + m * TE;
+                R e1 = o[0], e2 = o[NF * TE];
+                const R h1 = o[2 * NF * TE], h2 = o[3 * NF * TE];
+                if (ic != nullptr) {
+                    const R z = f == 0 ? ic[3 * m] : R(0);
+                    e1 += ic[3 * m + tang_comp(f, 0)] - z;
+                    e2 += ic[3 * m + tang_comp(f, 1)] - z;
+                }
+                R p1 = fmaa(cE, h2, fmaa(e22, e1, ne12 * e2));
+                R p2 = fmaa(ncE, h1, fmaa(e11, e2, ne12 * e1));
+                o[2 * NF * TE] = fmaa(cH, e2, fmaa(h12, h2, nh22 * h1));
+                o[3 * NF * TE] = fmaa(ncH, e1, fmaa(h12, h1, nh11 * h2));
+                if constexpr (SIP) {
+                    // both sides: gamma += m_f x (A^T h_s); owner: dh_s/dt =
+                    // -ks A (m_f x de) = -ks sigma (A t_1 de_2 - A t_2 de_1)
+                    if (hsv != nullptr) {
+                        p1 += sig * (T2[0] * hv[j][0] + T2[1] * hv[j][1] + T2[2] * hv[j][2]);
+                        p2 -= sig * (T1[0] * hv[j][0] + T1[1] * hv[j][1] + T1[2] * hv[j][2]);
+                    }
+                    if (hso != nullptr) {
+#pragma unroll
+                        for (int r = 0; r < 3; ++r) {
+                            const R d = -ks * sig * (T1[r] * e2 - T2[r] * e1);
+                            const int64_t oo = int64_t(r * NF + m) * fs;
+                            if (MODE == MODE_RHS) {
+                                hso[oo] = d;
+                            } else {
+                                const R rr = ca * hr[j][r] + dt * d;
+                                hsr[oo] = rr;
+                                hso[oo] = hv[j][r] + cb * rr;
+                            }
+                        }
+                    }
+                }
+                o[0] = p1;
+                o[NF * TE] = p2;
+            }
+        }
+    }
+    __syncthreads();
+
+    // ---- phase B: curl, lift, mass block, update ----------------------------------
+    if constexpr (LF) {
+        // one field; NG = 8 would need eight row parts, its second half idles
+        constexpr int F = MODE == MODE_LF_E ? 0 : 1;
+        if (grp < 4) tang_part<P, R, TE, MODE, IX, PML, 4>(prm, F, grp, us + c, gs + c, id);
+    } else if constexpr (NG == 4) {
+        constexpr bool BAL = tang_balance<P, R, PML>();
+        const int F = BAL ? grp >> 1 : grp & 1;
+        const int part = BAL ? (grp == 1 || grp == 2 ? 0 : 1) : grp >> 1;
+        tang_part<P, R, TE, MODE, IX, PML, 2>(prm, F, part, us + c, gs + c, id);
+    } else {
+        tang_part<P, R, TE, MODE, IX, PML, 4>(prm, grp & 1, grp >> 1, us + c, gs + c, id);
+    }
+}
+
+}  // namespace dgm

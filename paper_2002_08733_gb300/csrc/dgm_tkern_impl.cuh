@@ -1,0 +1,122 @@
+// Body of one translation unit of the tangential-trace stage kernel: instantiates
+// tang_kernel for one polynomial degree (DGM_P), one field precision (DGM_REAL)
+// and one mode (DGM_MODE; MODE_LF_E with DGM_LAUNCH2 also instantiates
+// MODE_LF_H), and exports its launchers.  Included by the
+// dgm_tkern_p<P>_<precision>_<mode>.cu files; one mode per file keeps the
+// heavily unrolled kernels compiling in parallel.
+#include <cuda_runtime.h>
+
+#include "dgm_internal.h"
+#include "dgm_tang.cuh"
+#include "dgmax.h"
+
+namespace dgm {
+namespace {
+
+constexpr int kP = DGM_P;
+using Real = DGM_REAL;
+// Tile shape of tang_kernel: threads side by side (columns per CTA), threads per
+// column, and resident CTAs per SM asked of the register allocator (DGM_TE /
+// DGM_NG / DGM_MINB select an autotuner variant).
+template <int MODE, bool SIP, bool PML>
+struct Shape {
+    static constexpr bool kLF = MODE == MODE_LF_E || MODE == MODE_LF_H, kF64 = sizeof(Real) == 8;
+#ifdef DGM_TE
+    static constexpr int TE = DGM_TE, NG = DGM_NG, MINB = DGM_MINB;
+#else
+    // FP32: four threads per column while a thread's rows (half of them) and a
+    // trace's coefficients fit its registers, eight from p = 5 on, and at p = 4
+    // with the PML's matrices or the penalty's facet values besides.
+    // FP64 (bound by the FP64 pipe, which few warps saturate): full warps of 32
+    // columns, so that no warp runs two faces or row parts in turn.
+    static constexpr int TE = 32;
+    static constexpr int NG = kLF ? (kF64 ? 4 : kP <= 4 ? 4 : 8)
+                                  : kF64 || SIP || kP == 5 || (kP == 4 && PML) ? 8 : 4;
+    static constexpr int MINB =
+        kF64 ? (kLF ? (kP <= 3 ? 2 : 1) : kP <= 3 ? 2 : 1)
+        : SIP ? (kP <= 3 ? 3 : 2)
+        : kP == 1 ? 8 : kP == 2 ? (PML ? 6 : 7) : kP == 3 ? (kLF ? 5 : 4)
+        : kP == 4 ? 3 : 2;
+#endif
+};
+
+// the interior penalty runs in the default shape
+#ifndef DGM_TE
+constexpr bool kSIP = true;
+#else
+constexpr bool kSIP = false;
+#endif
+
+template <int MODE, typename IX, bool SIP, bool PML>
+int launch_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
+    using Sh = Shape<MODE, SIP, PML>;
+    constexpr size_t smem = tang_smem_bytes<kP, Real, Sh::TE>();
+    static bool configured = false;
+    auto k = tang_kernel<kP, Real, Sh::TE, Sh::NG, MODE, IX, SIP, PML, Sh::MINB>;
+    if (!configured) {
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
+            cudaSuccess)
+            return DGM_ECUDA;
+        configured = true;
+    }
+    k<<<grid, Sh::TE * Sh::NG, smem, st>>>(q);
+    return cudaGetLastError() == cudaSuccess ? DGM_OK : DGM_ECUDA;
+}
+
+// true when every index the kernel forms for this plan is below 2^32: field
+// rows (6N x C), auxiliaries (6N x npml S), geometry (G_COUNT x K), the constant
+// table (TG_ROWS x K), incident jump terms (3 NF per boundary face)
+bool fits_32bit(const StageParams& p) {
+    const uint64_t lim = uint64_t(1) << 32;
+    const uint64_t K = uint64_t(p.K), C = K * uint64_t(p.S);
+    const uint64_t N = uint64_t(nmodes(kP)), NF = uint64_t(nfmodes(kP));
+    return 6 * N * C < lim && 6 * N * uint64_t(p.npml) * uint64_t(p.S) < lim &&
+           uint64_t(G_COUNT) * K < lim && uint64_t(TG_ROWS) * K < lim && 12 * NF * K < lim;
+}
+
+template <int MODE>
+int launch_mode(const StageParams& prm, cudaStream_t st) {
+    const int64_t C = prm.K_active * prm.S;   // columns updated
+    if (C <= 0) return DGM_OK;
+    constexpr int kTE = Shape<MODE, false, false>::TE;   // (the same for every shape of a mode)
+    const unsigned grid = unsigned((C + kTE - 1) / kTE);
+    StageParams q = prm;
+    q.dt_f = float(prm.dt);
+    q.a_f = float(prm.a);
+    q.b_f = float(prm.b);
+    const bool i32 = !q.force_index64 && fits_32bit(q);
+    // the tile's bulk copy: the plan's tensor-map set of this tile width and the
+    // map of this stage's input
+    q.tm_u = -1;
+    if (q.tmaps != nullptr) {
+        constexpr int kSet = kTE == tmap_columns(0) ? 0 : 1;
+        static_assert(kTE == tmap_columns(kSet), "a tensor-map set of this tile width");
+        q.tmaps = static_cast<const char*>(q.tmaps) + size_t(kSet) * TMAP_COUNT * TMAP_BYTES;
+        q.tm_u = q.u == q.tm_f0 ? TM_U0
+                 : q.u == q.tm_f1 ? TM_U1
+                 : (q.tm_fw != nullptr && q.u == q.tm_fw) ? TM_UW : -1;
+    }
+    if (q.hs != nullptr) {   // interior penalty
+        if constexpr (kSIP && (MODE == MODE_LSRK || MODE == MODE_RHS)) {
+            return i32 ? launch_ix<MODE, uint32_t, true, false>(q, grid, st) : launch_ix<MODE, int64_t, true, false>(q, grid, st);
+        } else {
+            return DGM_EUNSUP;
+        }
+    }
+    if (q.pml != nullptr && q.npml > 0)
+        return i32 ? launch_ix<MODE, uint32_t, false, true>(q, grid, st) : launch_ix<MODE, int64_t, false, true>(q, grid, st);
+    return i32 ? launch_ix<MODE, uint32_t, false, false>(q, grid, st) : launch_ix<MODE, int64_t, false, false>(q, grid, st);
+}
+
+}  // namespace
+
+int DGM_LAUNCH(const StageParams& prm, void* stream) {
+    return launch_mode<DGM_MODE>(prm, static_cast<cudaStream_t>(stream));
+}
+#ifdef DGM_LAUNCH2
+int DGM_LAUNCH2(const StageParams& prm, void* stream) {
+    return launch_mode<MODE_LF_H>(prm, static_cast<cudaStream_t>(stream));
+}
+#endif
+
+}  // namespace dgm

@@ -1,0 +1,6 @@
+// Tangential-trace stage kernel: degree 1, double fields, LSRK4 stage.
+#define DGM_P 1
+#define DGM_REAL double
+#define DGM_MODE MODE_LSRK
+#define DGM_LAUNCH launch_t_p1_f64_lsrk
+#include "dgm_tkern_impl.cuh"

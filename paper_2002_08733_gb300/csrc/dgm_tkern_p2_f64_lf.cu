@@ -1,0 +1,7 @@
+// Tangential-trace stage kernel: degree 2, double fields, leapfrog half steps.
+#define DGM_P 2
+#define DGM_REAL double
+#define DGM_MODE MODE_LF_E
+#define DGM_LAUNCH2 launch_t_p2_f64_lfh
+#define DGM_LAUNCH launch_t_p2_f64_lf
+#include "dgm_tkern_impl.cuh"

@@ -1,0 +1,6 @@
+// Tangential-trace stage kernel: degree 4, float fields, right-hand side.
+#define DGM_P 4
+#define DGM_REAL float
+#define DGM_MODE MODE_RHS
+#define DGM_LAUNCH launch_t_p4_f32_rhs
+#include "dgm_tkern_impl.cuh"

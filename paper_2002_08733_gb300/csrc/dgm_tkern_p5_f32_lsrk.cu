@@ -1,0 +1,6 @@
+// Tangential-trace stage kernel: degree 5, float fields, LSRK4 stage.
+#define DGM_P 5
+#define DGM_REAL float
+#define DGM_MODE MODE_LSRK
+#define DGM_LAUNCH launch_t_p5_f32_lsrk
+#include "dgm_tkern_impl.cuh"
