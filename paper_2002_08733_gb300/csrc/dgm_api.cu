@@ -144,7 +144,7 @@ struct dgm_plan {
     // geometry buffer layout (byte offsets)
     size_t off_geo = 0, off_nbr = 0, off_pml = 0, off_src = 0, off_part = 0, off_status = 0,
            off_rec = 0, off_time = 0, off_geo32 = 0, off_fnb = 0, off_fnb32 = 0, off_tcb = 0,
-           bytes_tcb = 0, off_ops = 0, bytes_ops = 0, bytes_geom = 0;
+           bytes_tcb = 0, bytes_geom = 0;
     int n_rec = 0;
     std::vector<double> src_host;   // S * (SRC_HDR + 3N)
     bool have_src = false;
@@ -354,9 +354,10 @@ static int plan_create(dgm_plan** out, int64_t nv, const double* xyz, int64_t nt
             return fail(DGM_EINVAL, "degree-p operators are not submatrices of degree p + 1");
         }
     }
-    if (!mixed) {   // the kernels carry the reference operators as compiled literals: check them
-        const double* cs = ref_S_compiled(opt->p);
-        const double* cr = ref_R_compiled(opt->p);
+    {   // the kernels carry the reference operators as compiled literals: check them
+        // (a mixed-order plan's H operators are leading submatrices of these, see above)
+        const double* cs = ref_S_compiled(pE);
+        const double* cr = ref_R_compiled(pE);
         double worst = 0.0, scale = 0.0;
         for (size_t i = 0; i < P->S.size(); ++i) {
             worst = std::fmax(worst, std::fabs(P->S[i] - cs[i]));
@@ -404,10 +405,6 @@ static int plan_create(dgm_plan** out, int64_t nv, const double* xyz, int64_t nt
     P->bytes_tcb = (opt->precision == DGM_FP32 && !mixed) ? tc_image_bytes(opt->p) : 0;
     P->off_tcb = off;
     off = align256(off + P->bytes_tcb);
-    // dense reference operators of a mixed-order plan (S then R, degree p + 1)
-    P->bytes_ops = mixed ? (P->S.size() + P->R.size()) * size_t(kt->real_size) : 0;
-    P->off_ops = off;
-    off = align256(off + P->bytes_ops);
     // incident plane wave: FP64 table and per-stage jump terms, sized for every boundary face
     for (int64_t i = 0; i < 4 * K; ++i) P->n_bfaces += P->mesh.nbr[i] < 0;
     P->inc_nq = (pE + 6) * (pE + 6);
@@ -534,10 +531,12 @@ static bool tmap_fields(dgm_plan* P, void* base, int slot) {
     if (reinterpret_cast<uintptr_t>(base) % 16 != 0) return false;
     const cuuint64_t C = cuuint64_t(P->mesh.K) * cuuint64_t(P->opt.n_columns);
     const cuuint64_t row = C * cuuint64_t(P->kt->real_size);
-    const cuuint64_t dims[3] = {C, cuuint64_t(P->N), 6};
-    const cuuint64_t str[2] = {row, row * cuuint64_t(P->N)};
+    // [6][N][C], or all 3 (N + N_H) rows of a mixed-order plan at once
+    const cuuint64_t rows = P->mixed ? 3 * cuuint64_t(P->N + P->NH) : cuuint64_t(P->N), nb = P->mixed ? 1 : 6;
+    const cuuint64_t dims[3] = {C, rows, nb};
+    const cuuint64_t str[2] = {row, row * rows};
     for (int set = 0; set < TMAP_SETS; ++set) {
-        const cuuint32_t box[3] = {cuuint32_t(tmap_columns(set)), cuuint32_t(P->N), 6};
+        const cuuint32_t box[3] = {cuuint32_t(tmap_columns(set)), cuuint32_t(rows), cuuint32_t(nb)};
         if (!tmap_encode(P, &P->tmap_host[size_t(set) * TMAP_COUNT + slot], base, 3, dims, str, box))
             return false;
     }
@@ -564,8 +563,7 @@ static int build_tmaps(dgm_plan* P) {
     P->tmaps_ok = false;
     const int rs = P->kt->real_size;
     const int64_t K = P->mesh.K, S = P->opt.n_columns;
-    // (mixed-order plans run their own kernel on fields of 3 (N + N_H) rows)
-    if (P->mixed || K <= 0 || (K * S * rs) % 16 != 0 || (S > 1 && (S * rs) % 16 != 0) ||
+    if (K <= 0 || (K * S * rs) % 16 != 0 || (S > 1 && (S * rs) % 16 != 0) ||
         K * S >= (int64_t(1) << 31))
         return DGM_OK;
     if (tmap_encoder() == nullptr) return DGM_OK;
@@ -575,7 +573,7 @@ static int build_tmaps(dgm_plan* P) {
     const cuuint64_t Ke = cuuint64_t(K), row = cuuint64_t(K) * cuuint64_t(rs);   // row stride in bytes
     unsigned char* geo = P->geom + P->off_geo32;
     unsigned char* fcp = P->geom + P->off_fcp;
-    for (int set = 0; set < TMAP_SETS && rs == 4 && S == 1; ++set) {
+    for (int set = 0; set < TMAP_SETS && rs == 4 && S == 1 && !P->mixed; ++set) {
         const cuuint32_t te = cuuint32_t(tmap_columns(set));
         CUtensorMap* m = P->tmap_host.data() + size_t(set) * TMAP_COUNT;
         bool ok = true;
@@ -616,12 +614,11 @@ static int build_face_table(dgm_plan* P) {
         reinterpret_cast<double*>(P->geom + P->off_fnb), reinterpret_cast<float*>(P->geom + P->off_fnb32));
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "face table");
-    if (P->mixed) return DGM_OK;   // the mixed-order kernel forms its face terms itself
     StageParams prm;
     stage_params(P, prm);
     const bool sip = P->sip_alpha > 0.0;
     prm.sfid = sip ? reinterpret_cast<const int32_t*>(P->geom + P->off_sfid) : nullptr;
-    int rc = launch_face_consts(prm, P->kt->real_size, false, P->geom + P->off_fcp, P->stream);
+    int rc = P->mixed ? DGM_OK : launch_face_consts(prm, P->kt->real_size, false, P->geom + P->off_fcp, P->stream);
     if (!rc) rc = launch_tang_consts(prm, P->kt->real_size, sip, P->geom + P->off_fct, P->stream);
     return rc ? fail(rc, "face constants") : DGM_OK;
 }
@@ -676,18 +673,6 @@ int dgm_bind(dgm_plan* P, void* geom, void* fields0, void* fields1, void* res, v
                                  cudaMemcpyHostToDevice, st)) != cudaSuccess)
             return cuda_fail(e, "upload tensor-core operator image");
     }
-    std::vector<unsigned char> ops(P->bytes_ops);
-    if (P->bytes_ops) {
-        const size_t n = P->S.size() + P->R.size();
-        for (size_t i = 0; i < n; ++i) {
-            const double v = i < P->S.size() ? P->S[i] : P->R[i - P->S.size()];
-            if (P->kt->real_size == 8) std::memcpy(ops.data() + 8 * i, &v, 8);
-            else { const float f = float(v); std::memcpy(ops.data() + 4 * i, &f, 4); }
-        }
-        if ((e = cudaMemcpyAsync(P->geom + P->off_ops, ops.data(), ops.size(), cudaMemcpyHostToDevice,
-                                 st)) != cudaSuccess)
-            return cuda_fail(e, "upload mixed-order operators");
-    }
     if (P->n_inc > 0 &&
         (e = cudaMemcpyAsync(P->geom + P->off_inc, P->inc_host.data(), sizeof(double) * P->inc_host.size(),
                              cudaMemcpyHostToDevice, st)) != cudaSuccess)
@@ -725,7 +710,6 @@ static void stage_params(dgm_plan* P, StageParams& prm) {
     prm.tile_groups = P->tile_groups;
     prm.tc_b = P->bytes_tcb ? static_cast<const void*>(P->geom + P->off_tcb) : nullptr;
     prm.K_active = P->k_active;
-    prm.ops = P->bytes_ops ? static_cast<const void*>(P->geom + P->off_ops) : nullptr;
     prm.inc = P->n_inc > 0 ? static_cast<const void*>(P->geom + P->off_incv) : nullptr;
     prm.sip_alpha = P->sip_alpha;
     prm.n_facets = P->n_facets;

@@ -109,7 +109,6 @@ struct StageParams {
     int32_t tile_groups;  // tile visiting order: G interleaved segments (1: in order)
     const void* tc_b;     // tensor-core variant: B operand image (TcShape<P>::B_BYTES), or null
     int64_t K_active;     // elements updated: the first K_active (the rest are halo copies)
-    const void* ops;      // mixed-order plans: dense reference operators S, R of degree p + 1
     const void* inc;      // incident faces: [i][NF][3] reference-frame jump terms
                           // 2 A^T E_inc traced on face mode m at the stage time (R), or null
     // interior penalty with a facet field (null when off): per (face, element)
@@ -201,7 +200,7 @@ struct KernelTable {
 };
 
 const KernelTable* kernel_table(int p, int precision);
-// Mixed-order plans (E of degree pE, H of degree pE - 1; dgm_mixed.cu).
+// Mixed-order plans (E of degree pE, H of degree pE - 1).
 const KernelTable* kernel_table_mixed(int pE, int precision);
 
 // Host setup (dgm_setup.cpp)

@@ -120,6 +120,20 @@ int launch_p5_f32_lsrk_v2(const StageParams&, void*);
 int launch_p5_f32_lsrk_v3(const StageParams&, void*);
 int launch_p5_f32_adj(const AdjParams&, void*);
 
+// mixed orders (E of degree p, H of degree p - 1)
+int launch_t_m2_f32_lsrk(const StageParams&, void*);
+int launch_t_m2_f32_rhs(const StageParams&, void*);
+int launch_t_m2_f64_lsrk(const StageParams&, void*);
+int launch_t_m2_f64_rhs(const StageParams&, void*);
+int launch_t_m3_f32_lsrk(const StageParams&, void*);
+int launch_t_m3_f32_rhs(const StageParams&, void*);
+int launch_t_m3_f64_lsrk(const StageParams&, void*);
+int launch_t_m3_f64_rhs(const StageParams&, void*);
+int launch_t_m4_f32_lsrk(const StageParams&, void*);
+int launch_t_m4_f32_rhs(const StageParams&, void*);
+int launch_t_m4_f64_lsrk(const StageParams&, void*);
+int launch_t_m4_f64_rhs(const StageParams&, void*);
+
 namespace {
 
 int launch_p1_f32(const StageParams& prm, int mode, void* st) {
@@ -261,6 +275,42 @@ int launch_p5_f32(const StageParams& prm, int mode, void* st) {
     }
 }
 
+int launch_m2_f32(const StageParams& prm, int mode, void* st) {
+    if (mode == MODE_RHS) return launch_t_m2_f32_rhs(prm, st);
+    if (mode == MODE_LSRK) return launch_t_m2_f32_lsrk(prm, st);
+    return DGM_EUNSUP;
+}
+
+int launch_m2_f64(const StageParams& prm, int mode, void* st) {
+    if (mode == MODE_RHS) return launch_t_m2_f64_rhs(prm, st);
+    if (mode == MODE_LSRK) return launch_t_m2_f64_lsrk(prm, st);
+    return DGM_EUNSUP;
+}
+
+int launch_m3_f32(const StageParams& prm, int mode, void* st) {
+    if (mode == MODE_RHS) return launch_t_m3_f32_rhs(prm, st);
+    if (mode == MODE_LSRK) return launch_t_m3_f32_lsrk(prm, st);
+    return DGM_EUNSUP;
+}
+
+int launch_m3_f64(const StageParams& prm, int mode, void* st) {
+    if (mode == MODE_RHS) return launch_t_m3_f64_rhs(prm, st);
+    if (mode == MODE_LSRK) return launch_t_m3_f64_lsrk(prm, st);
+    return DGM_EUNSUP;
+}
+
+int launch_m4_f32(const StageParams& prm, int mode, void* st) {
+    if (mode == MODE_RHS) return launch_t_m4_f32_rhs(prm, st);
+    if (mode == MODE_LSRK) return launch_t_m4_f32_lsrk(prm, st);
+    return DGM_EUNSUP;
+}
+
+int launch_m4_f64(const StageParams& prm, int mode, void* st) {
+    if (mode == MODE_RHS) return launch_t_m4_f64_rhs(prm, st);
+    if (mode == MODE_LSRK) return launch_t_m4_f64_lsrk(prm, st);
+    return DGM_EUNSUP;
+}
+
 }  // namespace
 
 extern const KernelTable kernels_p1_f32 = {launch_p1_f32, 4, launch_p1_f32_adj, 5};
@@ -272,5 +322,13 @@ extern const KernelTable kernels_p3_f64 = {launch_p3_f64, 8, launch_p3_f64_adj, 
 extern const KernelTable kernels_p4_f32 = {launch_p4_f32, 4, launch_p4_f32_adj, 4};
 extern const KernelTable kernels_p4_f64 = {launch_p4_f64, 8, launch_p4_f64_adj, 1};
 extern const KernelTable kernels_p5_f32 = {launch_p5_f32, 4, launch_p5_f32_adj, 4};
+
+// Kernels of mixed-order plans: E degree pE = 2..4 (H degree pE - 1).
+const KernelTable* kernel_table_mixed(int pE, int precision) {
+    static const KernelTable f32[] = {{launch_m2_f32, 4, nullptr, 1}, {launch_m3_f32, 4, nullptr, 1}, {launch_m4_f32, 4, nullptr, 1}};
+    static const KernelTable f64[] = {{launch_m2_f64, 8, nullptr, 1}, {launch_m3_f64, 8, nullptr, 1}, {launch_m4_f64, 8, nullptr, 1}};
+    if (pE < 2 || pE > 4) return nullptr;
+    return precision == DGM_FP64 ? &f64[pE - 2] : (precision == DGM_FP32 ? &f32[pE - 2] : nullptr);
+}
 
 }  // namespace dgm

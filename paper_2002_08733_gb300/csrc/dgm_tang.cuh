@@ -48,6 +48,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 
 #include "dgm_internal.h"
 #include "dgm_ops_gen.cuh"
@@ -140,11 +141,21 @@ __global__ void tang_consts_kernel(const StageParams prm, bool sip, R* __restric
     out[int64_t(TG_IH) * K + e] = R(-1.0 / (mu * det));
 }
 
-// shared memory: the tile's coefficients [6N][TE], the face quantities
+// Mixed orders (MX): E of degree P, H of degree P - 1.  The bases are hierarchical,
+// so H's operators are those of degree P - 1, the curl of H tested against E is the
+// degree P - 1 curl, the curl of E tested against H the rows of the degree-P one,
+// and an E jump enters the H flux with its first face modes.
+// Field rows: E component k, mode l at k N + l, H at 3 N + k N_H + l.
+template <int P, bool MX> __host__ __device__ constexpr int deg_h() { return MX ? P - 1 : P; }
+template <int P, bool MX> __host__ __device__ constexpr int field_rows() {
+    return 3 * (nmodes(P) + nmodes(deg_h<P, MX>()));
+}
+
+// shared memory: the tile's coefficients [rows][TE], the face quantities
 // [face][field][tangent][NF][TE] (jumps, then fluxes), an mbarrier
-template <int P, typename R, int TE>
+template <int P, typename R, int TE, bool MX = false>
 __host__ __device__ constexpr size_t tang_smem_bytes() {
-    return sizeof(R) * size_t(TE) * (6 * nmodes(P) + 16 * nfmodes(P)) + 16;
+    return sizeof(R) * size_t(TE) * (field_rows<P, MX>() + 16 * nfmodes(P)) + 16;
 }
 
 // minus the own trace of face f of the row block at v (row stride TE), less that at v0 on face 0
@@ -201,11 +212,13 @@ struct Column {
 };
 
 // Phase B of one thread: rows [LO, HI) of the three components of field F
-// (0: E, 1: H).  us, gs: shared memory at this thread's columns.
-template <int P, typename R, int TE, int MODE, typename IX, bool PML, int LO, int HI>
+// (0: E, 1: H) of degree P, the other field of degree PO.  us, gs: shared memory
+// at this thread's column; r0, ro: first field rows of this and the other field;
+// NF: face modes per row group of gs.
+template <int P, int PO, int NF, typename R, int TE, int MODE, typename IX, bool PML, int LO, int HI>
 __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R* us, const R* gs,
-                                          const Column<IX>& id) {
-    constexpr int N = nmodes(P), NF = nfmodes(P), NR = HI - LO;
+                                          const Column<IX>& id, int r0, int ro) {
+    constexpr int N = nmodes(P), NR = HI - LO;
     constexpr bool LF = MODE == MODE_LF_E || MODE == MODE_LF_H;
     // residual rows requested before the arithmetic where the registers allow it
     constexpr bool EARLY = MODE == MODE_LSRK && 3 * NR * int(sizeof(R)) <= tang_early_bytes<P, R, PML>();
@@ -213,8 +226,7 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
     const IX K = prm.K, C = id.C;
     const bool active = id.active;
     const R ca = coef(prm.a, prm.a_f), cb = coef(prm.b, prm.b_f), dt = coef(prm.dt, prm.dt_f);
-    const int fb = 3 * F;
-    const IX gb = IX(fb * N + LO) * C + id.col;
+    const IX gb = IX(r0 + LO) * C + id.col;
     const R* __restrict__ resi = static_cast<const R*>(prm.res);
     const bool ld = active && ca != R(0);
     R rv[EARLY ? NR : 1][3];
@@ -241,7 +253,7 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
     LiftOp<P, 0>::template apply<R, LO, HI>(g + NF * TE, TE, a2);
 #pragma unroll
     for (int l = LO; l < HI; ++l) a0[l] = (a1[l] + a2[l]) * R(-1);
-    CurlOp<P>::template apply<R, LO, HI>(us + (3 - fb) * N * TE, N * TE, TE, a0, a1, a2);
+    CurlOp<PO>::template apply<R, LO, HI>(us + ro * TE, nmodes(PO) * TE, TE, a0, a1, a2);
     LiftOp<P, 1>::template apply<R, LO, HI>(g + 4 * NF * TE, TE, a1);
     LiftOp<P, 1>::template apply<R, LO, HI>(g + 5 * NF * TE, TE, a2);
     LiftOp<P, 2>::template apply<R, LO, HI>(g + 8 * NF * TE, TE, a0);
@@ -251,7 +263,7 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
     if (!active) return;
 
     if (F == 0 && prm.src != nullptr) {
-        const double* rec = prm.src + IX(id.s) * (SRC_HDR + 3 * N);
+        const double* rec = prm.src + IX(id.s) * (SRC_HDR + 3 * N);   // (E's N)
         if (rec[0] >= 0.0 && IX(rec[0]) == id.e) {   // -1 marks a column without a source
             const double tt = prm.tdev ? *prm.tdev + prm.t : prm.t;
             // the rows carry the factor s_T = sign of det A
@@ -277,7 +289,7 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
         a2[l] = fmaa(b22, r2, fmaa(b12, r1, b02 * r0));
     }
     if constexpr (PML) {
-        const int32_t pi = prm.pml[id.e];
+        const int32_t pi = prm.pml != nullptr ? prm.pml[id.e] : -1;
         if (pi >= 0) {
             // PML: D -> A^T D A^-T for D = eta, Sigma, xi ; leapfrog works
             // per Cartesian component in the physical frame
@@ -304,14 +316,14 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
             const IX acol = IX(pi) * IX(prm.S) + id.s;
             auto load_aux = [&](const R* p, IX row) -> R { return p[row * C2 + acol]; };
             auto store_aux = [&](R* p, IX row, R v) { p[row * C2 + acol] = v; };
-            const IX ab = IX(fb * N + LO);
+            const IX ab = IX(r0 + LO);   // (both fields of degree P)
             if constexpr (LF) {
                 // Leapfrog with the PML terms by the trapezoid rule (Sec. V), X = A^-T x:
                 //   X_new = ((1 - dt eta/2) X + dt (A^-T du - A^-T aux / mat)) / (1 + dt eta/2)
                 // then the other field's auxiliary, Y = A^-T (other field), mat' its material:
                 //   Z_new = ((1 - dt sigma/2) Z + dt mat' xi Y) / (1 + dt sigma/2)
                 const R omat = table(prm.geo_r, G_EPS + 1 - F);
-                const IX abo = IX((3 - fb) * N + LO);
+                const IX abo = IX(ro + LO);
                 R* auxl = static_cast<R*>(prm.aux_out);   // in place: aux_out == aux
                 R xx[3], xy[3], za[3], zb[3];
                 const R ndi = imat * -dt;
@@ -346,8 +358,8 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
                         R ov[3], uv[3], Xn[3], Zn[3];
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
-                            uv[k] = us[((fb + k) * N + l) * TE];
-                            ov[k] = us[((3 - fb + k) * N + l) * TE];
+                            uv[k] = us[(r0 + k * N + l) * TE];
+                            ov[k] = us[(ro + k * N + l) * TE];
                         }
 #pragma unroll
                         for (int a = 0; a < 3; ++a) {
@@ -407,7 +419,7 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
                         const int l = LO + i0 + i;
                         R uv[3], d[3];
 #pragma unroll
-                        for (int k = 0; k < 3; ++k) uv[k] = us[((fb + k) * N + l) * TE];
+                        for (int k = 0; k < 3; ++k) uv[k] = us[(r0 + k * N + l) * TE];
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
                             d[k] = fmaa(ni, av[i][k], fmaa(ETA[k][2], uv[2], fmaa(ETA[k][1], uv[1], ETA[k][0] * uv[0])));
@@ -459,21 +471,22 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
                 } else if (MODE == MODE_LSRK) {
                     const R rr = fmaa(ca, rc[i][k], du[k]);
                     res[gi] = rr;
-                    uo[gi] = fmaa(cb, rr, us[((fb + k) * N + l) * TE]);
+                    uo[gi] = fmaa(cb, rr, us[(r0 + k * N + l) * TE]);
                 } else {
-                    uo[gi] = us[((fb + k) * N + l) * TE] + du[k];
+                    uo[gi] = us[(r0 + k * N + l) * TE] + du[k];
                 }
             }
         }
     }
 }
 
-template <int P, typename R, int TE, int MODE, typename IX, bool PML, int NPART>
-__device__ __forceinline__ void tang_part(const StageParams& prm, int F, int part, const R* us, const R* gs,
-                                          const Column<IX>& id) {
+template <int P, int PO, int NF, typename R, int TE, int MODE, typename IX, bool PML, int NPART>
+__device__ __forceinline__ void tang_parts(const StageParams& prm, int F, int part, const R* us, const R* gs,
+                                           const Column<IX>& id, int r0, int ro) {
     static_assert(NPART == 2 || NPART == 4, "row parts");
-#define DGM_ROWS(K_) \
-    tang_rows<P, R, TE, MODE, IX, PML, tang_split<P, R, PML>(NPART, K_), tang_split<P, R, PML>(NPART, K_ + 1)>(prm, F, us, gs, id)
+#define DGM_ROWS(K_)                                                                                       \
+    tang_rows<P, PO, NF, R, TE, MODE, IX, PML, tang_split<P, R, PML>(NPART, K_),                           \
+              tang_split<P, R, PML>(NPART, K_ + 1)>(prm, F, us, gs, id, r0, ro)
     if constexpr (NPART == 2) {
         if (part == 0) DGM_ROWS(0);
         else DGM_ROWS(1);
@@ -488,21 +501,36 @@ __device__ __forceinline__ void tang_part(const StageParams& prm, int F, int par
 #undef DGM_ROWS
 }
 
+// one code path for both fields where their degrees are equal
+template <int P, typename R, int TE, int MODE, typename IX, bool PML, bool MX, int NPART>
+__device__ __forceinline__ void tang_part(const StageParams& prm, int F, int part, const R* us, const R* gs,
+                                          const Column<IX>& id) {
+    constexpr int PH = deg_h<P, MX>(), N = nmodes(P), NF = nfmodes(P);
+    if constexpr (!MX) {
+        tang_parts<P, P, NF, R, TE, MODE, IX, PML, NPART>(prm, F, part, us, gs, id, 3 * F * N, 3 * (1 - F) * N);
+    } else {
+        if (F == 0) tang_parts<P, PH, NF, R, TE, MODE, IX, PML, NPART>(prm, 0, part, us, gs, id, 0, 3 * N);
+        else tang_parts<PH, P, NF, R, TE, MODE, IX, PML, NPART>(prm, 1, part, us, gs, id, 3 * N, 0);
+    }
+}
+
 // IX: type of the element/column/row index arithmetic (uint32_t when every
 // index of the plan fits, else int64_t).  MINB: resident CTAs per SM asked of
 // the register allocator.  NG = 4: thread groups = faces (both fields), then
 // (field, half of the rows); NG = 8: (face, field), then (field, quarter of the
 // rows), the two fields of a face in the two halves of a warp (TE = 16) or in
 // two neighbouring warps (TE = 32).
-template <int P, typename R, int TE, int NG, int MODE, typename IX, bool SIP, bool PML, int MINB>
+template <int P, typename R, int TE, int NG, int MODE, typename IX, bool SIP, bool PML, bool MX, int MINB>
 __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams prm) {
     static_assert((TE == 32 && (NG == 4 || NG == 8)) || (TE == 16 && NG == 8), "tile shape");
-    static_assert(!SIP || MODE == MODE_LSRK || MODE == MODE_RHS, "interior penalty modes");
+    static_assert(!(SIP || MX) || MODE == MODE_LSRK || MODE == MODE_RHS, "interior penalty and mixed-order modes");
+    static_assert(!(MX && (SIP || PML)), "mixed orders: no penalty, no PML");
     constexpr int N = nmodes(P), NF = nfmodes(P);
+    constexpr int PH = deg_h<P, MX>(), NH = nmodes(PH), NFH = nfmodes(PH), ROWS = field_rows<P, MX>();
     constexpr bool LF = MODE == MODE_LF_E || MODE == MODE_LF_H;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    R* us = reinterpret_cast<R*>(smem_raw);   // [6N][TE]
-    R* gs = us + 6 * N * TE;                  // [4][2][2][NF][TE]
+    R* us = reinterpret_cast<R*>(smem_raw);   // [ROWS][TE]
+    R* gs = us + ROWS * TE;                   // [4][2][2][NF][TE]
     uint64_t* bar = reinterpret_cast<uint64_t*>(gs + 16 * NF * TE);
 
     const int c = threadIdx.x % TE;
@@ -523,14 +551,14 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
     const R* u = static_cast<const R*>(prm.u);   // may alias u_out (leapfrog)
     auto coef = [&](double d, float f) { return sizeof(R) == 4 ? R(f) : R(d); };
 
-    // The tile: one bulk tensor copy of the box [6][N][TE] where the plan has a
+    // The tile: one bulk tensor copy of its rows where the plan has a
     // map of u (aligned rows), issued first and waited for by thread 0; columns
     // past the end arrive as zeros.  Otherwise every thread loads its rows.
     const bool bulk = prm.tm_u >= 0 && (tc::smem_addr(smem_raw) & 127u) == 0;
     if (bulk && threadIdx.x == 0) {
-        static_assert(sizeof(R) * TE * 6 * N < (1u << 20), "bytes of an mbarrier phase");
+        static_assert(sizeof(R) * TE * ROWS < (1u << 20), "bytes of an mbarrier phase");
         tc::mbar_init(bar, 1);
-        bulk::arrive_expect_tx(bar, uint32_t(sizeof(R)) * TE * 6 * N);
+        bulk::arrive_expect_tx(bar, uint32_t(sizeof(R)) * TE * ROWS);
         bulk::load_3d(us, static_cast<const char*>(prm.tmaps) + prm.tm_u * TMAP_BYTES, int(x0), 0, 0, bar);
     }
 
@@ -549,16 +577,23 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
     const int q0 = QF + (NG == 4 ? 0 : half * QN);
     constexpr bool AHEAD = P <= 3 || (P == 4 && PML);   // gathers of a slanted neighbour face in two register sets
     R vn[N], vm[AHEAD ? N : 1];
-    auto fetch = [&](int comp, R* v) {   // the neighbour's coefficients of one component
-        const R* p = u + (IX(comp * N) * C + nc);
+    // first field row of component `comp` of a field
+    auto row_of = [&](int fld, int comp) { return fld == 0 ? comp * N : 3 * N + comp * NH; };
+    auto fetch = [&](int fld, int comp, R* v) {   // the neighbour's coefficients of one component
+        const R* p = u + (IX(row_of(fld, comp)) * C + nc);
+        if (!MX || fld == 0) {
 #pragma unroll
-        for (int l = 0; l < N; ++l) v[l] = p[IX(l) * C];
+            for (int l = 0; l < N; ++l) v[l] = p[IX(l) * C];
+        } else {
+#pragma unroll
+            for (int l = 0; l < NH; ++l) v[l] = p[IX(l) * C];
+        }
     };
     auto gather = [&](int q) {
         if (!has) return;
-        fetch((q >> 1) * 3 + tang_comp(nf, q & 1), vn);
+        fetch(q >> 1, tang_comp(nf, q & 1), vn);
         if constexpr (AHEAD) {
-            if (nf == 0) fetch((q >> 1) * 3, vm);
+            if (nf == 0) fetch(q >> 1, 0, vm);
         }
     };
     gather(q0);
@@ -581,55 +616,63 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
             return;
         }
     } else {
-        constexpr int UR = (6 * N + NG - 1) / NG, BATCH = UR < 16 ? UR : 16;
+        constexpr int UR = (ROWS + NG - 1) / NG, BATCH = UR < 16 ? UR : 16;
 #pragma unroll 1
         for (int i0 = 0; i0 < UR; i0 += BATCH) {
             R tmp[BATCH];
 #pragma unroll
             for (int i = 0; i < BATCH; ++i) {
                 const int q = grp + (i0 + i) * NG;
-                tmp[i] = (active && q < 6 * N) ? u[IX(q) * C + id.col] : R(0);
+                tmp[i] = (active && q < ROWS) ? u[IX(q) * C + id.col] : R(0);
             }
 #pragma unroll
             for (int i = 0; i < BATCH; ++i) {
                 const int q = grp + (i0 + i) * NG;
-                if (q < 6 * N) us[q * TE + c] = tmp[i];
+                if (q < ROWS) us[q * TE + c] = tmp[i];
             }
         }
         __syncthreads();
     }
     R* gf = gs + f * 4 * NF * TE + c;   // this face's rows: [field][tangent][NF]
     const bool inc = code <= -2 && prm.inc != nullptr;
-#pragma unroll 1
-    for (int k = 0; k < QN; ++k) {
-        const int q = q0 + k, fld = q >> 1, i = q & 1;
-        const R* v0 = us + fld * 3 * N * TE + c;
-        R acc[NF];
-        own_trace<P, R, TE>(f, v0 + tang_comp(f, i) * N * TE, v0, acc);
+    // jump of item q of a field of degree PF: own trace, then the neighbour's
+    auto item = [&](auto deg, int q) {
+        constexpr int PF = decltype(deg)::value, NP = nmodes(PF), NPF = nfmodes(PF);
+        const int fld = q >> 1, i = q & 1;
+        const R* v0 = us + row_of(fld, 0) * TE + c;
+        R acc[NPF];
+        own_trace<PF, R, TE>(f, v0 + tang_comp(f, i) * NP * TE, v0, acc);
         if (has) {
+            R(&w)[NP] = *reinterpret_cast<R(*)[NP]>(vn);
             if (nf == 0) {   // slanted neighbour face: less component 0
                 if constexpr (AHEAD) {
 #pragma unroll
-                    for (int l = 0; l < N; ++l) vn[l] -= vm[l];
+                    for (int l = 0; l < NP; ++l) w[l] -= vm[l];
                 } else {
-                    const R* p0 = u + (IX(fld * 3 * N) * C + nc);
+                    const R* p0 = u + (IX(row_of(fld, 0)) * C + nc);
 #pragma unroll
-                    for (int l = 0; l < N; ++l) vn[l] -= p0[IX(l) * C];
+                    for (int l = 0; l < NP; ++l) w[l] -= p0[IX(l) * C];
                 }
             }
-            jump_trace<P, R>(nf, vn, acc);
+            jump_trace<PF, R>(nf, w, acc);
         } else {
             // boundary face, acc = -own: PEC (e+ = -e-, h+ = h-) or incident
             // (e+ = e- + 2 E_inc, h+ = -h-; the E_inc part is added with the flux)
             const R al = ((fld == 0) != inc) ? R(2) : R(0);
 #pragma unroll
-            for (int m = 0; m < NF; ++m) acc[m] *= al;
+            for (int m = 0; m < NPF; ++m) acc[m] *= al;
         }
         // central flux of the leapfrog: gamma_1 = c tau_2, gamma_2 = -c tau_1 of the other field
         const R cc = LF ? (MODE == MODE_LF_E ? cE : cH) * R(i ? 1 : -1) : R(1);
         R* o = gf + (LF ? 2 * (1 - fld) + 1 - i : q) * NF * TE;
 #pragma unroll
-        for (int m = 0; m < NF; ++m) o[m * TE] = LF ? cc * acc[m] : acc[m];
+        for (int m = 0; m < NPF; ++m) o[m * TE] = LF ? cc * acc[m] : acc[m];
+    };
+#pragma unroll 1
+    for (int k = 0; k < QN; ++k) {
+        const int q = q0 + k;
+        if (!MX || (q >> 1) == 0) item(std::integral_constant<int, P>{}, q);
+        else item(std::integral_constant<int, PH>{}, q);
         if (k + 1 < QN) gather(q + 1);
     }
     if constexpr (!LF) {
@@ -692,8 +735,9 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
                 const int m = mb + j;
                 if (SIP && m >= m1) break;
                 R* o = gf + m * TE;
+                const bool hm = !MX || m < NFH;   // a mode of H's traces
                 R e1 = o[0], e2 = o[NF * TE];
-                const R h1 = o[2 * NF * TE], h2 = o[3 * NF * TE];
+                const R h1 = hm ? o[2 * NF * TE] : R(0), h2 = hm ? o[3 * NF * TE] : R(0);
                 if (ic != nullptr) {
                     const R z = f == 0 ? ic[3 * m] : R(0);
                     e1 += ic[3 * m + tang_comp(f, 0)] - z;
@@ -701,8 +745,10 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
                 }
                 R p1 = fmaa(cE, h2, fmaa(e22, e1, ne12 * e2));
                 R p2 = fmaa(ncE, h1, fmaa(e11, e2, ne12 * e1));
-                o[2 * NF * TE] = fmaa(cH, e2, fmaa(h12, h2, nh22 * h1));
-                o[3 * NF * TE] = fmaa(ncH, e1, fmaa(h12, h1, nh11 * h2));
+                if (hm) {
+                    o[2 * NF * TE] = fmaa(cH, e2, fmaa(h12, h2, nh22 * h1));
+                    o[3 * NF * TE] = fmaa(ncH, e1, fmaa(h12, h1, nh11 * h2));
+                }
                 if constexpr (SIP) {
                     // both sides: gamma += m_f x (A^T h_s); owner: dh_s/dt =
                     // -ks A (m_f x de) = -ks sigma (A t_1 de_2 - A t_2 de_1)
@@ -736,14 +782,14 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
     if constexpr (LF) {
         // one field; NG = 8 would need eight row parts, its second half idles
         constexpr int F = MODE == MODE_LF_E ? 0 : 1;
-        if (grp < 4) tang_part<P, R, TE, MODE, IX, PML, 4>(prm, F, grp, us + c, gs + c, id);
+        if (grp < 4) tang_part<P, R, TE, MODE, IX, PML, MX, 4>(prm, F, grp, us + c, gs + c, id);
     } else if constexpr (NG == 4) {
-        constexpr bool BAL = tang_balance<P, R, PML>();
+        constexpr bool BAL = tang_balance<P, R, PML>() && !MX;
         const int F = BAL ? grp >> 1 : grp & 1;
         const int part = BAL ? (grp == 1 || grp == 2 ? 0 : 1) : grp >> 1;
-        tang_part<P, R, TE, MODE, IX, PML, 2>(prm, F, part, us + c, gs + c, id);
+        tang_part<P, R, TE, MODE, IX, PML, MX, 2>(prm, F, part, us + c, gs + c, id);
     } else {
-        tang_part<P, R, TE, MODE, IX, PML, 4>(prm, grp & 1, grp >> 1, us + c, gs + c, id);
+        tang_part<P, R, TE, MODE, IX, PML, MX, 4>(prm, grp & 1, grp >> 1, us + c, gs + c, id);
     }
 }
 

@@ -1,7 +1,8 @@
 // Body of one translation unit of the tangential-trace stage kernel: instantiates
 // tang_kernel for one polynomial degree (DGM_P), one field precision (DGM_REAL)
 // and one mode (DGM_MODE; MODE_LF_E with DGM_LAUNCH2 also instantiates
-// MODE_LF_H), and exports its launchers.  Included by the
+// MODE_LF_H; DGM_MIXED: E of degree DGM_P, H of
+// DGM_P - 1), and exports its launchers.  Included by the
 // dgm_tkern_p<P>_<precision>_<mode>.cu files; one mode per file keeps the
 // heavily unrolled kernels compiling in parallel.
 #include <cuda_runtime.h>
@@ -41,7 +42,12 @@ struct Shape {
 };
 
 // the interior penalty runs in the default shape
-#ifndef DGM_TE
+#ifdef DGM_MIXED
+constexpr bool kMX = true;   // E of degree kP, H of degree kP - 1
+#else
+constexpr bool kMX = false;
+#endif
+#if !defined(DGM_TE) && !defined(DGM_MIXED)
 constexpr bool kSIP = true;
 #else
 constexpr bool kSIP = false;
@@ -50,9 +56,9 @@ constexpr bool kSIP = false;
 template <int MODE, typename IX, bool SIP, bool PML>
 int launch_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
     using Sh = Shape<MODE, SIP, PML>;
-    constexpr size_t smem = tang_smem_bytes<kP, Real, Sh::TE>();
+    constexpr size_t smem = tang_smem_bytes<kP, Real, Sh::TE, kMX>();
     static bool configured = false;
-    auto k = tang_kernel<kP, Real, Sh::TE, Sh::NG, MODE, IX, SIP, PML, Sh::MINB>;
+    auto k = tang_kernel<kP, Real, Sh::TE, Sh::NG, MODE, IX, SIP, PML, kMX, Sh::MINB>;
     if (!configured) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
             cudaSuccess)
@@ -103,9 +109,12 @@ int launch_mode(const StageParams& prm, cudaStream_t st) {
             return DGM_EUNSUP;
         }
     }
-    if (q.pml != nullptr && q.npml > 0)
-        return i32 ? launch_ix<MODE, uint32_t, false, true>(q, grid, st) : launch_ix<MODE, int64_t, false, true>(q, grid, st);
-    return i32 ? launch_ix<MODE, uint32_t, false, false>(q, grid, st) : launch_ix<MODE, int64_t, false, false>(q, grid, st);
+    // (64-bit indices: the PML instantiation serves plans without a layer too)
+    if (!i32) return launch_ix<MODE, int64_t, false, !kMX>(q, grid, st);
+    if constexpr (!kMX) {
+        if (q.pml != nullptr && q.npml > 0) return launch_ix<MODE, uint32_t, false, true>(q, grid, st);
+    }
+    return launch_ix<MODE, uint32_t, false, false>(q, grid, st);
 }
 
 }  // namespace

@@ -1,0 +1,8 @@
+// Tangential-trace stage kernel, mixed orders: E of degree 2, H of degree 1,
+// double fields, LSRK4 stage.
+#define DGM_P 2
+#define DGM_REAL double
+#define DGM_MODE MODE_LSRK
+#define DGM_MIXED
+#define DGM_LAUNCH launch_t_m2_f64_lsrk
+#include "dgm_tkern_impl.cuh"

@@ -1,0 +1,8 @@
+// Tangential-trace stage kernel, mixed orders: E of degree 3, H of degree 2,
+// float fields, right-hand side.
+#define DGM_P 3
+#define DGM_REAL float
+#define DGM_MODE MODE_RHS
+#define DGM_MIXED
+#define DGM_LAUNCH launch_t_m3_f32_rhs
+#include "dgm_tkern_impl.cuh"

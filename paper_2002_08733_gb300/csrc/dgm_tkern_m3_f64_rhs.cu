@@ -1,0 +1,8 @@
+// Tangential-trace stage kernel, mixed orders: E of degree 3, H of degree 2,
+// double fields, right-hand side.
+#define DGM_P 3
+#define DGM_REAL double
+#define DGM_MODE MODE_RHS
+#define DGM_MIXED
+#define DGM_LAUNCH launch_t_m3_f64_rhs
+#include "dgm_tkern_impl.cuh"
