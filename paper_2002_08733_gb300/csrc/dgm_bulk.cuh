@@ -40,5 +40,14 @@ __device__ __forceinline__ void load_3d(void* dst, const void* tmap, int x, int 
         : "memory");
 }
 
+// Programmatic dependent launch: wait until the launch before this one has ended
+// and its writes are visible (at once when this launch was an ordinary one), then
+// let the next one start.  Every thread of a grid passes here before it ends, so
+// that a launch that waits for this one has waited for all before it too.
+__device__ __forceinline__ void wait_previous_launch() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 }  // namespace bulk
 }  // namespace dgm

@@ -133,7 +133,39 @@ struct StageParams {
     const void* tm_f1;
     const void* tm_fw;    // the autotuner's scratch field buffer (map TM_UW), or null
     int32_t tm_u;
+    // 1: the launch may start while the one before it in the stream still runs
+    // (programmatic dependent launch); tang_kernel and lf_kernel then wait for it
+    // before they touch fields, auxiliaries, facet values or incident terms.  The
+    // plan's tables are read before that wait, so the first launch of a call is 0.
+    int32_t pdl;
 };
+
+// Launch of `k` in clusters of `cluster` CTAs, with the programmatic-dependent-launch
+// attribute when pdl is set.
+template <typename... A>
+inline cudaError_t launch_ex(void (*k)(A...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, bool pdl,
+                             unsigned cluster, A... args) {
+    cudaLaunchAttribute at[2] = {};
+    unsigned n = 0;
+    if (pdl) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = cluster;
+        at[n].val.clusterDim.y = 1;
+        at[n++].val.clusterDim.z = 1;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
 
 // Tensor maps (CUtensorMap, 128 bytes each) of one tile width, all with the
 // tile's columns as the innermost box dimension: the field buffers as

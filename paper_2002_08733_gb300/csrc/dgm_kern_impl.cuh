@@ -1,6 +1,6 @@
 // Body of one kernel translation unit: instantiates the fused stage kernel for
 // one polynomial degree (DGM_P), one field precision (DGM_REAL) and one mode
-// (DGM_MODE) and exports its launcher DGM_LAUNCH.  Included by the
+// (DGM_MODE; DGM_LF: both leapfrog half steps) and exports its launcher DGM_LAUNCH.  Included by the
 // dgm_kern_p<P>_<precision>_<mode>.cu files; one mode per file keeps the
 // heavily unrolled kernels compiling in parallel.
 #include <cuda_runtime.h>
@@ -14,6 +14,8 @@
 #include "dgm_adjoint.cuh"
 #elif defined(DGM_PAIR)
 #include "dgm_stage2.cuh"
+#elif defined(DGM_LF)
+#include "dgm_lf.cuh"
 #else
 #include "dgm_stage.cuh"
 #endif
@@ -113,6 +115,42 @@ int launch_mode(const StageParams& prm, cudaStream_t st) {
     return (!q.force_index64 && fits_32bit(q)) ? launch_pair_ix<uint32_t>(q, grid, st)
                                                : launch_pair_ix<int64_t>(q, grid, st);
 }
+#elif defined(DGM_LF)
+// leapfrog half steps
+template <int MODE, typename IX>
+int launch_lf_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
+    constexpr size_t smem = lf_smem_bytes<kP, Real, 32>();
+    static bool configured = false;
+    auto k = lf_kernel<kP, Real, 32, MODE, IX>;
+    if (!configured) {
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
+            cudaSuccess)
+            return DGM_ECUDA;
+        configured = true;
+    }
+    return launch_ex(k, grid, 32 * LF_NG, smem, st, q.pdl != 0, 1, q) == cudaSuccess ? DGM_OK : DGM_ECUDA;
+}
+
+// every index below 2^32: field rows, auxiliaries, geometry, face constants
+// (FC_ROWS x K), incident terms (3 NF per boundary face)
+bool fits_32bit(const StageParams& p) {
+    const uint64_t lim = uint64_t(1) << 32;
+    const uint64_t K = uint64_t(p.K), C = K * uint64_t(p.S);
+    const uint64_t N = uint64_t(nmodes(kP)), NF = uint64_t(nfmodes(kP));
+    return 6 * N * C < lim && 6 * N * uint64_t(p.npml) * uint64_t(p.S) < lim &&
+           uint64_t(FC_ROWS) * K < lim && 12 * NF * K < lim;
+}
+
+template <int MODE>
+int launch_mode(const StageParams& prm, cudaStream_t st) {
+    const int64_t C = prm.K_active * prm.S;   // columns updated
+    if (C <= 0) return DGM_OK;
+    const unsigned grid = unsigned((C + 31) / 32);
+    StageParams q = prm;
+    q.dt_f = float(prm.dt);
+    return (!q.force_index64 && fits_32bit(q)) ? launch_lf_ix<MODE, uint32_t>(q, grid, st)
+                                               : launch_lf_ix<MODE, int64_t>(q, grid, st);
+}
 #else
 template <typename IX>
 int launch_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
@@ -170,6 +208,13 @@ int launch_mode(const StageParams& prm, cudaStream_t st) {
 #ifdef DGM_ADJ
 int DGM_LAUNCH(const AdjParams& prm, void* stream) {
     return launch_adj(prm, static_cast<cudaStream_t>(stream));
+}
+#elif defined(DGM_LF)
+int DGM_LAUNCH(const StageParams& prm, void* stream) {
+    return launch_mode<MODE_LF_E>(prm, static_cast<cudaStream_t>(stream));
+}
+int DGM_LAUNCH2(const StageParams& prm, void* stream) {
+    return launch_mode<MODE_LF_H>(prm, static_cast<cudaStream_t>(stream));
 }
 #else
 int DGM_LAUNCH(const StageParams& prm, void* stream) {

@@ -1,0 +1,7 @@
+// Leapfrog half steps of plans with receivers: degree 1, float fields.
+#define DGM_P 1
+#define DGM_REAL float
+#define DGM_LF 1
+#define DGM_LAUNCH launch_p1_f32_lfe
+#define DGM_LAUNCH2 launch_p1_f32_lfh
+#include "dgm_kern_impl.cuh"

@@ -545,7 +545,9 @@ __device__ __forceinline__ void flux_face(int m0, int m1, int c, R* trO, const R
 
 // Right-hand side rows [LO, HI) of component `comp` (before the mass inverse):
 // volume curl of the other field plus the lift of the pulled-back fluxes.
-template <int P, typename R, int TE, int LO, int HI>
+// FC: components held per face and field pair, 6 (us: both fields) or 3 (us: the
+// other field alone, trO: this field's fluxes alone).
+template <int P, typename R, int TE, int LO, int HI, int FC = 6>
 __device__ __forceinline__ void rhs_rows(int comp, int c, const R* us, const R* trO, R sgn,
                                          R (&acc)[nmodes(P)]) {
     constexpr int N = nmodes(P);
@@ -555,12 +557,12 @@ __device__ __forceinline__ void rhs_rows(int comp, int c, const R* us, const R* 
     // curl_x = d_y v_z - d_z v_y, curl_y = d_z v_x - d_x v_z, curl_z = d_x v_y - d_y v_x,
     // of H for the E equation (+s_T) and of E for the H equation (-s_T)
     const int j = comp % 3;
-    const int srcf = comp < 3 ? 3 : 0;
+    const int srcf = FC == 6 && comp < 3 ? 3 : 0;
     const R sg = comp < 3 ? sgn : -sgn;
     // The pulled-back flux of face a + 1 (normal -e_a) has no component a, so
     // component j lifts the fluxes of the three other faces only.
     const R* base = us + c;
-    const R* g = trO + comp * NF * TE + c;    // face f of this component: g + f * 6 * NF * TE
+    const R* g = trO + (FC == 6 ? comp : j) * NF * TE + c;    // face f of this component: g + f * FC * NF * TE
     switch (j) {
         case 0:
             DerivOp<P, 1>::template apply<R, LO, HI>(base + (srcf + 2) * N * TE, TE, R(1), acc);
@@ -579,22 +581,22 @@ __device__ __forceinline__ void rhs_rows(int comp, int c, const R* us, const R* 
     for (int l = LO; l < HI; ++l) acc[l] *= sg;
     // one copy of each lift, skipped by a branch that is uniform over the
     // group (lifts inside the cases above would triple the code of this phase)
-    LiftOp<P, 0>::template apply<R, LO, HI>(g + 0 * 6 * NF * TE, TE, acc);
-    if (j != 0) LiftOp<P, 1>::template apply<R, LO, HI>(g + 1 * 6 * NF * TE, TE, acc);
-    if (j != 1) LiftOp<P, 2>::template apply<R, LO, HI>(g + 2 * 6 * NF * TE, TE, acc);
-    if (j != 2) LiftOp<P, 3>::template apply<R, LO, HI>(g + 3 * 6 * NF * TE, TE, acc);
+    LiftOp<P, 0>::template apply<R, LO, HI>(g + 0 * FC * NF * TE, TE, acc);
+    if (j != 0) LiftOp<P, 1>::template apply<R, LO, HI>(g + 1 * FC * NF * TE, TE, acc);
+    if (j != 1) LiftOp<P, 2>::template apply<R, LO, HI>(g + 2 * FC * NF * TE, TE, acc);
+    if (j != 2) LiftOp<P, 3>::template apply<R, LO, HI>(g + 3 * FC * NF * TE, TE, acc);
 }
 
-template <int P, typename R, int TE, int NPART>
+template <int P, typename R, int TE, int NPART, int FC = 6>
 __device__ __forceinline__ void rhs_part(int part, int comp, int c, const R* us, const R* trO,
                                          R sgn, R (&acc)[nmodes(P)]) {
     constexpr int N = nmodes(P);
     static_assert(NPART >= 1 && NPART <= 4, "row partition");
     switch (part) {
-        case 0: rhs_rows<P, R, TE, 0, (NPART == 1 ? N : N / NPART)>(comp, c, us, trO, sgn, acc); break;
-        case 1: rhs_rows<P, R, TE, N / NPART, (NPART == 2 ? N : 2 * N / NPART)>(comp, c, us, trO, sgn, acc); break;
-        case 2: rhs_rows<P, R, TE, 2 * N / NPART, (NPART == 3 ? N : 3 * N / NPART)>(comp, c, us, trO, sgn, acc); break;
-        default: rhs_rows<P, R, TE, 3 * N / NPART, N>(comp, c, us, trO, sgn, acc); break;
+        case 0: rhs_rows<P, R, TE, 0, (NPART == 1 ? N : N / NPART), FC>(comp, c, us, trO, sgn, acc); break;
+        case 1: rhs_rows<P, R, TE, N / NPART, (NPART == 2 ? N : 2 * N / NPART), FC>(comp, c, us, trO, sgn, acc); break;
+        case 2: rhs_rows<P, R, TE, 2 * N / NPART, (NPART == 3 ? N : 3 * N / NPART), FC>(comp, c, us, trO, sgn, acc); break;
+        default: rhs_rows<P, R, TE, 3 * N / NPART, N, FC>(comp, c, us, trO, sgn, acc); break;
     }
 }
 
