@@ -13,6 +13,7 @@
 #include <string>
 #include <vector>
 
+#include "dgm_bulk.cuh"
 #include "dgm_internal.h"
 #include "dgm_ops_gen.cuh"
 #include "dgmax.h"
@@ -751,7 +752,7 @@ static void sip_stage(const dgm_plan* P, StageParams& prm) {
 }  // extern "C"
 
 // Incident plane-wave table (FP64, in the geometry buffer):
-//   [0, INC_HDR)  header: f0, bw, t0, nq, n_faces, 0, 0, 0
+//   [0, INC_HDR)  header: f0, bw, t0, nq, n_faces, 1 / (2 pi bw), 0, 0
 //   then the face rule: (s_q, t_q) (2 nq values), W[m][q] = w_q psi_m(s_q, t_q)
 //       (NF nq values; the parametrisation of the trace operators)
 //   then per incident face i (INC_FACE values): A^T E0 (the polarisation's
@@ -763,7 +764,9 @@ static void sip_stage(const dgm_plan* P, StageParams& prm) {
 // One warp per face: the lanes take the rule's points, then reduce per mode.
 // The delay x = t - t0 - tau_q is formed in FP64 (t may be large against the
 // pulse width); the pulse and the sums run in the plan's precision (an FP32
-// plan rounds the jump terms to FP32 anyway).
+// plan rounds the jump terms to FP32 anyway).  Inside a call of several steps
+// the launch overlaps the stage before it, whose slots it overwrites only after
+// that stage has ended (it took 5 of a step's 49 us on a 9^3 grid at p = 2).
 struct IncTimes {
     double t[INC_SLOTS];
 };
@@ -775,9 +778,12 @@ __global__ void incident_eval(const double* __restrict__ tab, int NF, IncTimes t
     const int lane = threadIdx.x & 31;
     const int64_t i = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int64_t nf = int64_t(tab[4]);
-    if (i >= nf) return;
+    if (i >= nf) {
+        bulk::wait_previous_launch();
+        return;
+    }
     const double twopi = 6.283185307179586476925286766559;
-    const R f0 = R(tab[0]), sg = R(1.0 / (twopi * tab[1]));
+    const R f0 = R(tab[0]), sg = R(tab[5]);
     const double t0 = tab[2];
     const int nq = int(tab[3]);
     const double* pts = tab + INC_HDR;
@@ -793,6 +799,7 @@ __global__ void incident_eval(const double* __restrict__ tab, int NF, IncTimes t
             g[k] = cos(R(twopi) * f0 * x) * exp(-x * x / (R(2) * sg * sg));
         }
     }
+    bulk::wait_previous_launch();
     for (int m = 0; m < NF; ++m) {
         R acc = R(0);
 #pragma unroll
@@ -808,19 +815,18 @@ __global__ void incident_eval(const double* __restrict__ tab, int NF, IncTimes t
 
 // The incident jump terms at n (<= INC_SLOTS) times, into slots 0 .. n-1: one
 // launch for the five stages of an LSRK step.
-static int incident_eval_times(dgm_plan* P, const double* t, int n, cudaStream_t st) {
+static int incident_eval_times(dgm_plan* P, const double* t, int n, cudaStream_t st, bool pdl = false) {
     IncTimes ts{};
     for (int k = 0; k < n; ++k) ts.t[k] = t[k];
     const double* tab = reinterpret_cast<const double*>(P->geom + P->off_inc);
     const dim3 grid(unsigned((P->n_inc + 3) / 4), unsigned(n));
     const int64_t slot = int64_t(P->n_inc) * P->NF * 3;   // reals per slot in use
-    if (P->kt->real_size == 8)
-        incident_eval<double><<<grid, 128, 0, st>>>(tab, P->NF, ts, slot,
-                                                     reinterpret_cast<double*>(P->geom + P->off_incv));
-    else
-        incident_eval<float><<<grid, 128, 0, st>>>(tab, P->NF, ts, slot,
-                                                    reinterpret_cast<float*>(P->geom + P->off_incv));
-    return cudaGetLastError() == cudaSuccess ? DGM_OK : DGM_ECUDA;
+    unsigned char* out = P->geom + P->off_incv;
+    const cudaError_t e =
+        P->kt->real_size == 8
+            ? launch_ex(incident_eval<double>, grid, 128, 0, st, pdl, 1, tab, P->NF, ts, slot, reinterpret_cast<double*>(out))
+            : launch_ex(incident_eval<float>, grid, 128, 0, st, pdl, 1, tab, P->NF, ts, slot, reinterpret_cast<float*>(out));
+    return e == cudaSuccess ? DGM_OK : DGM_ECUDA;
 }
 
 // A stage launch.  With incident faces the kernel reads the jump terms of
@@ -1023,7 +1029,7 @@ int dgm_advance(dgm_plan* P, int64_t n_steps, double t0) {
             if (P->n_inc > 0) {   // the step's five stage times in one launch
                 double ts[5];
                 for (int k = 0; k < 5; ++k) ts[k] = t + LSRK_C[k] * dt;
-                if (int rc = incident_eval_times(P, ts, 5, P->stream)) return fail(rc, "incident launch failed");
+                if (int rc = incident_eval_times(P, ts, 5, P->stream, n > 0)) return fail(rc, "incident launch failed");
             }
             for (int k = 0; k < 5; ++k) {
                 prm.u = P->fields[P->cur];
@@ -1036,6 +1042,7 @@ int dgm_advance(dgm_plan* P, int64_t n_steps, double t0) {
                 prm.a = LSRK_A[k];
                 prm.b = LSRK_B[k];
                 sip_stage(P, prm);
+                prm.pdl = n > 0 || k > 0;   // (behind another launch of this call)
                 int rc = launch_stage(P, prm, MODE_LSRK, P->stream, k);
                 if (rc) return fail(rc, "stage kernel launch failed");
                 P->cur = 1 - P->cur;
@@ -1046,9 +1053,11 @@ int dgm_advance(dgm_plan* P, int64_t n_steps, double t0) {
             prm.aux = P->aux[P->cur];   // PML auxiliaries, updated in place
             prm.aux_out = P->aux[P->cur];
             prm.t = t + 0.5 * dt;
+            prm.pdl = n > 0;
             int rc = launch_stage(P, prm, MODE_LF_E, P->stream);
             if (rc) return fail(rc, "stage kernel launch failed");
             prm.t = t + dt;
+            prm.pdl = 1;
             rc = launch_stage(P, prm, MODE_LF_H, P->stream);
             if (rc) return fail(rc, "stage kernel launch failed");
         }
@@ -1126,6 +1135,7 @@ int dgm_set_incident(dgm_plan* P, int64_t n, const int64_t* faces, const dgm_inc
         tab[2] = w->t0;
         tab[3] = nq;
         tab[4] = double(n);
+        tab[5] = 1.0 / (6.283185307179586476925286766559 * w->bw);
         for (int q = 0; q < nq; ++q) {
             tab[INC_HDR + 2 * q] = pts[2 * q];
             tab[INC_HDR + 2 * q + 1] = pts[2 * q + 1];

@@ -551,6 +551,17 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
     const R* u = static_cast<const R*>(prm.u);   // may alias u_out (leapfrog)
     auto coef = [&](double d, float f) { return sizeof(R) == 4 ? R(f) : R(d); };
 
+    // What no earlier launch of the call writes: the face's code and constants
+    const int f = NG == 4 ? grp : grp >> 1;
+    const int half = NG == 4 ? 0 : grp & 1;      // field (leapfrog: tangent) of this thread when NG = 8
+    auto table = [&](int row) -> R {
+        const R* b = static_cast<const R*>(prm.fct) + IX(row) * K;
+        return b[id.e];
+    };
+    const int32_t code = active ? prm.nbr[IX(f) * K + id.e] : -1;
+    const R cE = table(f * TG_FACE + TG_CE), cH = table(f * TG_FACE + TG_CH);
+    bulk::wait_previous_launch();
+
     // The tile: one bulk tensor copy of its rows where the plan has a
     // map of u (aligned rows), issued first and waited for by thread 0; columns
     // past the end arrive as zeros.  Otherwise every thread loads its rows.
@@ -561,11 +572,7 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
         bulk::arrive_expect_tx(bar, uint32_t(sizeof(R)) * TE * ROWS);
         bulk::load_3d(us, static_cast<const char*>(prm.tmaps) + prm.tm_u * TMAP_BYTES, int(x0), 0, 0, bar);
     }
-
     // ---- phase A: jumps and fluxes of one face -----------------------------------
-    const int f = NG == 4 ? grp : grp >> 1;
-    const int half = NG == 4 ? 0 : grp & 1;      // field (leapfrog: tangent) of this thread when NG = 8
-    const int32_t code = active ? prm.nbr[IX(f) * K + id.e] : -1;
     const bool bad = code >= 0 && IX(code >> 2) >= K;
     if (bad) atomicOr(prm.status, int32_t(ST_BAD_NEIGHBOUR));
     const bool has = code >= 0 && !bad;
@@ -597,11 +604,6 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
         }
     };
     gather(q0);
-    auto table = [&](int row) -> R {
-        const R* b = static_cast<const R*>(prm.fct) + IX(row) * K;
-        return b[id.e];
-    };
-    const R cE = table(f * TG_FACE + TG_CE), cH = table(f * TG_FACE + TG_CH);
     if (bulk) {
         bool ok = true;
         if (threadIdx.x == 0) ok = tc::mbar_wait(bar, 0, 500000000ull);

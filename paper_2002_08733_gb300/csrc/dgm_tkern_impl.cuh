@@ -65,8 +65,7 @@ int launch_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
             return DGM_ECUDA;
         configured = true;
     }
-    k<<<grid, Sh::TE * Sh::NG, smem, st>>>(q);
-    return cudaGetLastError() == cudaSuccess ? DGM_OK : DGM_ECUDA;
+    return launch_ex(k, grid, Sh::TE * Sh::NG, smem, st, q.pdl != 0, 1, q) == cudaSuccess ? DGM_OK : DGM_ECUDA;
 }
 
 // true when every index the kernel forms for this plan is below 2^32: field
