@@ -192,6 +192,7 @@ template <int P, typename R, bool PML>
 __host__ __device__ constexpr bool tang_balance() { return sizeof(R) == 4 && !PML && (P == 3 || P == 4); }
 template <int P, typename R, bool PML>
 __host__ __device__ constexpr int tang_split(int np, int k) {
+    if (np > 4) return k * nmodes(P) / np;
     if (np == 2 && tang_balance<P, R, PML>() && P == 3) return k == 0 ? 0 : k == 1 ? 13 : nmodes(P);
     return row_split(P, np, k);
 }
@@ -480,25 +481,14 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
     }
 }
 
-template <int P, int PO, int NF, typename R, int TE, int MODE, typename IX, bool PML, int NPART>
+template <int P, int PO, int NF, typename R, int TE, int MODE, typename IX, bool PML, int NPART, int K0 = 0>
 __device__ __forceinline__ void tang_parts(const StageParams& prm, int F, int part, const R* us, const R* gs,
                                            const Column<IX>& id, int r0, int ro) {
-    static_assert(NPART == 2 || NPART == 4, "row parts");
-#define DGM_ROWS(K_)                                                                                       \
-    tang_rows<P, PO, NF, R, TE, MODE, IX, PML, tang_split<P, R, PML>(NPART, K_),                           \
-              tang_split<P, R, PML>(NPART, K_ + 1)>(prm, F, us, gs, id, r0, ro)
-    if constexpr (NPART == 2) {
-        if (part == 0) DGM_ROWS(0);
-        else DGM_ROWS(1);
-    } else {
-        switch (part) {
-            case 0: DGM_ROWS(0); break;
-            case 1: DGM_ROWS(1); break;
-            case 2: DGM_ROWS(2); break;
-            default: DGM_ROWS(3); break;
-        }
-    }
-#undef DGM_ROWS
+    if (part == K0)
+        tang_rows<P, PO, NF, R, TE, MODE, IX, PML, tang_split<P, R, PML>(NPART, K0),
+                  tang_split<P, R, PML>(NPART, K0 + 1)>(prm, F, us, gs, id, r0, ro);
+    else if constexpr (K0 + 1 < NPART)
+        tang_parts<P, PO, NF, R, TE, MODE, IX, PML, NPART, K0 + 1>(prm, F, part, us, gs, id, r0, ro);
 }
 
 // one code path for both fields where their degrees are equal
@@ -514,14 +504,31 @@ __device__ __forceinline__ void tang_part(const StageParams& prm, int F, int par
     }
 }
 
+constexpr int CLW = 4;   // warps of a cluster's CTA
+
+// barrier of all threads of the cluster; shared-memory writes before it, remote
+// ones too, are visible after it
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // IX: type of the element/column/row index arithmetic (uint32_t when every
 // index of the plan fits, else int64_t).  MINB: resident CTAs per SM asked of
 // the register allocator.  NG = 4: thread groups = faces (both fields), then
 // (field, half of the rows); NG = 8: (face, field), then (field, quarter of the
 // rows), the two fields of a face in the two halves of a warp (TE = 16) or in
 // two neighbouring warps (TE = 32).
-template <int P, typename R, int TE, int NG, int MODE, typename IX, bool SIP, bool PML, bool MX, int MINB>
-__global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams prm) {
+// CL = 8 (FP64 on small meshes): a tile of 32 columns takes the eight CTAs of a
+// cluster, CTA = the thread group of the face items, four warps each.  An SM's FP64
+// pipes work through a warp's instruction in 64 cycles, so that a launch lasts as
+// long as its longest warp however few tiles there are: here a warp has a quarter
+// of an item's face modes and a sixteenth of a field's rows.  Face values are
+// written into every CTA's shared memory, and cluster barriers take the place of
+// the CTA's.
+template <int P, typename R, int TE, int NG, int MODE, typename IX, bool SIP, bool PML, bool MX, int MINB, int CL = 1>
+__global__ void __launch_bounds__(CL > 1 ? TE * CLW : TE * NG, MINB) tang_kernel(const StageParams prm) {
+    static_assert(CL == 1 || (CL == 8 && NG == CL && TE == 32 && sizeof(R) == 8 && !SIP && !MX), "cluster shape");
     static_assert((TE == 32 && (NG == 4 || NG == 8)) || (TE == 16 && NG == 8), "tile shape");
     static_assert(!(SIP || MX) || MODE == MODE_LSRK || MODE == MODE_RHS, "interior penalty and mixed-order modes");
     static_assert(!(MX && (SIP || PML)), "mixed orders: no penalty, no PML");
@@ -534,10 +541,13 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
     uint64_t* bar = reinterpret_cast<uint64_t*>(gs + 16 * NF * TE);
 
     const int c = threadIdx.x % TE;
-    const int grp = threadIdx.x / TE;
+    const int grp = CL > 1 ? int(blockIdx.x % CL) : threadIdx.x / TE;   // (CL: the rank in the cluster)
+    const int sub = CL > 1 ? int(threadIdx.x / TE) : 0;                 // (CL: the warp in the CTA)
     const IX K = prm.K;
     const int S = prm.S;
-    const IX x0 = IX(tile_index(prm.tile_groups)) * TE;
+    const IX x0 = IX(CL > 1 ? blockIdx.x / CL : tile_index(prm.tile_groups)) * TE;
+    // no CTA writes into another's shared memory before all of the cluster run
+    if constexpr (CL > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     Column<IX> id;
     id.C = K * S;
     id.col = x0 + c;
@@ -565,7 +575,7 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
     // The tile: one bulk tensor copy of its rows where the plan has a
     // map of u (aligned rows), issued first and waited for by thread 0; columns
     // past the end arrive as zeros.  Otherwise every thread loads its rows.
-    const bool bulk = prm.tm_u >= 0 && (tc::smem_addr(smem_raw) & 127u) == 0;
+    const bool bulk = CL == 1 && prm.tm_u >= 0 && (tc::smem_addr(smem_raw) & 127u) == 0;
     if (bulk && threadIdx.x == 0) {
         static_assert(sizeof(R) * TE * ROWS < (1u << 20), "bytes of an mbarrier phase");
         tc::mbar_init(bar, 1);
@@ -617,6 +627,19 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
             }
             return;
         }
+    } else if constexpr (CL > 1) {
+        // every CTA of the cluster holds the tile; asynchronous copies, all in flight
+        if (active) {
+#pragma unroll 4
+            for (int q = sub; q < ROWS; q += CLW)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;"
+                             :: "r"(tc::smem_addr(us + q * TE + c)), "l"(u + (IX(q) * C + id.col)) : "memory");
+            asm volatile("cp.async.wait_all;" ::: "memory");
+        } else {
+            for (int q = sub; q < ROWS; q += CLW) us[q * TE + c] = R(0);
+        }
+        __syncthreads();
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     } else {
         constexpr int UR = (ROWS + NG - 1) / NG, BATCH = UR < 16 ? UR : 16;
 #pragma unroll 1
@@ -636,9 +659,29 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
         __syncthreads();
     }
     R* gf = gs + f * 4 * NF * TE + c;   // this face's rows: [field][tangent][NF]
+    // a face value into the shared memory of the cluster's ranks lo .. lo + n - 1
+    const uint32_t sbase = tc::smem_addr(smem_raw);
+    uint32_t rbase[CL];
+    if constexpr (CL > 1) {
+#pragma unroll
+        for (int r = 0; r < CL; ++r) asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rbase[r]) : "r"(sbase), "r"(r));
+    }
+    auto put = [&](R* o, R v, bool pair) {
+        if constexpr (CL > 1) {
+            const uint32_t off = tc::smem_addr(o) - sbase;
+#pragma unroll
+            for (int r = 0; r < CL; ++r)
+                if (!pair || r / 2 == f)   // pair: the two ranks of this face
+                    asm volatile("st.shared::cluster.f64 [%0], %1;" :: "r"(rbase[r] + off), "d"(double(v)) : "memory");
+        } else {
+            *o = v;
+        }
+    };
     const bool inc = code <= -2 && prm.inc != nullptr;
     // jump of item q of a field of degree PF: own trace, then the neighbour's
-    auto item = [&](auto deg, int q) {
+    // (CL: modes of quarter `mq` only; the arithmetic of the others falls away)
+    auto item = [&](auto deg, int q, auto mq) {
+        constexpr int part = decltype(mq)::value;
         constexpr int PF = decltype(deg)::value, NP = nmodes(PF), NPF = nfmodes(PF);
         const int fld = q >> 1, i = q & 1;
         const R* v0 = us + row_of(fld, 0) * TE + c;
@@ -668,19 +711,37 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
         const R cc = LF ? (MODE == MODE_LF_E ? cE : cH) * R(i ? 1 : -1) : R(1);
         R* o = gf + (LF ? 2 * (1 - fld) + 1 - i : q) * NF * TE;
 #pragma unroll
-        for (int m = 0; m < NPF; ++m) o[m * TE] = LF ? cc * acc[m] : acc[m];
+        for (int m = 0; m < NPF; ++m) {
+            if (CL > 1 && m * CLW / NPF != part) continue;
+            if constexpr (LF) put(o + m * TE, cc * acc[m], false);
+            else put(o + m * TE, acc[m], true);   // both threads of the face
+        }
     };
 #pragma unroll 1
     for (int k = 0; k < QN; ++k) {
         const int q = q0 + k;
-        if (!MX || (q >> 1) == 0) item(std::integral_constant<int, P>{}, q);
-        else item(std::integral_constant<int, PH>{}, q);
+        auto quarter = [&](auto mq) {
+            if (!MX || (q >> 1) == 0) item(std::integral_constant<int, P>{}, q, mq);
+            else item(std::integral_constant<int, PH>{}, q, mq);
+        };
+        if constexpr (CL > 1) {
+            switch (sub) {
+                case 0: quarter(std::integral_constant<int, 0>{}); break;
+                case 1: quarter(std::integral_constant<int, 1>{}); break;
+                case 2: quarter(std::integral_constant<int, 2>{}); break;
+                default: quarter(std::integral_constant<int, 3>{}); break;
+            }
+        } else {
+            quarter(std::integral_constant<int, 0>{});
+        }
         if (k + 1 < QN) gather(q + 1);
     }
     if constexpr (!LF) {
         // fluxes in place; with NG = 8 the face's two threads split the modes
         // and first wait for each other's jumps
-        if (NG == 8) {
+        if constexpr (CL > 1) {
+            cluster_sync();
+        } else if (NG == 8) {
             if (TE == 16) __syncwarp();
             else asm volatile("bar.sync %0, 64;" :: "r"(1 + f) : "memory");
         }
@@ -718,9 +779,9 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
             }
         }
         // the modes in chunks, so that a chunk's facet values arrive together
-        constexpr int MC = SIP ? (NF + 3) / 4 : 1;
+        constexpr int MC = SIP ? (NF + 3) / 4 : 1, MSTEP = CL > 1 ? CLW : MC;
 #pragma unroll(SIP ? 1 : (P <= 3 ? 10 : 3))
-        for (int mb = m0; mb < m1; mb += MC) {
+        for (int mb = m0 + sub; mb < m1; mb += MSTEP) {
             R hv[SIP ? MC : 1][3], hr[SIP ? MC : 1][3];
             if constexpr (SIP) {
 #pragma unroll
@@ -748,8 +809,8 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
                 R p1 = fmaa(cE, h2, fmaa(e22, e1, ne12 * e2));
                 R p2 = fmaa(ncE, h1, fmaa(e11, e2, ne12 * e1));
                 if (hm) {
-                    o[2 * NF * TE] = fmaa(cH, e2, fmaa(h12, h2, nh22 * h1));
-                    o[3 * NF * TE] = fmaa(ncH, e1, fmaa(h12, h1, nh11 * h2));
+                    put(o + 2 * NF * TE, fmaa(cH, e2, fmaa(h12, h2, nh22 * h1)), false);
+                    put(o + 3 * NF * TE, fmaa(ncH, e1, fmaa(h12, h1, nh11 * h2)), false);
                 }
                 if constexpr (SIP) {
                     // both sides: gamma += m_f x (A^T h_s); owner: dh_s/dt =
@@ -773,18 +834,27 @@ __global__ void __launch_bounds__(TE * NG, MINB) tang_kernel(const StageParams p
                         }
                     }
                 }
-                o[0] = p1;
-                o[NF * TE] = p2;
+                put(o, p1, false);
+                put(o + NF * TE, p2, false);
             }
         }
     }
-    __syncthreads();
+    if constexpr (CL > 1) cluster_sync();
+    else __syncthreads();
 
     // ---- phase B: curl, lift, mass block, update ----------------------------------
     if constexpr (LF) {
         // one field; NG = 8 would need eight row parts, its second half idles
         constexpr int F = MODE == MODE_LF_E ? 0 : 1;
-        if (grp < 4) tang_part<P, R, TE, MODE, IX, PML, MX, 4>(prm, F, grp, us + c, gs + c, id);
+        if constexpr (CL > 1) {
+            constexpr int NPB = N < 16 ? N : 16;
+            if (const int part = sub * CL + grp; part < NPB)
+                tang_part<P, R, TE, MODE, IX, PML, MX, NPB>(prm, F, part, us + c, gs + c, id);
+        } else if (grp < 4) tang_part<P, R, TE, MODE, IX, PML, MX, 4>(prm, F, grp, us + c, gs + c, id);
+    } else if constexpr (CL > 1) {
+        constexpr int NPB = N < 16 ? N : 16;
+        if (const int part = sub * 4 + (grp >> 1); part < NPB)
+            tang_part<P, R, TE, MODE, IX, PML, MX, NPB>(prm, grp & 1, part, us + c, gs + c, id);
     } else if constexpr (NG == 4) {
         constexpr bool BAL = tang_balance<P, R, PML>() && !MX;
         const int F = BAL ? grp >> 1 : grp & 1;

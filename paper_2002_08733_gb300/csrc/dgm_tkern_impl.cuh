@@ -53,6 +53,10 @@ constexpr bool kSIP = true;
 constexpr bool kSIP = false;
 #endif
 
+// Most tiles (of 32 columns) for which the cluster form is taken: two of its CTAs per
+// SM (8 x 38 = 2 x 152; three would wait for one another's FP64 pipes).
+constexpr unsigned kClusterTiles = 38;
+
 template <int MODE, typename IX, bool SIP, bool PML>
 int launch_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
     using Sh = Shape<MODE, SIP, PML>;
@@ -77,6 +81,24 @@ bool fits_32bit(const StageParams& p) {
     const uint64_t N = uint64_t(nmodes(kP)), NF = uint64_t(nfmodes(kP));
     return 6 * N * C < lim && 6 * N * uint64_t(p.npml) * uint64_t(p.S) < lim &&
            uint64_t(G_COUNT) * K < lim && uint64_t(TG_ROWS) * K < lim && 12 * NF * K < lim;
+}
+
+// FP64 meshes of few tiles: a cluster of eight CTAs per tile (see tang_kernel).
+// With a tile per CTA the launch takes as long as one SM's FP64 pipe needs for one
+// tile, however few there are; a cluster spreads a tile over eight SMs.  us per launch
+// of 12 tiles, one CTA | cluster: leapfrog p = 2 15.1 | 7.0; with clusters of
+// one-warp CTAs p = 3 37 | 23, LSRK4 p = 4 140 | 90, and from 65 tiles on no gain.
+template <int MODE>
+int launch_cluster(const StageParams& q, unsigned tiles, cudaStream_t st) {
+    constexpr size_t smem = tang_smem_bytes<kP, Real, 32, false>();
+    static bool configured = false;
+    auto k = tang_kernel<kP, Real, 32, 8, MODE, uint32_t, false, true, false, 1, 8>;
+    if (!configured) {
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
+            return DGM_ECUDA;
+        configured = true;
+    }
+    return launch_ex(k, 8 * tiles, 32 * CLW, smem, st, q.pdl != 0, 8, q) == cudaSuccess ? DGM_OK : DGM_ECUDA;
 }
 
 template <int MODE>
@@ -107,6 +129,9 @@ int launch_mode(const StageParams& prm, cudaStream_t st) {
         } else {
             return DGM_EUNSUP;
         }
+    }
+    if constexpr (sizeof(Real) == 8 && !kMX && MODE != MODE_RHS) {
+        if (i32 && grid <= kClusterTiles) return launch_cluster<MODE>(q, grid, st);
     }
     // (64-bit indices: the PML instantiation serves plans without a layer too)
     if (!i32) return launch_ix<MODE, int64_t, false, !kMX>(q, grid, st);

@@ -30,12 +30,12 @@ def D():
     return dgmax
 
 
-def _run(D, n, p, integrator, flux, S, pml, receivers, steps, index64=False):
+def _run(D, n, p, integrator, flux, S, pml, receivers, steps, index64=False, prec="fp32"):
     xyz, tets = W.kuhn_mesh(n, (-1, -1, -1), (1, 1, 1), jitter=0.1, seed=200 + n)
     K = len(tets)
     eps = W.lognormal_material(K, 1.5, 0.2, 201)
     mu = W.lognormal_material(K, 1.0, 0.1, 202)
-    g = D.Solver(xyz, tets, eps, mu, p, "fp32", flux, integrator, W.stable_dt(2.0 / n, p) / 2, S=S,
+    g = D.Solver(xyz, tets, eps, mu, p, prec, flux, integrator, W.stable_dt(2.0 / n, p) / 2, S=S,
                  pml=PML if pml else None, max_receivers=1)
     g.set_sources([W.dipole((0.11, -0.07, 0.05), 2.0, 0.2)] + [None] * (S - 1))
     if receivers:
@@ -91,3 +91,16 @@ def test_leapfrog_with_receivers_matches_oracle(D, p, n, S):
     o = build(xyz, tets, p, eps, 1.0, "central", S=S)
     ref = o.unpack(o.leapfrog(o.pack(u), 0.0, dt, 3))[0]
     assert rel_err(g.state(), ref) < TOL
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+@pytest.mark.parametrize("n,S,pml", [(1, 1, False), (2, 3, True), (5, 1, True), (6, 1, False)])
+@pytest.mark.parametrize("integrator,flux", [("leapfrog", "central"), ("lsrk4", "upwind")])
+def test_fp64_cluster_agrees_with_one_cta_per_tile(D, p, n, S, pml, integrator, flux):
+    """FP64 plans of at most 38 tiles run a cluster of CTAs per tile (n = 1, 2, 5: 1, 5 and
+    24 tiles; n = 6: 41, one CTA per tile); 64-bit indices always one CTA.  The same sums of
+    a few hundred terms: 1e-13 of the max-norm covers their rounding over three steps."""
+    a, aa = _run(D, n, p, integrator, flux, S, pml, False, 3, prec="fp64")
+    b, ba = _run(D, n, p, integrator, flux, S, pml, False, 3, index64=True, prec="fp64")
+    assert rel_err(a, b) < 1e-13
+    assert not pml or rel_err(aa, ba) < 1e-13
