@@ -1,7 +1,7 @@
 // Dispatch tables over the per-(degree, precision, mode) kernel modules.
 //
 // tang_kernel (dgm_tang.cuh) is the default; FP32 LSRK variants for the
-// autotuner: 0 = the shape measured best, 1 = 32 columns x 8 threads per column
+// autotuner: 0 = the shape measured best (by the number of tiles, see few_tiles), 1 = 32 columns x 8 threads per column
 // (p >= 4: x 4), 2 = 16 columns x 8, p >= 4: 3 = 32 x 8 with more registers; up to
 // p = 3 (where 64 columns of pairs fit in shared memory) 3 = paired kernel with
 // packed FP32x2 arithmetic, 4 = paired kernel with scalar arithmetic; at p = 2, 3
@@ -136,6 +136,17 @@ int launch_t_m4_f64_rhs(const StageParams&, void*);
 
 namespace {
 
+// No more tiles of 32 columns than SMs: a CTA has its SM to itself, and eight
+// threads per column fill it better than four, which win once several CTAs share
+// it.  us per FP32 LSRK4 stage, four | eight threads: 137 tiles p = 1 3.99 | 3.28,
+// p = 2 5.10 | 4.71 (PML 9.05 | 7.35), p = 3 9.26 | 7.86, p = 4 19.7 | 15.3; 324
+// tiles p = 1 4.06 | 4.24, p = 2 5.40 | 5.51, p = 4 19.0 | 23.9.  (The penalty and
+// p = 5 always run eight.)
+bool few_tiles(const StageParams& prm) {
+    constexpr int64_t kSMs = 152;
+    return prm.hs == nullptr && (prm.K_active * prm.S + 31) / 32 <= kSMs;
+}
+
 int launch_p1_f32(const StageParams& prm, int mode, void* st) {
     const bool rec = prm.recorded != 0;
     switch (mode) {
@@ -146,7 +157,10 @@ int launch_p1_f32(const StageParams& prm, int mode, void* st) {
                 case 2: return rec ? launch_p1_f32_lsrk_v2(prm, st) : launch_t_p1_f32_lsrk_v2(prm, st);
                 case 3: return launch_p1_f32_lsrk_v3(prm, st);
                 case 4: return launch_p1_f32_lsrk_v4(prm, st);
-                default: return rec ? launch_p1_f32_lsrk(prm, st) : launch_t_p1_f32_lsrk(prm, st);
+                default:
+                    return rec              ? launch_p1_f32_lsrk(prm, st)
+                           : few_tiles(prm) ? launch_t_p1_f32_lsrk_v1(prm, st)
+                                            : launch_t_p1_f32_lsrk(prm, st);
             }
         case MODE_LF_E: return rec ? launch_p1_f32_lfe(prm, st) : launch_t_p1_f32_lf(prm, st);
         case MODE_LF_H: return rec ? launch_p1_f32_lfh(prm, st) : launch_t_p1_f32_lfh(prm, st);
@@ -177,7 +191,10 @@ int launch_p2_f32(const StageParams& prm, int mode, void* st) {
                 case 3: return launch_p2_f32_lsrk_v3(prm, st);
                 case 4: return launch_p2_f32_lsrk_v4(prm, st);
                 case 5: return launch_p2_f32_lsrk_v5(prm, st);
-                default: return rec ? launch_p2_f32_lsrk(prm, st) : launch_t_p2_f32_lsrk(prm, st);
+                default:
+                    return rec              ? launch_p2_f32_lsrk(prm, st)
+                           : few_tiles(prm) ? launch_t_p2_f32_lsrk_v1(prm, st)
+                                            : launch_t_p2_f32_lsrk(prm, st);
             }
         case MODE_LF_E: return rec ? launch_p2_f32_lfe(prm, st) : launch_t_p2_f32_lf(prm, st);
         case MODE_LF_H: return rec ? launch_p2_f32_lfh(prm, st) : launch_t_p2_f32_lfh(prm, st);
@@ -208,7 +225,10 @@ int launch_p3_f32(const StageParams& prm, int mode, void* st) {
                 case 3: return launch_p3_f32_lsrk_v3(prm, st);
                 case 4: return launch_p3_f32_lsrk_v4(prm, st);
                 case 5: return launch_p3_f32_lsrk_v5(prm, st);
-                default: return rec ? launch_p3_f32_lsrk(prm, st) : launch_t_p3_f32_lsrk(prm, st);
+                default:
+                    return rec              ? launch_p3_f32_lsrk(prm, st)
+                           : few_tiles(prm) ? launch_t_p3_f32_lsrk_v1(prm, st)
+                                            : launch_t_p3_f32_lsrk(prm, st);
             }
         case MODE_LF_E: return rec ? launch_p3_f32_lfe(prm, st) : launch_t_p3_f32_lf(prm, st);
         case MODE_LF_H: return rec ? launch_p3_f32_lfh(prm, st) : launch_t_p3_f32_lfh(prm, st);
@@ -237,7 +257,10 @@ int launch_p4_f32(const StageParams& prm, int mode, void* st) {
                 case 1: return rec ? launch_p4_f32_lsrk_v1(prm, st) : launch_t_p4_f32_lsrk_v1(prm, st);
                 case 2: return rec ? launch_p4_f32_lsrk_v2(prm, st) : launch_t_p4_f32_lsrk_v2(prm, st);
                 case 3: return rec ? launch_p4_f32_lsrk_v3(prm, st) : launch_t_p4_f32_lsrk_v3(prm, st);
-                default: return rec ? launch_p4_f32_lsrk(prm, st) : launch_t_p4_f32_lsrk(prm, st);
+                default:
+                    return rec              ? launch_p4_f32_lsrk(prm, st)
+                           : few_tiles(prm) ? launch_t_p4_f32_lsrk_v3(prm, st)
+                                            : launch_t_p4_f32_lsrk(prm, st);
             }
         case MODE_LF_E: return rec ? launch_p4_f32_lfe(prm, st) : launch_t_p4_f32_lf(prm, st);
         case MODE_LF_H: return rec ? launch_p4_f32_lfh(prm, st) : launch_t_p4_f32_lfh(prm, st);
