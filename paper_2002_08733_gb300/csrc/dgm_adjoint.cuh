@@ -134,10 +134,12 @@ __device__ __host__ constexpr size_t adjoint_smem_bytes() {
     constexpr int NPART = NG >= 24 ? 4 : (NG >= 12 ? 2 : 1);
     constexpr int CH = NG >= 12 ? NG / 4 : 1;
     return sizeof(R) * size_t(TE) * (12 * nmodes(P) + 48 * nfmodes(P) + 4 * FGA + EG) +
-           sizeof(double) * size_t(TE) * (4 * CH + 2 * 6 * NPART);
+           sizeof(double) * size_t(TE) * (4 * CH + 6 * NPART);
 }
 
 // IX: index type (uint32_t when every index of the plan fits, else int64_t)
+// The stage also forms the next stage's residual (in another buffer: neighbours still
+// read this one), which as a pass of its own read both vectors again.
 template <int P, typename R, int TE, int NT, typename IX = int64_t>
 __global__ void __launch_bounds__(NT, sizeof(R) == 4 && P <= 3 ? 2 : 1) adjoint_kernel(const AdjParams prm) {
     constexpr int N = nmodes(P);
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 && P <= 3 ? 2 : 1) adjoint_
     R* fg = trN + 24 * NF * TE;                  // [4][FGA][TE]
     R* eg = fg + 4 * FGA * TE;                   // [EG][TE]
     double* zs = reinterpret_cast<double*>(eg + EG * TE);   // [4 CH][TE]   dJ/dZ partials
-    double* gp = zs + 4 * CH * TE;                           // [2][6 NPART][TE] gradient partials
+    double* gp = zs + 4 * CH * TE;                           // [6 NPART][TE] gradient partials
 
     const int c = threadIdx.x % TE;
     const int grp = threadIdx.x / TE;
@@ -245,8 +247,6 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 && P <= 3 ? 2 : 1) adjoint_
             const int k = lg + i * LG;
             if (k < EG) eg[k * TE + c] = tmpe[i];
         }
-        for (int i = lg; i < 4 * CH; i += LG) zs[i * TE + c] = 0.0;
-        for (int i = lg; i < 2 * 6 * NPART; i += LG) gp[i * TE + c] = 0.0;
     }
     if (FACE_GROUPS == 0) {
         for (int f = grp; f < 4; f += NG) face_consts(f);
@@ -339,8 +339,27 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 && P <= 3 ? 2 : 1) adjoint_
         const R zp = bnd ? zm : sqrt(d[FA_MUN * TE] / d[FA_EPSN * TE]);
         const R D = (zm + zp) * (zm + zp);
         const R* jp = static_cast<const R*>(prm.jumps);
+        // the jumps of a mode are requested while the mode before it is worked on
+        const bool jmp = prm.upwind && active;
+        const int mend = (ch + 1) * NF / CH;
+        R jE[3] = {0, 0, 0}, jH[3] = {0, 0, 0};
+        auto request_jumps = [&](int m) {
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                jE[r] = jp[IX((f * 6 + r) * NF + m) * C + col];
+                jH[r] = jp[IX((f * 6 + 3 + r) * NF + m) * C + col];
+            }
+        };
+        if (jmp && ch * NF / CH < mend) request_jumps(ch * NF / CH);
         R zacc = R(0);   // partial sums in the kernel's precision, FP64 from phase 6 on
-        for (int m = ch * NF / CH; m < (ch + 1) * NF / CH; ++m) {
+        for (int m = ch * NF / CH; m < mend; ++m) {
+            R dE[3], dH[3];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                dE[r] = jE[r];
+                dH[r] = jH[r];
+            }
+            if (jmp && m + 1 < mend) request_jumps(m + 1);
             R* own = trO + (f * 6 * NF + m) * TE + c;
             const R* nbt = trN + (f * 6 * NF + m) * TE + c;
             R gE[3], gH[3], phiE[3], phiH[3];
@@ -405,13 +424,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 && P <= 3 ? 2 : 1) adjoint_
                 own[k * NF * TE] = zE[k];
                 own[(3 + k) * NF * TE] = zH[k];
             }
-            if (prm.upwind && active) {
-                R dE[3], dH[3];
-#pragma unroll
-                for (int r = 0; r < 3; ++r) {
-                    dE[r] = jp[IX((f * 6 + r) * NF + m) * C + col];
-                    dH[r] = jp[IX((f * 6 + 3 + r) * NF + m) * C + col];
-                }
+            if (jmp) {
                 R nxdE[3], nnxdE[3], nxdH[3], nnxdH[3];
                 cross3(n, dE, nxdE);
                 cross3(n, nxdE, nnxdE);
@@ -504,51 +517,66 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 && P <= 3 ? 2 : 1) adjoint_
         const R* af = static_cast<const R*>(prm.aux);
         const R* raw = static_cast<const R*>(prm.raw);
         const R dt = R(prm.dt);
+        R* lrn = static_cast<R*>(prm.lr_next);
+        R* lran = static_cast<R*>(prm.lr_aux_next);
+        const R an = R(prm.a_next), bn = R(prm.b_next);
         R gmass = R(0), gpml = R(0);   // partial sums in the kernel's precision
         const int lo = part * N / NPART, hi = (part + 1) * N / NPART;
-        // the item's forward right-hand-side and adjoint rows, all requested
-        // before the arithmetic so that their round trips overlap
-        constexpr int RP = (N + NPART - 1) / NPART;
-        R rawv[RP], luv[RP];
+        // the rows in chunks whose loads are all requested before their arithmetic
+        // (row by row, the stores to lu and lu_aux kept the next row's loads behind
+        // them: ten round trips to DRAM one after the other in the layer)
+        constexpr int RP = (N + NPART - 1) / NPART, CR = sizeof(R) == 8 ? 2 : 4;
 #pragma unroll
-        for (int i = 0; i < RP; ++i) {
-            const bool ok = lo + i < hi;
-            const IX gi = IX(comp * N + lo + i) * C + col;
-            rawv[i] = ok ? raw[gi] : R(0);
-            luv[i] = ok ? lu[gi] : R(0);
-        }
+        for (int i0 = 0; i0 < RP; i0 += CR) {
+            R rawv[CR], luv[CR], pv[CR][3], uvv[CR][3], apv[CR], lav[CR];
 #pragma unroll
-        for (int i = 0; i < RP; ++i) {
-            const int l = lo + i;
-            if (l >= hi) break;
-            R w = rh[(comp * N + l) * TE + c];
-            const IX gi = IX(comp * N + l) * C + col;
-            // mass term of the gradient: -(1/mat) rho_c . rhs_c
-            gmass += rs[(comp * N + l) * TE + c] * rawv[i];
-            if (pi >= 0) {
-                const R l0 = us[((fb + 0) * N + l) * TE + c];
-                const R l1 = us[((fb + 1) * N + l) * TE + c];
-                const R l2 = us[((fb + 2) * N + l) * TE + c];
-                const IX ai = IX(fb * N + l) * C2 + acol;
-                const R p0 = lra[ai], p1 = lra[ai + IX(N) * C2], p2 = lra[ai + 2 * IX(N) * C2];
-                w -= etaT[0] * l0 + etaT[1] * l1 + etaT[2] * l2;
-                w += mat * (xiT[0] * p0 + xiT[1] * p1 + xiT[2] * p2);
-                const R lj = j == 0 ? l0 : (j == 1 ? l1 : l2);
-                const R pj = j == 0 ? p0 : (j == 1 ? p1 : p2);
-                const R wa = -lj / mat - (sigT[0] * p0 + sigT[1] * p1 + sigT[2] * p2);
-                const IX aj2 = IX(comp * N + l) * C2 + acol;
-                lua[aj2] += dt * wa;
-                // PML gradient terms: lam_j p_j / mat^2 + lam_aux_j (A^T xi A^-T u)_j
-                const R apj = af[aj2];
-                const R u0 = uf[IX((fb + 0) * N + l) * C + col];
-                const R u1 = uf[IX((fb + 1) * N + l) * C + col];
-                const R u2 = uf[IX((fb + 2) * N + l) * C + col];
-                gpml += lj * apj / (mat * mat) + pj * (xiR[0] * u0 + xiR[1] * u1 + xiR[2] * u2);
+            for (int i = 0; i < CR; ++i) {
+                const int l = lo + i0 + i;
+                const bool ok = i0 + i < RP && l < hi, okp = ok && pi >= 0;
+                const IX gi = IX(comp * N + l) * C + col, aj = IX(comp * N + l) * C2 + acol;
+                rawv[i] = ok ? raw[gi] : R(0);
+                luv[i] = ok ? lu[gi] : R(0);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    pv[i][k] = okp ? lra[IX((fb + k) * N + l) * C2 + acol] : R(0);
+                    uvv[i][k] = okp ? uf[IX((fb + k) * N + l) * C + col] : R(0);
+                }
+                apv[i] = okp ? af[aj] : R(0);
+                lav[i] = okp ? lua[aj] : R(0);
             }
-            lu[gi] = luv[i] + dt * w;
+#pragma unroll
+            for (int i = 0; i < CR; ++i) {
+                const int l = lo + i0 + i;
+                if (i0 + i >= RP || l >= hi) break;
+                R w = rh[(comp * N + l) * TE + c];
+                const IX gi = IX(comp * N + l) * C + col;
+                // mass term of the gradient: -(1/mat) rho_c . rhs_c
+                gmass += rs[(comp * N + l) * TE + c] * rawv[i];
+                if (pi >= 0) {
+                    const R l0 = us[((fb + 0) * N + l) * TE + c];
+                    const R l1 = us[((fb + 1) * N + l) * TE + c];
+                    const R l2 = us[((fb + 2) * N + l) * TE + c];
+                    const R p0 = pv[i][0], p1 = pv[i][1], p2 = pv[i][2];
+                    w -= etaT[0] * l0 + etaT[1] * l1 + etaT[2] * l2;
+                    w += mat * (xiT[0] * p0 + xiT[1] * p1 + xiT[2] * p2);
+                    const R lj = j == 0 ? l0 : (j == 1 ? l1 : l2);
+                    const R pj = j == 0 ? p0 : (j == 1 ? p1 : p2);
+                    const R wa = -lj / mat - (sigT[0] * p0 + sigT[1] * p1 + sigT[2] * p2);
+                    const R la = lav[i] + dt * wa;
+                    const IX aj = IX(comp * N + l) * C2 + acol;
+                    lua[aj] = la;
+                    if (lrn != nullptr) lran[aj] = an == R(0) ? bn * la : fmaa(an, pj, bn * la);
+                    // PML gradient terms: lam_j p_j / mat^2 + lam_aux_j (A^T xi A^-T u)_j
+                    const R apj = apv[i];
+                    const R u0 = uvv[i][0], u1 = uvv[i][1], u2 = uvv[i][2];
+                    gpml += lj * apj / (mat * mat) + pj * (xiR[0] * u0 + xiR[1] * u1 + xiR[2] * u2);
+                }
+                const R ln = luv[i] + dt * w;
+                lu[gi] = ln;
+                if (lrn != nullptr) lrn[gi] = an == R(0) ? bn * ln : fmaa(an, us[(comp * N + l) * TE + c], bn * ln);
+            }
         }
-        const int slot = comp < 3 ? 0 : 1;
-        gp[(slot * 6 * NPART + it) * TE + c] = double(-gmass / mat + gpml);
+        gp[it * TE + c] = double(-gmass / mat + gpml);
     }
     __syncthreads();
 
@@ -558,9 +586,9 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 && P <= 3 ? 2 : 1) adjoint_
         const double Z = sqrt(mu / eps);
         double dz = 0.0, ge = 0.0, gm = 0.0;
         for (int i = 0; i < 4 * CH; ++i) dz += zs[i * TE + c];
-        for (int i = 0; i < 6 * NPART; ++i) {
-            ge += gp[(0 * 6 * NPART + i) * TE + c];
-            gm += gp[(1 * 6 * NPART + i) * TE + c];
+        for (int i = 0; i < 3 * NPART; ++i) {   // items of E's components, then H's
+            ge += gp[i * TE + c];
+            gm += gp[(3 * NPART + i) * TE + c];
         }
         ge += -Z / (2.0 * eps) * dz;
         gm += Z / (2.0 * mu) * dz;

@@ -1651,15 +1651,10 @@ extern "C" void dgm_batch_destroy(dgm_batch* B) { batch_release(B); }
 
 // ---------------------------------------------------------------------------
 // Discrete adjoint driver (dgm_forward_record / dgm_adjoint).
+// lu[(j N + l), e_r S + s] += sum_c W_r[c][j N + l] g[s][r][c], receivers in a fixed
+// order; lr = b lu there (the residual of a step's first adjoint stage)
 template <typename R>
-__global__ void axpby_kernel(R* y, const R* x, double a, double b, int64_t n) {
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-        y[i] = (a == 0.0 ? R(0) : R(a) * y[i]) + R(b) * x[i];
-}
-
-// lu[(j N + l), e_r S + s] += sum_c W_r[c][j N + l] g[s][r][c], receivers in a fixed order
-template <typename R>
-__global__ void inject_receivers(R* lu, const double* rec, int nrec, int64_t K, int S, int N,
+__global__ void inject_receivers(R* lu, R* lr, R b, const double* rec, int nrec, int64_t K, int S, int N,
                                  const double* g) {
     // one thread per (column, component-mode row); receivers in a fixed order,
     // so that receivers sharing an element accumulate without a race
@@ -1672,8 +1667,10 @@ __global__ void inject_receivers(R* lu, const double* rec, int nrec, int64_t K, 
         const double* w = rec + int64_t(r) * (REC_HDR + 9 * N);
         const int64_t col = int64_t(w[0]) * S + s;
         const double* gr = g + (int64_t(s) * nrec + r) * 3;
-        lu[int64_t(jl) * C + col] +=
-            R(w[REC_HDR + jl] * gr[0] + w[REC_HDR + 3 * N + jl] * gr[1] + w[REC_HDR + 6 * N + jl] * gr[2]);
+        const R v = lu[int64_t(jl) * C + col] +
+                    R(w[REC_HDR + jl] * gr[0] + w[REC_HDR + 3 * N + jl] * gr[1] + w[REC_HDR + 6 * N + jl] * gr[2]);
+        lu[int64_t(jl) * C + col] = v;
+        lr[int64_t(jl) * C + col] = b * v;
     }
 }
 
@@ -1694,7 +1691,7 @@ namespace {
 struct AdjLayout {
     size_t fb = 0, ab = 0, sb = 0;   // field, aux, state bytes
     int64_t seg = 0, nseg = 0;
-    size_t ck = 0, sg = 0, tmp = 0, res = 0, lu = 0, lr = 0, raw = 0, jmp = 0, grad = 0, total = 0;
+    size_t ck = 0, sg = 0, res = 0, lu = 0, lr = 0, raw = 0, jmp = 0, grad = 0, total = 0;
 };
 
 AdjLayout adj_layout(const dgm_plan* P, int64_t n) {
@@ -1712,10 +1709,9 @@ AdjLayout adj_layout(const dgm_plan* P, int64_t n) {
     size_t off = 0;
     L.ck = off; off += L.sb * size_t(std::max<int64_t>(L.nseg, 1));
     L.sg = off; off += L.sb * size_t(5 * L.seg);
-    L.tmp = off; off += L.sb * 2;
     L.res = off; off += L.sb;
     L.lu = off; off += L.sb;
-    L.lr = off; off += L.sb;
+    L.lr = off; off += L.sb * 2;
     L.raw = off; off += L.fb;
     L.jmp = off; off += align256(size_t(24) * P->NF * C * rs);
     L.grad = off; off += align256(sizeof(double) * 2 * C);
@@ -1793,18 +1789,17 @@ extern "C" int dgm_forward_record(dgm_plan* P, int64_t n_steps, double t0, doubl
     return DGM_OK;
 }
 
-// LSRK4 stages of one step from `in` (= st[0]): the inputs of stages 1..4 go to
-// st[1..4] (to scratch buffers when st is null), the step's result to `out`;
-// with out.f == nullptr the sweep stops after the first nst stages.
-static int lsrk_stages(dgm_plan* P, StateRef in, StateRef* st, int nst, StateRef tmp0, StateRef tmp1,
-                       StateRef res, StateRef out, double t) {
+// LSRK4 stages of one step from st[0]: the inputs of stages 1..4 go to st[1..4], the
+// step's result to `out`; with out.f == nullptr the sweep stops after the first nst
+// stages.
+static int lsrk_stages(dgm_plan* P, StateRef* st, int nst, StateRef res, StateRef out, double t) {
     StageParams prm;
     stage_params(P, prm);
     const double dt = P->opt.dt;
-    StateRef cur = in;
+    StateRef cur = st[0];
     for (int k = 0; k < 5; ++k) {
         StateRef nxt;
-        if (k < 4) nxt = st ? st[k + 1] : ((k % 2) ? tmp1 : tmp0);
+        if (k < 4) nxt = st[k + 1];
         else nxt = out;
         if (k >= nst && !out.f) break;
         prm.u = cur.f;
@@ -1823,18 +1818,6 @@ static int lsrk_stages(dgm_plan* P, StateRef in, StateRef* st, int nst, StateRef
     return DGM_OK;
 }
 
-template <typename R>
-static int axpby(dgm_plan* P, StateRef y, StateRef x, double a, double b, const AdjLayout& L) {
-    const int64_t nf = int64_t(L.fb / sizeof(R));
-    axpby_kernel<R><<<1216, 256, 0, P->stream>>>(static_cast<R*>(y.f), static_cast<const R*>(x.f), a, b, nf);
-    if (L.ab) {
-        const int64_t na = int64_t(L.ab / sizeof(R));
-        axpby_kernel<R><<<1216, 256, 0, P->stream>>>(static_cast<R*>(y.a), static_cast<const R*>(x.a), a, b, na);
-    }
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? DGM_OK : cuda_fail(e, "axpby launch");
-}
-
 extern "C" int dgm_adjoint(dgm_plan* P, int64_t n_steps, double t0, const double* drec, void* ws_,
                            double* deps, double* dmu) {
     if (P && P->k_active < P->mesh.K) return fail(DGM_EUNSUP, "the adjoint needs every element active");
@@ -1851,11 +1834,13 @@ extern "C" int dgm_adjoint(dgm_plan* P, int64_t n_steps, double t0, const double
     const int Sc = P->opt.n_columns;
     const int64_t per = int64_t(Sc) * P->n_rec * 3;
     const double dt = P->opt.dt;
-    StateRef lu = slot(ws, L.lu, 0, L), lr = slot(ws, L.lr, 0, L), res = slot(ws, L.res, 0, L);
-    StateRef tmp0 = slot(ws, L.tmp, 0, L), tmp1 = slot(ws, L.tmp, 1, L);
+    // the stage residual lr and the one the stage kernel forms for the next stage
+    StateRef lu = slot(ws, L.lu, 0, L), lr = slot(ws, L.lr, 0, L), lrn = slot(ws, L.lr, 1, L);
+    StateRef res = slot(ws, L.res, 0, L);
     StateRef st[5];
     cudaError_t e;
     if ((e = cudaMemsetAsync(lu.f, 0, L.sb, P->stream)) != cudaSuccess) return cuda_fail(e, "clear");
+    if ((e = cudaMemsetAsync(lr.f, 0, L.sb, P->stream)) != cudaSuccess) return cuda_fail(e, "clear");
     double* gcol = reinterpret_cast<double*>(ws + L.grad);
     if ((e = cudaMemsetAsync(gcol, 0, sizeof(double) * 2 * K * Sc, P->stream)) != cudaSuccess)
         return cuda_fail(e, "clear");
@@ -1871,7 +1856,7 @@ extern "C" int dgm_adjoint(dgm_plan* P, int64_t n_steps, double t0, const double
             for (int k = 0; k < 5; ++k) sti[k] = slot(ws, L.sg, size_t(5 * (i - start) + k), L);
             const StateRef nxt = (i + 1 < end) ? slot(ws, L.sg, size_t(5 * (i + 1 - start)), L)
                                                : StateRef{nullptr, nullptr};
-            rc = lsrk_stages(P, sti[0], sti, 4, tmp0, tmp1, res, nxt, t0 + double(i) * dt);
+            rc = lsrk_stages(P, sti, 4, res, nxt, t0 + double(i) * dt);
             if (rc) return rc;
         }
         for (int64_t n = end - 1; n >= start; --n) {
@@ -1879,18 +1864,14 @@ extern "C" int dgm_adjoint(dgm_plan* P, int64_t n_steps, double t0, const double
                 const unsigned nb = unsigned((int64_t(Sc) * 3 * P->N + 127) / 128);
                 if (f64)
                     inject_receivers<double><<<nb, 128, 0, P->stream>>>(
-                        static_cast<double*>(lu.f), recw, P->n_rec, K, Sc, P->N, drec + n * per);
+                        static_cast<double*>(lu.f), static_cast<double*>(lr.f), LSRK_B[4], recw, P->n_rec, K, Sc, P->N, drec + n * per);
                 else
                     inject_receivers<float><<<nb, 128, 0, P->stream>>>(
-                        static_cast<float*>(lu.f), recw, P->n_rec, K, Sc, P->N, drec + n * per);
+                        static_cast<float*>(lu.f), static_cast<float*>(lr.f), float(LSRK_B[4]), recw, P->n_rec, K, Sc, P->N, drec + n * per);
             }
             const double tn = t0 + double(n) * dt;
             for (int k = 0; k < 5; ++k) st[k] = slot(ws, L.sg, size_t(5 * (n - start) + k), L);
             for (int k = 4; k >= 0; --k) {
-                // lr = a_{k+1} lr + b_k lu  (a_5 := 0 starts each step)
-                const double a = (k == 4) ? 0.0 : LSRK_A[k + 1];
-                rc = f64 ? axpby<double>(P, lr, lu, a, LSRK_B[k], L) : axpby<float>(P, lr, lu, a, LSRK_B[k], L);
-                if (rc) return rc;
                 StageParams prm;
                 stage_params(P, prm);
                 prm.u = st[k].f;
@@ -1905,6 +1886,13 @@ extern "C" int dgm_adjoint(dgm_plan* P, int64_t n_steps, double t0, const double
                 ap.lr = lr.f;
                 ap.lu = lu.f;
                 ap.lr_aux = lr.a;
+                // next: lr = a_k lr + b_{k-1} lu; a step starts with lr = b_4 lu
+                if (n > 0 || k > 0) {
+                    ap.lr_next = lrn.f;
+                    ap.lr_aux_next = lrn.a;
+                    ap.a_next = k > 0 ? LSRK_A[k] : 0.0;
+                    ap.b_next = LSRK_B[k > 0 ? k - 1 : 4];
+                }
                 ap.lu_aux = lu.a;
                 ap.u = st[k].f;
                 ap.aux = st[k].a;
@@ -1926,6 +1914,7 @@ extern "C" int dgm_adjoint(dgm_plan* P, int64_t n_steps, double t0, const double
                 ap.dt = dt;
                 rc = P->kt->launch_adjoint(ap, P->stream);
                 if (rc) return fail(rc, "adjoint kernel launch failed");
+                std::swap(lr, lrn);
             }
         }
     }

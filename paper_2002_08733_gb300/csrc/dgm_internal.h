@@ -203,6 +203,9 @@ struct AdjParams {
     void* lu;             // adjoint state (fields), updated in place
     const void* lr_aux;   // adjoint residual (PML aux)     [6][N][P][S]
     void* lu_aux;         // adjoint state (PML aux), updated in place
+    void* lr_next;        // the next stage's residual a_next lr + b_next lu (fields), or null
+    void* lr_aux_next;    // the same for the PML aux
+    double a_next, b_next;
     const void* u;        // forward stage input (fields)
     const void* aux;      // forward stage input (PML aux)
     const void* raw;      // forward right-hand side before the mass inverse

@@ -625,8 +625,6 @@ stage_kernel(const StageParams prm) {
     constexpr int NF = nfmodes(P);
     constexpr int NG = NT / TE;                         // column groups working side by side
     constexpr int NPART = NG >= 24 ? 4 : (NG >= 12 ? 2 : 1);  // row parts of phases 4 and 5
-    constexpr bool DO_E = (MODE != MODE_LF_H);   // E equation updated
-    constexpr bool DO_H = (MODE != MODE_LF_E);   // H equation updated
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R* us = reinterpret_cast<R*>(smem_raw);      // [6N][TE]
     R* trO = us + 6 * N * TE;                    // [4][6][NF][TE]  own traces -> g
@@ -1059,8 +1057,6 @@ stage_kernel(const StageParams prm) {
     for (int it = grp; it < 6 * NPART && !TC; it += NG) {
         const int comp = it / NPART;
         const int part = it % NPART;
-        if (!DO_E && comp < 3) continue;
-        if (!DO_H && comp >= 3) continue;
         const R sgn = eg[G_DET * TE + c] < R(0) ? R(-1) : R(1);
         R acc[N];
         rhs_part<P, R, TE, NPART>(part, comp, c, us, trO, sgn, acc);
@@ -1092,8 +1088,6 @@ stage_kernel(const StageParams prm) {
     for (int it = grp; it < 2 * NP5; it += NG) {
         const int field = it / NP5;
         const int part = it % NP5;
-        if (!DO_E && field == 0) continue;
-        if (!DO_H && field == 1) continue;
         if (!active) continue;
         const int fb = 3 * field;   // first component of this field
         const R det = eg[G_DET * TE + c];
@@ -1113,7 +1107,6 @@ stage_kernel(const StageParams prm) {
         int32_t pi = -1;
         if (prm.pml != nullptr) pi = prm.pml[e];
         R ETA[3][3], SIG[3][3], XI[3][3];
-        constexpr bool LF = (MODE == MODE_LF_E || MODE == MODE_LF_H);
         R ait[9], AT[3][3], sg3[3], et3[3], xi3[3];   // PML: A^-T, A^T, sigma, eta, xi
         if (pi >= 0) {
 #pragma unroll
@@ -1138,7 +1131,7 @@ stage_kernel(const StageParams prm) {
             et3[0] = sy + sz - sx; et3[1] = sz + sx - sy; et3[2] = sx + sy - sz;
             xi3[0] = (sx - sy) * (sx - sz); xi3[1] = (sy - sz) * (sy - sx); xi3[2] = (sz - sx) * (sz - sy);
 #pragma unroll
-            for (int j = 0; j < 3 && !LF; ++j)
+            for (int j = 0; j < 3; ++j)
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     ETA[j][k] = R(0);
@@ -1165,93 +1158,53 @@ stage_kernel(const StageParams prm) {
         const int lo = part * N / NP5, hi = (part + 1) * N / NP5;
         const IX gb = IX(fb * N + lo) * C + col;          // (fb, lo) in the fields
         const IX ab = IX(fb * N + lo) * C2 + acol;        // (fb, lo) in the auxiliaries
-        // rows l = lo + i with a compile-time i, so that the prefetched
-        // residuals stay in registers
+        // rows l = lo + i with a compile-time i, so that the prefetched residuals
+        // stay in registers; in the layer in chunks whose loads are all requested
+        // before their arithmetic
+        constexpr int CR = RP5 < 2 ? RP5 : 2;
 #pragma unroll
-        for (int i = 0; i < RP5; ++i) {
-            const int l = lo + i;
-            if (!P5_EVEN && l >= hi) break;
-            R r[3], uv[3], du[3];
+        for (int i0 = 0; i0 < RP5; i0 += CR) {
+            R av[CR][3], ar[CR][3];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                r[k] = rh[((fb + k) * N + l) * TE + c];
-                uv[k] = us[((fb + k) * N + l) * TE + c];
-            }
-#pragma unroll
-            for (int k = 0; k < 3; ++k) du[k] = B[k][0] * r[0] + B[k][1] * r[1] + B[k][2] * r[2];
-            if (LF && pi >= 0) {
-                // Leapfrog with the PML terms by the trapezoid rule (Sec. V), per
-                // Cartesian component in the physical frame X = A^-T x (the 3x3
-                // mass blocks become diagonal there):
-                //   X_new = ((1 - dt eta/2) X + dt (A^-T du - A^-T aux / mat)) / (1 + dt eta/2)
-                // with du the mass-inverted curl/flux terms and aux this field's
-                // auxiliary (p for E, q for H); then the other field's auxiliary
-                //   Z_new = gamma Z + dt beta mat' xi Y,  beta = 1/(1 + dt sigma/2),
-                //   gamma = (1 - dt sigma/2) beta,  Y = A^-T (other field), mat' its
-                // material; covariant coefficients are A^T times physical ones.
-                const int ob = 3 - fb;                         // the other field
-                const R omat = field == 0 ? eg[G_MU * TE + c] : eg[G_EPS * TE + c];
-                const IX abo = IX(ob * N + lo) * C2 + acol;    // (ob, lo) in the auxiliaries
-                R* auxl = static_cast<R*>(prm.aux_out);        // in place: aux_out == aux
-                R av[3], ov[3], oa[3];
+            for (int i = 0; i < CR; ++i)
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                    av[k] = auxl[ab + IX(k * N + i) * C2];
-                    ov[k] = us[((ob + k) * N + l) * TE + c];
-                    oa[k] = auxl[abo + IX(k * N + i) * C2];
+                    const bool ok = pi >= 0 && i0 + i < RP5 && (P5_EVEN || lo + i0 + i < hi);
+                    const IX aj = ab + IX(k * N + i0 + i) * C2;
+                    av[i][k] = ok ? aux[aj] : R(0);
+                    ar[i][k] = ok && ca != R(0) ? auxr[aj] : R(0);
                 }
-                R Xn[3], Zn[3];
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const R x = ait[3 * a] * uv[0] + ait[3 * a + 1] * uv[1] + ait[3 * a + 2] * uv[2];
-                    const R y = ait[3 * a] * du[0] + ait[3 * a + 1] * du[1] + ait[3 * a + 2] * du[2];
-                    const R z = ait[3 * a] * av[0] + ait[3 * a + 1] * av[1] + ait[3 * a + 2] * av[2];
-                    const R hd = R(0.5) * dt * et3[a];
-                    Xn[a] = ((R(1) - hd) * x + dt * (y - z * imat)) / (R(1) + hd);
-                    const R yo = ait[3 * a] * ov[0] + ait[3 * a + 1] * ov[1] + ait[3 * a + 2] * ov[2];
-                    const R zo = ait[3 * a] * oa[0] + ait[3 * a + 1] * oa[1] + ait[3 * a + 2] * oa[2];
-                    const R beta = R(1) / (R(1) + R(0.5) * dt * sg3[a]);
-                    const R gamma = (R(1) - R(0.5) * dt * sg3[a]) * beta;
-                    Zn[a] = gamma * zo + dt * beta * omat * xi3[a] * yo;
-                }
+            for (int i = 0; i < CR; ++i) {
+                const int l = lo + i0 + i;
+                if (i0 + i >= RP5 || (!P5_EVEN && l >= hi)) break;
+                R r[3], uv[3], du[3];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                    uo[gb + IX(k * N + i) * C] = AT[k][0] * Xn[0] + AT[k][1] * Xn[1] + AT[k][2] * Xn[2];
-                    auxl[abo + IX(k * N + i) * C2] = AT[k][0] * Zn[0] + AT[k][1] * Zn[1] + AT[k][2] * Zn[2];
+                    r[k] = rh[((fb + k) * N + l) * TE + c];
+                    uv[k] = us[((fb + k) * N + l) * TE + c];
                 }
-                continue;
-            }
-            if (pi >= 0) {
-                R av[3];
 #pragma unroll
-                for (int k = 0; k < 3; ++k) av[k] = aux[ab + IX(k * N + i) * C2];
+                for (int k = 0; k < 3; ++k) du[k] = B[k][0] * r[0] + B[k][1] * r[1] + B[k][2] * r[2];
+                if (pi >= 0) {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    du[k] -= ETA[k][0] * uv[0] + ETA[k][1] * uv[1] + ETA[k][2] * uv[2] + av[k] * imat;
-                    const R da = -(SIG[k][0] * av[0] + SIG[k][1] * av[1] + SIG[k][2] * av[2]) +
-                                 mat * (XI[k][0] * uv[0] + XI[k][1] * uv[1] + XI[k][2] * uv[2]);
-                    const IX aj = ab + IX(k * N + i) * C2;
-                    if (MODE == MODE_RHS) {
-                        auxo[aj] = da;
-                    } else if (MODE == MODE_LSRK) {
-                        const R rr = (ca == R(0) ? R(0) : ca * auxr[aj]) + dt * da;
+                    for (int k = 0; k < 3; ++k) {
+                        du[k] -= ETA[k][0] * uv[0] + ETA[k][1] * uv[1] + ETA[k][2] * uv[2] + av[i][k] * imat;
+                        const R da = -(SIG[k][0] * av[i][0] + SIG[k][1] * av[i][1] + SIG[k][2] * av[i][2]) +
+                                     mat * (XI[k][0] * uv[0] + XI[k][1] * uv[1] + XI[k][2] * uv[2]);
+                        const IX aj = ab + IX(k * N + i0 + i) * C2;
+                        const R rr = (ca == R(0) ? R(0) : ca * ar[i][k]) + dt * da;
                         auxr[aj] = rr;
-                        auxo[aj] = av[k] + cb * rr;
+                        auxo[aj] = av[i][k] + cb * rr;
                     }
                 }
-            }
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const IX gi = gb + IX(k * N + i) * C;
-                if (MODE == MODE_RHS) {
-                    uo[gi] = du[k];
-                } else if (MODE == MODE_LSRK) {
+                for (int k = 0; k < 3; ++k) {
+                    const IX gi = gb + IX(k * N + i0 + i) * C;
                     // resv is 0 when a = 0 (first stage), so no branch on a here
-                    const R rr = ca * resv[PREFETCH_RES ? k : 0][PREFETCH_RES ? i : 0] + dt * du[k];
+                    const R rr = ca * resv[PREFETCH_RES ? k : 0][PREFETCH_RES ? i0 + i : 0] + dt * du[k];
                     res[gi] = rr;
                     uo[gi] = uv[k] + cb * rr;
-                } else {
-                    uo[gi] = uv[k] + dt * du[k];
                 }
             }
         }
