@@ -594,20 +594,16 @@ static int build_tmaps(dgm_plan* P) {
             const cuuint32_t box[2] = {te, cuuint32_t(TM_ROWS_EG)};
             ok = ok && tmap_encode(P, &m[TM_GEO], geo, 2, dims, &row, box);
         }
-        {   // face constants [4][16][K]: 15 rows per face, 16 with the penalty
-            const cuuint64_t dims[3] = {Ke, cuuint64_t(TM_ROWS_FACE), 4};
-            const cuuint64_t str[2] = {row, row * cuuint64_t(TM_ROWS_FACE)};
+        {   // face constants [4][15][K]
+            const cuuint64_t dims[3] = {Ke, cuuint64_t(TM_ROWS_FC), 4};
+            const cuuint64_t str[2] = {row, row * cuuint64_t(TM_ROWS_FC)};
             const cuuint32_t box[3] = {te, cuuint32_t(TM_ROWS_FC), 4};
-            const cuuint32_t boxs[3] = {te, cuuint32_t(TM_ROWS_FACE), 4};
             ok = ok && tmap_encode(P, &m[TM_FC], fcp, 3, dims, str, box);
-            ok = ok && tmap_encode(P, &m[TM_FCS], fcp, 3, dims, str, boxs);
         }
-        {   // metric (and A^T) rows of the table [FC_ROWS][K], from row 4 * 16
+        {   // metric rows of the table [FC_ROWS][K], from row 4 * 15
             const cuuint64_t dims[2] = {Ke, cuuint64_t(FC_ROWS)};
             const cuuint32_t box[2] = {te, cuuint32_t(TM_ROWS_GM)};
-            const cuuint32_t boxs[2] = {te, cuuint32_t(TM_ROWS_GM + TM_ROWS_GA)};
             ok = ok && tmap_encode(P, &m[TM_GM], fcp, 2, dims, &row, box);
-            ok = ok && tmap_encode(P, &m[TM_GMGA], fcp, 2, dims, &row, boxs);
         }
         if (!ok) return DGM_OK;   // a shape the encoder refuses: per-thread loads
     }
@@ -630,7 +626,7 @@ static int build_face_table(dgm_plan* P) {
     stage_params(P, prm);
     const bool sip = P->sip_alpha > 0.0;
     prm.sfid = sip ? reinterpret_cast<const int32_t*>(P->geom + P->off_sfid) : nullptr;
-    int rc = P->mixed ? DGM_OK : launch_face_consts(prm, P->kt->real_size, false, P->geom + P->off_fcp, P->stream);
+    int rc = P->mixed ? DGM_OK : launch_face_consts(prm, P->kt->real_size, P->geom + P->off_fcp, P->stream);
     if (!rc) rc = launch_tang_consts(prm, P->kt->real_size, sip, P->geom + P->off_fct, P->stream);
     return rc ? fail(rc, "face constants") : DGM_OK;
 }

@@ -170,27 +170,25 @@ inline cudaError_t launch_ex(void (*k)(A...), dim3 grid, unsigned block, size_t 
 // Tensor maps (CUtensorMap, 128 bytes each) of one tile width, all with the
 // tile's columns as the innermost box dimension: the field buffers as
 // [6][N][C] (box TE x N x 6), the element constants [G_COUNT][K] (box TE x 16),
-// the face constants as [4][16][K] (box TE x 15 x 4, or x 16 with the interior
-// penalty) and the metric rows of the face-constant table [FC_ROWS][K] (box
-// TE x 6, or TE x 15 with A^T); TM_UW: a field-shaped scratch buffer of the
+// the face constants as [4][15][K] (box TE x 15 x 4) and the metric rows of the
+// face-constant table [FC_ROWS][K] (box TE x 6); TM_UW: a field-shaped scratch buffer of the
 // autotuner (dgm_autotune), encoded while it times.
 enum TmapIndex {
-    TM_U0 = 0, TM_U1 = 1, TM_GEO = 2, TM_FC = 3, TM_FCS = 4, TM_GM = 5, TM_GMGA = 6, TM_UW = 7,
-    TMAP_COUNT = 8
+    TM_U0 = 0, TM_U1 = 1, TM_GEO = 2, TM_FC = 3, TM_GM = 4, TM_UW = 5,
+    TMAP_COUNT = 6
 };
 constexpr int TMAP_BYTES = 128;
 // rows of the boxes (the stage kernel's shared-memory rows): element constants,
-// face constants per face (15, or 16 with the penalty) of the 16 per face of
-// the table, metric, A^T
-constexpr int TM_ROWS_EG = 16, TM_ROWS_FC = 15, TM_ROWS_FACE = 16, TM_ROWS_GM = 6, TM_ROWS_GA = 9;
+// face constants per face, metric
+constexpr int TM_ROWS_EG = 16, TM_ROWS_FC = 15, TM_ROWS_GM = 6;
 constexpr int TMAP_SETS = 2;   // set 0: 32 columns, set 1: 16 columns
 constexpr int tmap_columns(int set) { return set == 0 ? 32 : 16; }
 
-// Rows per element of the precomputed face constants: 4 faces x 16, the
-// metric A^T A (6), A^T (9).
-constexpr int FC_ROWS = 4 * 16 + 6 + 9;
+// Rows per element of the precomputed face constants: 4 faces x 15, the
+// metric A^T A (6).
+constexpr int FC_ROWS = 4 * 15 + 6;
 // Computes them for a plan (dgm_facec.cu); real_size 4 or 8.
-int launch_face_consts(const StageParams& prm, int real_size, bool sip, void* out, void* stream);
+int launch_face_consts(const StageParams& prm, int real_size, void* out, void* stream);
 // Rows per element of the tangential face-constant table (dgm_tang.cuh): per face
 // 8, the metric A^T A (6), two mass factors, the penalty's 4 x 7; and its launcher.
 constexpr int TG_ROWS = 4 * 8 + 6 + 2 + 4 * 7;

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(TE * LF_NG, 2) lf_kernel(const StageParams prm
     // this thread's flux item (face, third of the modes): its constants
     const int ff = grp / 3, ch = grp % 3;
     R q[9], na = R(0), cc = R(0);
-    auto face_const = [&](int r) { return active ? fcp[IX(ff * FCF + r) * K + e] : R(0); };
+    auto face_const = [&](int r) { return active ? fcp[IX(ff * FGR + r) * K + e] : R(0); };
 #pragma unroll
     for (int i = 0; i < 9; ++i) q[i] = face_const(FR_Q + i);
     na = face_const(O == 0 ? FR_NAE : FR_NAH);
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(TE * LF_NG, 2) lf_kernel(const StageParams prm
             if (!active || q >= T1) continue;
             tmp[i] = q < 3 * N        ? u[IX(3 * O * N + q) * C + col]
                      : q < 3 * N + EG ? gr[IX(q - 3 * N) * K + e]
-                                      : fcp[IX(4 * FCF + q - 3 * N - EG) * K + e];
+                                      : fcp[IX(4 * FGR + q - 3 * N - EG) * K + e];
         }
 #pragma unroll
         for (int i = 0; i < UR; ++i) {

@@ -77,12 +77,11 @@ enum FaceConst {
     FC_BND = 17   // 1 on a PEC face
 };
 constexpr int EG = 16;   // element constants per column (same slots as G_*)
-constexpr int NBS = 4;   // neighbour codes per column staged in shared memory (+4 facet
-                         // codes with the interior penalty)
+constexpr int NBS = 4;   // neighbour codes per column staged in shared memory
 
 // Face constants of the stage kernel, whose flux works in the element's
 // reference frame (see face_constants_ref), per (face, column).
-constexpr int FGR = 15;   // (16 with the interior penalty: FR_KS)
+constexpr int FGR = 15;
 enum FaceConstRef {
     FR_Q = 0,     // Q = A^T A_n^-T (9, row major): neighbour reference components -> own
     FR_NAE = 9,   // -alpha_E: -1 on an interior face, -2 on a PEC face (e+ = -e-)
@@ -91,21 +90,17 @@ enum FaceConstRef {
     FR_CE = 11,   // s_T c_E
     FR_BE = 12,   // b_E / (|det A| |A^-T m_f|)
     FR_CH = 13,   // s_T c_H
-    FR_BH = 14,   // b_H / (|det A| |A^-T m_f|)
-    FR_KS = 15    // interior penalty, on the facet's owner side: (alpha / mu_F) / (det A |A^-T m_f|)
+    FR_BH = 14    // b_H / (|det A| |A^-T m_f|)
 };
 constexpr int GM = 6;    // metric A^T A per column: entries 00, 01, 02, 11, 12, 22
-constexpr int GA = 9;    // A^T per column, row major (interior penalty only)
-template <bool SIP> __host__ __device__ constexpr int fgr() { return SIP ? FGR + 1 : FGR; }
-template <bool SIP> __host__ __device__ constexpr int nbs_rows() { return SIP ? 2 * NBS : NBS; }
 
-template <int P, typename R, int TE, bool TC = false, bool SIP = false>
+template <int P, typename R, int TE, bool TC = false>
 __host__ __device__ constexpr size_t stage_smem_bytes() {
     // + an mbarrier (phase-1 bulk copies; the tensor-core variant's MMAs) and the
     // tensor-memory base (the operator image lives in the neighbour-trace array,
     // dead after phase 3)
     return sizeof(R) * size_t(TE) *
-               (6 * nmodes(P) + 48 * nfmodes(P) + 4 * fgr<SIP>() + EG + GM + (SIP ? GA : 0) + nbs_rows<SIP>()) +
+               (6 * nmodes(P) + 48 * nfmodes(P) + 4 * FGR + EG + GM + NBS) +
            size_t(32);
 }
 
@@ -201,13 +196,11 @@ __device__ __forceinline__ void face_constants_tab(int f, const R (&ait)[9], R d
 // is not needed.
 // incident: a boundary face through which an incident field enters (ghost state
 // e+ = e- + 2 E_inc, h+ = -h-, Z+ = Z-; the E_inc part is added by flux_face).
-// ks_num: alpha / mu_F on the owner side of a penalised interior face, else 0.
-// ga (with gm, face 0 only): the element's A^T, row major, for the penalty.
-template <typename R, bool SIP>
+template <typename R>
 __device__ __forceinline__ void face_constants_ref(int f, const R (&ait)[9], R det, R epsm, R mum,
                                                    bool has_nbr, const R (&aitn)[9], R zn,
                                                    int upwind, R* fc, R* gm, bool incident,
-                                                   R ks_num, R* ga, int64_t TE) {
+                                                   int64_t TE) {
     // A^T = det A adj(A^-T), row major
     R at[9];
     at[0] = ait[4] * ait[8] - ait[5] * ait[7];
@@ -252,12 +245,7 @@ __device__ __forceinline__ void face_constants_ref(int f, const R (&ait)[9], R d
     fc[FR_BE * TE] = kb * be;
     fc[FR_CH * TE] = st * ch;
     fc[FR_BH * TE] = kb * bh;
-    if constexpr (SIP) fc[FR_KS * TE] = ks_num * st * kb;
     if (gm != nullptr) {
-        if constexpr (SIP) {
-#pragma unroll
-            for (int k = 0; k < 9; ++k) ga[k * TE] = at[k];
-        }
         gm[0 * TE] = at[0] * at[0] + at[1] * at[1] + at[2] * at[2];
         gm[1 * TE] = at[0] * at[3] + at[1] * at[4] + at[2] * at[5];
         gm[2 * TE] = at[0] * at[6] + at[1] * at[7] + at[2] * at[8];
@@ -269,15 +257,11 @@ __device__ __forceinline__ void face_constants_ref(int f, const R (&ait)[9], R d
 
 // The stage kernel's face constants, computed once per plan (again when the
 // materials or the boundary codes change) for every element, stride K, in the
-// kernel's precision: rows f FCF + k (the penalty's layout), then the metric
-// A^T A and A^T.  The same function and inputs as a computation inside the
+// kernel's precision: rows f FGR + k, then the metric A^T A.  The same function and inputs as a computation inside the
 // stage kernel, so the same bits.
-constexpr int FCF = FGR + 1;
-static_assert(4 * FCF + GM + GA == FC_ROWS, "precomputed face-constant rows");
-static_assert(EG == TM_ROWS_EG && FGR == TM_ROWS_FC && FCF == TM_ROWS_FACE && GM == TM_ROWS_GM &&
-                  GA == TM_ROWS_GA,
-              "bulk-copy boxes match the shared-memory rows");
-template <typename R, bool SIP>
+static_assert(4 * FGR + GM == FC_ROWS, "precomputed face-constant rows");
+static_assert(EG == TM_ROWS_EG && FGR == TM_ROWS_FC && GM == TM_ROWS_GM, "bulk-copy boxes match the shared-memory rows");
+template <typename R>
 __global__ void face_consts_kernel(const StageParams prm, R* __restrict__ out) {
     const int64_t K = prm.K;
     const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -296,16 +280,9 @@ __global__ void face_consts_kernel(const StageParams prm, R* __restrict__ out) {
 #pragma unroll
         for (int k = 0; k < 9; ++k) aitn[k] = fn[int64_t(FNB_AIT + k) * K];
         const R zn = fn[int64_t(FNB_Z) * K];
-        R ksn = R(0);   // interior penalty on the facet's owner side: alpha / mu_F
-        if constexpr (SIP) {
-            const int32_t sf = prm.sfid[int64_t(f) * K + e];
-            if (sf >= 0 && (sf & 1)) ksn = R(prm.sip_alpha) / (R(0.5) * (mum + fn[int64_t(FNB_MU) * K]));
-        }
-        face_constants_ref<R, SIP>(f, ait, det, epsm, mum, code >= 0 && (code >> 2) < K, aitn, zn,
-                                   prm.upwind, out + int64_t(f * FCF) * K + e,
-                                   f == 0 ? out + int64_t(4 * FCF) * K + e : nullptr,
-                                   code <= -2 && prm.inc != nullptr, ksn,
-                                   out + int64_t(4 * FCF + GM) * K + e, K);
+        face_constants_ref<R>(f, ait, det, epsm, mum, code >= 0 && (code >> 2) < K, aitn, zn, prm.upwind,
+                              out + int64_t(f * FGR) * K + e, f == 0 ? out + int64_t(4 * FGR) * K + e : nullptr,
+                              code <= -2 && prm.inc != nullptr, K);
     }
 }
 
@@ -314,132 +291,20 @@ __host__ __device__ constexpr int sym3(int i, int j) {
     return i > j ? sym3(j, i) : (i == 0 ? j : (i == 1 ? 2 + j : 5));
 }
 
-// Interior penalty (phase 3 of the kernels instantiated with the penalty).
-// Owner side of face F, before its own traces become fluxes:
-// dh_s/dt = -(alpha / mu_F) A (m_f x de) / (det A |A^-T m_f|) per mode, with the
-// interior reference jump de = Q e+ - e-, and the facet field's stage update.
-template <int F, int NF, typename R, int TE, int MODE, int MC>
-__device__ __forceinline__ void sip_owner(int m0, int m1, int c, const R* trO, const R* trN, const R* d,
-                                          const R* hsv, R* hso, R* hsr, int64_t fs, const R* gac, R ca,
-                                          R cb, R dtc) {
-    constexpr int A = F == 0 ? -1 : F - 1;
-    constexpr int B = F % 3, CC = (F + 1) % 3;
-    // the item's facet values first (at most MC modes), so that their round
-    // trips overlap instead of following one another mode by mode
-    R hv[MC][3], rv[MC][3];
-#pragma unroll
-    for (int i = 0; i < MC; ++i)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int64_t j = int64_t(k * NF + m0 + i) * fs;
-            const bool ok = MODE == MODE_LSRK && m0 + i < m1;
-            hv[i][k] = ok ? hsv[j] : R(0);
-            rv[i][k] = ok ? hsr[j] : R(0);
-        }
-    R q[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) q[k] = k / 3 != A ? d[(FR_Q + k) * TE] : R(0);
-    R at[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) at[k] = gac[k * TE];
-    const R ks = d[FR_KS * TE];
-#pragma unroll
-    for (int i = 0; i < MC; ++i) {
-        const int m = m0 + i;
-        if (m >= m1) break;
-        const R* own = trO + (F * 6 * NF + m) * TE + c;
-        const R* nbt = trN + (F * 6 * NF + m) * TE + c;
-        R de[3] = {0, 0, 0};
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-            if (r != A)
-                de[r] = q[3 * r] * nbt[0] + q[3 * r + 1] * nbt[NF * TE] + q[3 * r + 2] * nbt[2 * NF * TE] -
-                        own[r * NF * TE];
-        R v[3];
-        if (F == 0) {
-            v[0] = de[2] - de[1];
-            v[1] = de[0] - de[2];
-            v[2] = de[1] - de[0];
-        } else {
-            v[A] = R(0);
-            v[B] = de[CC];
-            v[CC] = -de[B];
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const R r = -ks * (at[k] * v[0] + at[3 + k] * v[1] + at[6 + k] * v[2]);
-            const int64_t j = int64_t(k * NF + m) * fs;
-            if (MODE == MODE_RHS) {
-                hso[j] = r;
-            } else {
-                const R rr = ca * rv[i][k] + dtc * r;
-                hsr[j] = rr;
-                hso[j] = hv[i][k] + cb * rr;
-            }
-        }
-    }
-}
-
-// Both sides of face F, after the fluxes: the pulled-back E flux gains
-// s_T m_f x (A^T h_s) (central flux, c_E = 1/2, so s_T = 2 cE); the item's
-// facet values (at most MC modes) are loaded first.
-template <int F, int NF, typename R, int TE, int MC>
-__device__ __forceinline__ void sip_eflux(int m0, int m1, int c, R* trO, const R* hsv, int64_t fs,
-                                          const R* gac, R cE) {
-    constexpr int B = F % 3, CC = (F + 1) % 3;
-    R hv[MC][3];
-#pragma unroll
-    for (int i = 0; i < MC; ++i)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) hv[i][k] = m0 + i < m1 ? hsv[int64_t(k * NF + m0 + i) * fs] : R(0);
-    R at[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) at[k] = gac[k * TE];
-    const R sT = R(2) * cE;
-#pragma unroll
-    for (int i = 0; i < MC; ++i) {
-        const int m = m0 + i;
-        if (m >= m1) break;
-        R* own = trO + (F * 6 * NF + m) * TE + c;
-        R y[3];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) y[j] = at[3 * j] * hv[i][0] + at[3 * j + 1] * hv[i][1] + at[3 * j + 2] * hv[i][2];
-        if (F == 0) {
-            own[0 * NF * TE] += sT * (y[2] - y[1]);
-            own[1 * NF * TE] += sT * (y[0] - y[2]);
-            own[2 * NF * TE] += sT * (y[1] - y[0]);
-        } else {
-            own[B * NF * TE] += sT * y[CC];
-            own[CC * NF * TE] -= sT * y[B];
-        }
-    }
-}
-
 // Numerical flux of modes [m0, m1) of face F (compile time) in the reference
 // frame (face_constants_ref): reads both sides' reference traces, overwrites
 // the own traces with the pulled-back fluxes g.  On an axis face only the two
 // non-zero components of g are written.  FULL: the own trace has all three
 // components and the physical jumps M dx are stored for the adjoint.
-template <int F, int NF, typename R, int TE, int MODE, typename IX, bool SIP, int MC = 1>
+template <int F, int NF, typename R, int TE, int MODE, typename IX>
 __device__ __forceinline__ void flux_face(int m0, int m1, int c, R* trO, const R* trN,
                                           const R* fg, const R* gm, const R* eg, R* jumps,
                                           IX C, IX col, bool active, int32_t code,
-                                          const void* incp, const R* hsv, R* hso, R* hsr,
-                                          int64_t fs, const R* gac, R ca, R cb, R dtc) {
-    constexpr bool DO_E = (MODE != MODE_LF_H);   // E fluxes needed
-    constexpr bool DO_H = (MODE != MODE_LF_E);   // H fluxes needed
-    constexpr bool HAS_E = (MODE != MODE_LF_E);  // E jump used (H flux, upwind E flux)
-    constexpr bool HAS_H = DO_E;                 // H jump used (E flux, upwind H flux)
+                                          const void* incp) {
     constexpr bool FULL = (MODE == MODE_RAW);
     constexpr int A = F == 0 ? -1 : F - 1;       // axis of m_f = -e_A
     constexpr int B = F % 3, CC = (F + 1) % 3;   // the other two axes, (A, B, CC) cyclic
-    const R* d = fg + F * fgr<SIP>() * TE + c;
-    // interior penalty, owner side, first: it reads the traces before they
-    // become fluxes, and nothing of the flux is live yet
-    if constexpr (SIP) {
-        if (hso != nullptr)
-            sip_owner<F, NF, R, TE, MODE, MC>(m0, m1, c, trO, trN, d, hsv, hso, hsr, fs, gac, ca, cb, dtc);
-    }
+    const R* d = fg + F * FGR * TE + c;
     R q[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) q[k] = (FULL || k / 3 != A) ? d[(FR_Q + k) * TE] : R(0);
@@ -462,7 +327,7 @@ __device__ __forceinline__ void flux_face(int m0, int m1, int c, R* trO, const R
     const R kEcb = bE * gcb, kEcc = bE * gcc, kEbb = bE * gbb;
     const R kHcb = bH * gcb, kHcc = bH * gcc, kHbb = bH * gbb;
     // incident face (e+ = e- + 2 E_inc): the E jump is the incident term alone
-    const R* inc = (HAS_E && code <= -2 && incp != nullptr && active)
+    const R* inc = (code <= -2 && incp != nullptr && active)
                        ? static_cast<const R*>(incp) + IX(-code - 2) * NF * 3
                        : nullptr;
     // not unrolled: four copies of an unrolled loop (one per face) cost more in
@@ -472,7 +337,7 @@ __device__ __forceinline__ void flux_face(int m0, int m1, int c, R* trO, const R
         R* own = trO + (F * 6 * NF + m) * TE + c;
         const R* nbt = trN + (F * 6 * NF + m) * TE + c;
         R de[3] = {0, 0, 0}, dh[3] = {0, 0, 0};   // reference-frame jumps
-        if (HAS_E) {
+        {
             R tp[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) tp[k] = nbt[k * NF * TE];
@@ -487,7 +352,7 @@ __device__ __forceinline__ void flux_face(int m0, int m1, int c, R* trO, const R
             for (int r = 0; r < 3; ++r)
                 if (FULL || r != A) de[r] += inc[m * 3 + r];
         }
-        if (HAS_H) {
+        {
             R tp[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) tp[k] = nbt[(3 + k) * NF * TE];
@@ -510,7 +375,7 @@ __device__ __forceinline__ void flux_face(int m0, int m1, int c, R* trO, const R
             // m_f = (1, 1, 1): m x y = (y2 - y1, y0 - y2, y1 - y0)
             const R we[3] = {de[2] - de[1], de[0] - de[2], de[1] - de[0]};
             const R wh[3] = {dh[2] - dh[1], dh[0] - dh[2], dh[1] - dh[0]};
-            if (DO_E) {   // z = b_E A^T A w_e
+            {   // z = b_E A^T A w_e
                 const R z0 = bE * (g00 * we[0] + g01 * we[1] + g02 * we[2]);
                 const R z1 = bE * (g01 * we[0] + g11 * we[1] + g12 * we[2]);
                 const R z2 = bE * (g02 * we[0] + g12 * we[1] + g22 * we[2]);
@@ -518,7 +383,7 @@ __device__ __forceinline__ void flux_face(int m0, int m1, int c, R* trO, const R
                 own[1 * NF * TE] = cE * wh[1] - (z0 - z2);
                 own[2 * NF * TE] = cE * wh[2] - (z1 - z0);
             }
-            if (DO_H) {   // z = b_H A^T A w_h
+            {   // z = b_H A^T A w_h
                 const R z0 = bH * (g00 * wh[0] + g01 * wh[1] + g02 * wh[2]);
                 const R z1 = bH * (g01 * wh[0] + g11 * wh[1] + g12 * wh[2]);
                 const R z2 = bH * (g02 * wh[0] + g12 * wh[1] + g22 * wh[2]);
@@ -528,18 +393,15 @@ __device__ __forceinline__ void flux_face(int m0, int m1, int c, R* trO, const R
             }
         } else {
             // m_f = -e_A: (m x y)_A = 0, (m x y)_B = y_CC, (m x y)_CC = -y_B
-            if (DO_E) {
+            {
                 own[B * NF * TE] = cE * dh[CC] - kEcb * de[CC] + kEcc * de[B];
                 own[CC * NF * TE] = -cE * dh[B] + kEbb * de[CC] - kEcb * de[B];
             }
-            if (DO_H) {
+            {
                 own[(3 + B) * NF * TE] = -cH * de[CC] - kHcb * dh[CC] + kHcc * dh[B];
                 own[(3 + CC) * NF * TE] = cH * de[B] + kHbb * dh[CC] - kHcb * dh[B];
             }
         }
-    }
-    if constexpr (SIP) {
-        if (hsv != nullptr) sip_eflux<F, NF, R, TE, MC>(m0, m1, c, trO, hsv, fs, gac, cE);
     }
 }
 
@@ -612,15 +474,10 @@ __device__ __forceinline__ void rhs_part(int part, int comp, int c, const R* us,
 // tensor cores (dgm_tc.cuh, TcShape), with tensor-memory row (field, column);
 // phase 5 reads the pre-mass right-hand side from tensor memory.  The other
 // phases are shared with the SIMT kernel.
-// SIP: interior penalty with a facet field (LSRK and right-hand-side modes of
-// the SIMT kernel): facet codes staged in phase 1, A^T and one more face
-// constant, the facet terms in phase 3 (sip_owner, sip_eflux).
-template <int P, typename R, int TE, int NT, int MODE, typename IX = int64_t, bool TC = false,
-          bool SIP = false>
+template <int P, typename R, int TE, int NT, int MODE, typename IX = int64_t, bool TC = false>
 __global__ void __launch_bounds__(NT, TC ? 1 : ((sizeof(R) == 8 || P <= 3) ? 2 : 1))
 stage_kernel(const StageParams prm) {
-    static_assert(!SIP || (!TC && (MODE == MODE_LSRK || MODE == MODE_RHS)), "interior penalty modes");
-    constexpr int FGRT = fgr<SIP>();
+    static_assert(MODE == MODE_LSRK || MODE == MODE_RAW, "LSRK4 stages and the adjoint's forward quantities");
     constexpr int N = nmodes(P);
     constexpr int NF = nfmodes(P);
     constexpr int NG = NT / TE;                         // column groups working side by side
@@ -629,19 +486,18 @@ stage_kernel(const StageParams prm) {
     R* us = reinterpret_cast<R*>(smem_raw);      // [6N][TE]
     R* trO = us + 6 * N * TE;                    // [4][6][NF][TE]  own traces -> g
     R* trN = trO + 24 * NF * TE;                 // [4][6][NF][TE]  nbr traces -> rhs [6][N][TE]
-    R* fg = trN + 24 * NF * TE;                  // [4][FGRT][TE]
-    R* eg = fg + 4 * FGRT * TE;                  // [EG][TE]
+    R* fg = trN + 24 * NF * TE;                  // [4][FGR][TE]
+    R* eg = fg + 4 * FGR * TE;                  // [EG][TE]
     R* gm = eg + EG * TE;                        // [GM][TE] metric A^T A
-    R* ga = gm + GM * TE;                        // [GA][TE] A^T (interior penalty only)
-    int32_t* nbs = reinterpret_cast<int32_t*>(ga + (SIP ? GA : 0) * TE);   // neighbour (+ facet) codes
-    static_assert(!TC || (sizeof(R) == 4 && TE == 64 && (MODE == MODE_LSRK || MODE == MODE_RHS) &&
+    int32_t* nbs = reinterpret_cast<int32_t*>(gm + GM * TE);   // [NBS][TE] neighbour codes
+    static_assert(!TC || (sizeof(R) == 4 && TE == 64 && MODE == MODE_LSRK &&
                           (NT / TE) % 2 == 0 && TcShape<P>::FITS),
-                  "tensor-core variant: FP32, 64 columns, LSRK or right-hand side, even groups");
+                  "tensor-core variant: FP32, 64 columns, LSRK, even groups");
     // mbarrier (phase-1 bulk copies; tensor-core variant: its MMAs) and the
     // tensor-memory base address after the tables; the tensor-core variant's
     // operator image goes into the neighbour-trace array in phase 4
     uint64_t* tc_bar = reinterpret_cast<uint64_t*>(
-        (reinterpret_cast<uintptr_t>(nbs + nbs_rows<SIP>() * TE) + 7) & ~uintptr_t(7));
+        (reinterpret_cast<uintptr_t>(nbs + NBS * TE) + 7) & ~uintptr_t(7));
     uint32_t* tc_base = reinterpret_cast<uint32_t*>(tc_bar + 1);
     if constexpr (TC) {
         static_assert(TcShape<P>::B_BYTES <= int(sizeof(R)) * 24 * nfmodes(P) * TE,
@@ -669,8 +525,7 @@ stage_kernel(const StageParams prm) {
     // stage coefficients in the kernel's precision: FP32 kernels read the FP32
     // copies, so that no conversion runs on the FP64 pipe
     auto coef = [&](double d, float f) { return sizeof(R) == 4 ? R(f) : R(d); };
-    for (int r = grp; r < nbs_rows<SIP>(); r += NG)   // neighbour codes, then facet codes (-1: none)
-        nbs[r * TE + c] = !active ? -1 : r < 4 ? prm.nbr[IX(r) * K + e] : prm.sfid[IX(r - 4) * K + e];
+    for (int r = grp; r < NBS; r += NG) nbs[r * TE + c] = active ? prm.nbr[IX(r) * K + e] : -1;   // neighbour codes
 
     // ---- phase 1: tile coefficients, element and face constants --------------
     // Every group loads rows of the tile: the coefficients, the element
@@ -681,13 +536,10 @@ stage_kernel(const StageParams prm) {
     // round trips of the tile and the gathers overlap each other and work.
     constexpr int NOWN = 12, NNBR = 24;                 // phase-2 items
     R vn[N];                                            // neighbour coefficients (phase 2)
-    auto nbr_item_active = [&](int comp) {
-        return !((MODE == MODE_LF_E && comp < 3) || (MODE == MODE_LF_H && comp >= 3));
-    };
     // neighbour item ni = (face ni / 6, component ni % 6): request the
     // neighbour's coefficients of that component given the face's code
     auto request_nbr = [&](int ni, int32_t code, R (&dst)[N]) {
-        if (ni < NNBR && nbr_item_active(ni % 6) && active && code >= 0 && (code >> 2) < K) {
+        if (ni < NNBR && active && code >= 0 && (code >> 2) < K) {
             const IX ncol = IX(code >> 2) * S + s;
 #pragma unroll
             for (int l = 0; l < N; ++l) dst[l] = u[IX((ni % 6) * N + l) * C + ncol];
@@ -696,7 +548,7 @@ stage_kernel(const StageParams prm) {
     // neighbour item ni: the trace of the neighbour's coefficients v on its
     // face (code & 3) into trN (zeros without a neighbour)
     auto nbr_trace = [&](int ni, int32_t code, const R (&v)[N]) {
-        if (ni < NNBR && nbr_item_active(ni % 6)) {
+        if (ni < NNBR) {
             const int nf = ni / 6, ncomp = ni % 6;
             const bool has_nbr = code >= 0 && (code >> 2) < K;
             if (code >= 0 && (code >> 2) >= K) atomicOr(prm.status, ST_BAD_NEIGHBOUR);
@@ -728,7 +580,7 @@ stage_kernel(const StageParams prm) {
     constexpr bool BULK_OK = !TC && (TE * int(sizeof(R)) == 128 || (sizeof(R) == 4 && TE == 16));
     const bool bulk = BULK_OK && prm.tm_u >= 0 && (tc::smem_addr(smem_raw) & 127u) == 0;
     if (bulk) {
-        constexpr uint32_t BYTES = uint32_t(sizeof(R)) * TE * (6 * N + EG + 4 * FGRT + GM + (SIP ? GA : 0));
+        constexpr uint32_t BYTES = uint32_t(sizeof(R)) * TE * (6 * N + EG + 4 * FGR + GM);
         // every box dimension within the copy's limit of 256, the byte count
         // within the mbarrier's transaction count (2^20 - 1)
         static_assert(!BULK_OK || (TE <= 256 && N <= 256 && BYTES < (1u << 20)), "bulk-copy boxes");
@@ -739,16 +591,16 @@ stage_kernel(const StageParams prm) {
             const int x = int(tile_index(prm.tile_groups)) * TE;
             bulk::load_3d(us, tm + prm.tm_u * TMAP_BYTES, x, 0, 0, tc_bar);
             bulk::load_2d(eg, tm + TM_GEO * TMAP_BYTES, x, 0, tc_bar);
-            bulk::load_3d(fg, tm + (SIP ? TM_FCS : TM_FC) * TMAP_BYTES, x, 0, 0, tc_bar);
-            bulk::load_2d(gm, tm + (SIP ? TM_GMGA : TM_GM) * TMAP_BYTES, x, 4 * FCF, tc_bar);
+            bulk::load_3d(fg, tm + TM_FC * TMAP_BYTES, x, 0, 0, tc_bar);
+            bulk::load_2d(gm, tm + TM_GM * TMAP_BYTES, x, 4 * FGR, tc_bar);
         }
         request_nbr(grp, code0, vn);
         request_nbr(grp + NG, code1, vn1);
     } else {
         // rows q: [0, 6N) coefficients, then EG element constants, 4 FGRT face
         // constants, GM metric rows and (penalty) GA rows of A^T
-        constexpr int Q0 = 6 * N, Q1 = Q0 + EG, Q2 = Q1 + 4 * FGRT, Q3 = Q2 + GM;
-        constexpr int T1 = Q3 + (SIP ? GA : 0);
+        constexpr int Q0 = 6 * N, Q1 = Q0 + EG, Q2 = Q1 + 4 * FGR, Q3 = Q2 + GM;
+        constexpr int T1 = Q3;
         constexpr int UR = (T1 + NG - 1) / NG;          // rows per thread (at most)
         constexpr int BATCH = UR < 24 ? UR : 16;        // loads in flight per thread (one batch when it fits)
         const R* fcp = static_cast<const R*>(prm.fcp);
@@ -759,18 +611,16 @@ stage_kernel(const StageParams prm) {
                 return active ? gr[IX(k) * K + e] : R(k == G_DET || k == G_EPS || k == G_MU ? 1 : 0);
             }
             if (q < Q2) {
-                const int f = (q - Q1) / FGRT, k = (q - Q1) % FGRT;
-                return active ? fcp[IX(f * FCF + k) * K + e] : R(0);
+                const int f = (q - Q1) / FGR, k = (q - Q1) % FGR;
+                return active ? fcp[IX(f * FGR + k) * K + e] : R(0);
             }
-            if (q < Q3) return active ? fcp[IX(4 * FCF + q - Q2) * K + e] : R(0);
-            return active ? fcp[IX(4 * FCF + GM + q - Q3) * K + e] : R(0);
+            return active ? fcp[IX(4 * FGR + q - Q2) * K + e] : R(0);
         };
         auto store = [&](int q, R v) {
             if (q < Q0) us[q * TE + c] = v;
             else if (q < Q1) eg[(q - Q0) * TE + c] = v;
             else if (q < Q2) fg[(q - Q1) * TE + c] = v;
-            else if (q < Q3) gm[(q - Q2) * TE + c] = v;
-            else ga[(q - Q3) * TE + c] = v;
+            else gm[(q - Q2) * TE + c] = v;
         };
         R tmp[BATCH];
 #pragma unroll
@@ -833,7 +683,7 @@ stage_kernel(const StageParams prm) {
                 request_nbr(ni + NG, nbs[((ni + NG) / 6) * TE + c], vnx);
             if (rr >= 1) nbr_trace(ni, ni < NNBR ? nbs[(ni / 6) * TE + c] : -1, vn);
             const int oi = grp + (rr - (ROUNDS - OWN_ROUNDS)) * NG;   // own item of this round
-            if (rr >= ROUNDS - OWN_ROUNDS && oi < NOWN && nbr_item_active(oi % 6)) {
+            if (rr >= ROUNDS - OWN_ROUNDS && oi < NOWN) {
                 const int ocomp = oi % 6, fp = oi / 6;
                 R v[N];
                 R acc[NF];
@@ -873,29 +723,11 @@ stage_kernel(const StageParams prm) {
             const int ch = it % CHUNKS;
             const int m0 = ch * NF / CHUNKS, m1 = (ch + 1) * NF / CHUNKS;
             const int32_t fcode = nbs[f * TE + c];
-            // interior penalty: this column's facet field on face f (and, on the
-            // owner side, its output and residual), [3][NF][facet][S]: mode-major,
-            // so that the facets of neighbouring columns sit side by side
-            const R* hsv = nullptr;
-            R *hso = nullptr, *hsr = nullptr;
-            const int64_t fs = int64_t(prm.n_facets) * S;
-            if (SIP && active) {
-                const int32_t sf = nbs[(4 + f) * TE + c];
-                if (sf >= 0) {
-                    const IX off = IX(sf >> 1) * S + s;
-                    hsv = static_cast<const R*>(prm.hs) + off;
-                    if (sf & 1) {
-                        hso = static_cast<R*>(prm.hs_out) + off;
-                        hsr = MODE == MODE_LSRK ? static_cast<R*>(prm.hs_res) + off : nullptr;
-                    }
-                }
-            }
-            const R ca = coef(prm.a, prm.a_f), cb = coef(prm.b, prm.b_f), dtc = coef(prm.dt, prm.dt_f);
             switch (f) {
-                case 0: flux_face<0, NF, R, TE, MODE, IX, SIP, (NF + CHUNKS - 1) / CHUNKS>(m0, m1, c, trO, trN, fg, gm, eg, jp, C, col, active, fcode, prm.inc, hsv, hso, hsr, fs, ga + c, ca, cb, dtc); break;
-                case 1: flux_face<1, NF, R, TE, MODE, IX, SIP, (NF + CHUNKS - 1) / CHUNKS>(m0, m1, c, trO, trN, fg, gm, eg, jp, C, col, active, fcode, prm.inc, hsv, hso, hsr, fs, ga + c, ca, cb, dtc); break;
-                case 2: flux_face<2, NF, R, TE, MODE, IX, SIP, (NF + CHUNKS - 1) / CHUNKS>(m0, m1, c, trO, trN, fg, gm, eg, jp, C, col, active, fcode, prm.inc, hsv, hso, hsr, fs, ga + c, ca, cb, dtc); break;
-                default: flux_face<3, NF, R, TE, MODE, IX, SIP, (NF + CHUNKS - 1) / CHUNKS>(m0, m1, c, trO, trN, fg, gm, eg, jp, C, col, active, fcode, prm.inc, hsv, hso, hsr, fs, ga + c, ca, cb, dtc); break;
+                case 0: flux_face<0, NF, R, TE, MODE, IX>(m0, m1, c, trO, trN, fg, gm, eg, jp, C, col, active, fcode, prm.inc); break;
+                case 1: flux_face<1, NF, R, TE, MODE, IX>(m0, m1, c, trO, trN, fg, gm, eg, jp, C, col, active, fcode, prm.inc); break;
+                case 2: flux_face<2, NF, R, TE, MODE, IX>(m0, m1, c, trO, trN, fg, gm, eg, jp, C, col, active, fcode, prm.inc); break;
+                default: flux_face<3, NF, R, TE, MODE, IX>(m0, m1, c, trO, trN, fg, gm, eg, jp, C, col, active, fcode, prm.inc); break;
             }
         }
     }
