@@ -260,11 +260,12 @@ int dgm_set_index64(dgm_plan* plan, int32_t force);
 int dgm_set_tile_loads(dgm_plan* plan, int32_t per_thread);
 int dgm_get_tile_loads(const dgm_plan* plan, int32_t* bulk);
 /* Order in which the stage and adjoint kernels visit their column tiles:
- * with groups = G > 1 (and a tile count that G divides) consecutive CTAs
- * take tiles from G equal segments of the columns in turn, which keeps the
+ * with groups = G > 1 consecutive CTAs take tiles from G (nearly) equal
+ * segments of the columns in turn, which keeps the
  * neighbours' coefficients of meshes numbered in G blocks (e.g. a Kuhn grid
  * numbered by tetrahedron type) in L2; 1 = plain order.  Results do not
- * depend on it.  dgm_autotune picks it after the tile shape: the fastest of
+ * depend on it.  A new plan takes the order that brings most face neighbours
+ * close together.  dgm_autotune picks it after the tile shape: the fastest of
  * 1, 2, 3, 4, 6, 8, 12, or 1 unless that is at least 1 % faster than the plain
  * order; DGM_EINVAL outside 1..64. */
 int dgm_set_tile_groups(dgm_plan* plan, int32_t groups);

@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -299,6 +300,44 @@ extern "C" {
 
 const char* dgm_last_error(void) { return g_err.c_str(); }
 
+// Tile visiting order of a new plan (tile_index in dgm_stage.cuh): the number of
+// segments under which the most face neighbours are visited within one wave of CTAs
+// of their element, and among equals the smallest.  us per FP32 stage, plain | chosen:
+// 24^3 Kuhn grid with a PML, p = 3, 8 columns 922 | 740, 16 columns 1665 | 1477; 32^3,
+// p = 3, one column 134 | 118.  The plain order stays where the gathers find their
+// neighbours in L2 in any order, fields of less than 64 MB (`gathered`: of a leapfrog
+// half step one field; 24^3 with a PML, one column, p = 3 90.8 | 92.0), and in FP64,
+// bound by its pipe (32^3, p = 3: 11.87 | 12.35 ms per step).
+// dgm_autotune and dgm_set_tile_groups replace it.
+static int choose_tile_groups(const HostMesh& m, int64_t S, int real_size, size_t gathered) {
+    constexpr int64_t TE = 32, WAVE = 608;   // columns per tile; CTAs of one wave (four per SM)
+    const int64_t K = m.K, n = (K * S + TE - 1) / TE;
+    if (n <= WAVE || real_size == 8 || gathered < (size_t(64) << 20)) return 1;
+    const int64_t step = std::max<int64_t>(1, K / 2000);   // a sample of the elements
+    int best = 1;
+    int64_t most = -1;
+    for (int g : {1, 2, 3, 4, 6, 8, 12}) {
+        const int64_t q = n / g, r = n % g, big = r * (q + 1);
+        auto place = [&](int64_t e) {   // of the tile of element e in the visiting order
+            const int64_t t = e * S / TE;
+            const int64_t seg = t < big ? t / (q + 1) : r + (t - big) / q;
+            const int64_t idx = t < big ? t % (q + 1) : (t - big) % q;
+            return idx * g + seg;
+        };
+        int64_t near = 0;
+        for (int64_t e = 0; e < K; e += step)
+            for (int f = 0; f < 4; ++f) {
+                const int32_t code = m.nbr[size_t(f) * size_t(K) + size_t(e)];
+                if (code >= 0 && std::abs(place(e) - place(code >> 2)) < WAVE) ++near;
+            }
+        if (near > most + most / 50) {   // (a tie or a gain within 2 % keeps the smaller)
+            most = near;
+            best = g;
+        }
+    }
+    return best;
+}
+
 static int plan_create(dgm_plan** out, int64_t nv, const double* xyz, int64_t nt, const int64_t* tets,
                        const double* eps, const double* mu, const dgm_pml* pml,
                        const dgm_options* opt, int mixed) {
@@ -438,6 +477,8 @@ static int plan_create(dgm_plan** out, int64_t nv, const double* xyz, int64_t nt
     off = align256(off + size_t(TMAP_SETS) * TMAP_COUNT * TMAP_BYTES);
     P->bytes_geom = off;
     P->k_active = K;
+    P->tile_groups = choose_tile_groups(P->mesh, opt->n_columns, kt->real_size,
+                                        size_t(opt->integrator == DGM_LEAPFROG ? 3 : 6) * P->N * K * Sc * kt->real_size);
     P->src_host.assign(size_t(Sc) * (SRC_HDR + 3 * P->N), 0.0);
     for (int s = 0; s < Sc; ++s) P->src_host[size_t(s) * (SRC_HDR + 3 * P->N)] = -1.0;
     *out = P;

@@ -51,17 +51,17 @@
 
 namespace dgm {
 
-// Tile visited by this CTA.  With G > 1 groups (and a grid that G divides)
-// CTAs b = 0, 1, 2, ... take tiles from G equal segments in turn, so that
+// Tile visited by this CTA.  With G > 1 groups CTAs b = 0, 1, 2, ... take tiles
+// from G nearly equal segments in turn (the first n % G hold one tile more), so that
 // tiles far apart in the column numbering run at the same time: meshes whose
 // neighbours are numbered in G blocks (a Kuhn grid numbered type by type has
 // its face neighbours in other type blocks) then find their neighbours'
-// coefficients in L2.  Any order gives the same results.
+// coefficients in L1 and L2.  Any order gives the same results.
 __device__ __forceinline__ unsigned tile_index(int groups) {
     const unsigned b = blockIdx.x, n = gridDim.x;
-    if (groups <= 1 || n % unsigned(groups) != 0) return b;
-    const unsigned g = unsigned(groups);
-    return (b % g) * (n / g) + b / g;
+    if (groups <= 1) return b;
+    const unsigned g = unsigned(groups), seg = b % g, rest = n % g;
+    return seg * (n / g) + (seg < rest ? seg : rest) + b / g;
 }
 
 // offset of the first mode of total degree d (3-D) and (2-D)
