@@ -317,6 +317,31 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
             const IX acol = IX(pi) * IX(prm.S) + id.s;
             auto load_aux = [&](const R* p, IX row) -> R { return p[row * C2 + acol]; };
             auto store_aux = [&](R* p, IX row, R v) { p[row * C2 + acol] = v; };
+            // The rows run in chunks whose loads are all requested before their
+            // arithmetic.  FP32 from p = 4 on the chunks share one loop body, the
+            // right-hand side rotating through the registers, because the code far
+            // exceeds the instruction cache (249 -> 221 KB; two steps of the 40^3 dipole
+            // at p = 4 9.79 -> 9.27 ms).  At p = 3 (130 -> 114 KB) the rotation costs more
+            // than the misses (24^3 batch, 16 columns: 21.0 -> 21.9 ms): unrolled, where
+            // the rotation is only a renaming.
+            constexpr int CH = sizeof(R) == 8 ? 2 : LF ? 4 : 3, NRP = round_up(NR, CH);
+            constexpr int UNROLL = P >= 4 && sizeof(R) == 4 ? 1 : NRP / CH;
+            R q0[NRP], q1[NRP], q2[NRP];
+#pragma unroll
+            for (int i = 0; i < NRP; ++i) {
+                q0[i] = i < NR ? a0[LO + (i < NR ? i : 0)] : R(0);
+                q1[i] = i < NR ? a1[LO + (i < NR ? i : 0)] : R(0);
+                q2[i] = i < NR ? a2[LO + (i < NR ? i : 0)] : R(0);
+            }
+            auto rotate = [&](R (&q)[NRP]) {
+                R t[CH];
+#pragma unroll
+                for (int i = 0; i < CH; ++i) t[i] = q[i];
+#pragma unroll
+                for (int i = 0; i + CH < NRP; ++i) q[i] = q[i + CH];
+#pragma unroll
+                for (int i = 0; i < CH; ++i) q[NRP - CH + i] = t[i];
+            };
             const IX ab = IX(r0 + LO);   // (both fields of degree P)
             if constexpr (LF) {
                 // Leapfrog with the PML terms by the trapezoid rule (Sec. V), X = A^-T x:
@@ -338,18 +363,16 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
                     za[a] = (R(1) - hs) * iz;
                     zb[a] = iz * dt * omat * xi[a];
                 }
-                // rows in chunks whose loads are all requested before their arithmetic
-                constexpr int CH = sizeof(R) == 8 ? 2 : 4;
-#pragma unroll
+#pragma unroll(UNROLL)
                 for (int i0 = 0; i0 < NR; i0 += CH) {
                     R av[CH][3], oa[CH][3];
 #pragma unroll
                     for (int i = 0; i < CH; ++i) {
-                        if (i0 + i >= NR) break;
+                        const bool ok = i0 + i < NR;
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
-                            av[i][k] = load_aux(auxl, ab + IX(k * N + i0 + i));
-                            oa[i][k] = load_aux(auxl, abo + IX(k * N + i0 + i));
+                            av[i][k] = ok ? load_aux(auxl, ab + IX(k * N + i0 + i)) : R(0);
+                            oa[i][k] = ok ? load_aux(auxl, abo + IX(k * N + i0 + i)) : R(0);
                         }
                     }
 #pragma unroll
@@ -367,7 +390,7 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
                             auto phys = [&](R p, R q, R r) {
                                 return fmaa(M[3 * a + 2], r, fmaa(M[3 * a + 1], q, M[3 * a] * p));
                             };
-                            const R y = fmaa(ndi, phys(av[i][0], av[i][1], av[i][2]), phys(a0[l], a1[l], a2[l]));
+                            const R y = fmaa(ndi, phys(av[i][0], av[i][1], av[i][2]), phys(q0[i], q1[i], q2[i]));
                             Xn[a] = fmaa(xx[a], phys(uv[0], uv[1], uv[2]), xy[a] * y);
                             Zn[a] = fmaa(za[a], phys(oa[i][0], oa[i][1], oa[i][2]), zb[a] * phys(ov[0], ov[1], ov[2]));
                         }
@@ -379,6 +402,9 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
                                       fmaa(AT[k][2], Zn[2], fmaa(AT[k][1], Zn[1], AT[k][0] * Zn[0])));
                         }
                     }
+                    rotate(q0);
+                    rotate(q1);
+                    rotate(q2);
                 }
                 return;
             } else {
@@ -400,18 +426,16 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
                         SIG[j][k] = nst * fmaa(w2, sg[2], fmaa(w1, sg[1], w0 * sg[0]));
                         XI[j][k] = st * mat * fmaa(w2, xi[2], fmaa(w1, xi[1], w0 * xi[0]));
                     }
-                // rows in chunks whose loads are all requested before their arithmetic
-                constexpr int CH = sizeof(R) == 8 ? 2 : 3;
-#pragma unroll
+#pragma unroll(UNROLL)
                 for (int i0 = 0; i0 < NR; i0 += CH) {
                     R av[CH][3], ar[CH][3];
 #pragma unroll
                     for (int i = 0; i < CH; ++i) {
-                        if (i0 + i >= NR) break;
+                        const bool ok = i0 + i < NR;
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
-                            av[i][k] = load_aux(aux, ab + IX(k * N + i0 + i));
-                            ar[i][k] = (MODE == MODE_LSRK && ca != R(0)) ? load_aux(auxi, ab + IX(k * N + i0 + i)) : R(0);
+                            av[i][k] = ok ? load_aux(aux, ab + IX(k * N + i0 + i)) : R(0);
+                            ar[i][k] = (MODE == MODE_LSRK && ok && ca != R(0)) ? load_aux(auxi, ab + IX(k * N + i0 + i)) : R(0);
                         }
                     }
 #pragma unroll
@@ -435,10 +459,19 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
                                 store_aux(auxo, row, fmaa(cb, rr, av[i][k]));
                             }
                         }
-                        a0[l] += d[0];
-                        a1[l] += d[1];
-                        a2[l] += d[2];
+                        q0[i] += d[0];
+                        q1[i] += d[1];
+                        q2[i] += d[2];
                     }
+                    rotate(q0);
+                    rotate(q1);
+                    rotate(q2);
+                }
+#pragma unroll
+                for (int i = 0; i < NR; ++i) {
+                    a0[LO + i] = q0[i];
+                    a1[LO + i] = q1[i];
+                    a2[LO + i] = q2[i];
                 }
             }
         }
