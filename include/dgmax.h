@@ -69,7 +69,11 @@ typedef struct {
     int32_t flux;       /* DGM_CENTRAL or DGM_UPWIND */
     int32_t integrator; /* DGM_LEAPFROG or DGM_LSRK4 */
     int32_t n_columns;  /* S >= 1 independent problems (sources) sharing the mesh */
-    int32_t max_receivers; /* capacity for dgm_set_receivers (0: none) */
+    int32_t max_receivers; /* capacity for dgm_set_receivers (0: none).  FP32 plans
+                            * without the interior penalty: above 0 the steps keep
+                            * one fixed rounding, to which records (FP64, formed
+                            * from FP32 fields) are reproducible; at 0 they run a
+                            * faster kernel of another rounding */
     double dt;          /* time step */
 } dgm_options;
 
@@ -148,7 +152,8 @@ int dgm_set_sources(dgm_plan* plan, int32_t n, const int32_t* column, const doub
 /* Receivers: points at which dgm_sample_receivers evaluates E.  n <= the
  * plan's max_receivers; pos: host [n][3].  Each point is located in the
  * lowest-index element containing it.  Requires a bound plan (uploads and
- * synchronises).  Errors: DGM_EINVAL (too many, or a point outside the mesh). */
+ * synchronises).  The steps do not depend on which receivers are set, or when.
+ * Errors: DGM_EINVAL (too many, or a point outside the mesh). */
 int dgm_set_receivers(dgm_plan* plan, int32_t n, const double* pos);
 
 /* Physical E at the receivers for every column, E(r) = A^-T sum_l u_l phi_l(r_hat)

@@ -764,8 +764,10 @@ static void stage_params(dgm_plan* P, StageParams& prm) {
     prm.n_facets = P->n_facets;
     prm.fcp = P->geom + P->off_fcp;
     prm.fct = P->geom + P->off_fct;
-    // (the penalty runs in tang_kernel only, receivers or not)
-    prm.recorded = P->kt->real_size == 4 && P->n_rec > 0 && !(P->sip_alpha > 0.0);
+    // by what the plan was created for, not by the receivers set now: the rounding of a
+    // run, a captured batch and a tuned shape do not depend on when they are set
+    // (the penalty runs in tang_kernel only)
+    prm.recorded = P->kt->real_size == 4 && P->opt.max_receivers > 0 && !(P->sip_alpha > 0.0);
     if (P->tmaps_ok && P->tile_loads == 0) {   // phase-1 bulk copies (the launchers pick the map)
         prm.tmaps = P->geom + P->off_tmap;
         prm.tm_f0 = P->fields[0];

@@ -104,7 +104,7 @@ struct StageParams {
     void* raw;            // MODE_RAW: right-hand side before the mass inverse [6][N][K][S]
     void* jumps;          // MODE_RAW: physical face jumps dE, dH [4][6][NF][K][S]
     int32_t variant;      // tile-shape variant of the LSRK stage kernel (autotuner)
-    int32_t recorded;     // FP32 plan with receivers, no penalty: stage_kernel (its rounding), not tang_kernel
+    int32_t recorded;     // FP32 plan for receivers, no penalty: stage_kernel (its rounding), not tang_kernel
     int32_t force_index64;// 1: 64-bit index arithmetic even where 32 bits suffice
     int32_t tile_groups;  // tile visiting order: G interleaved segments (1: in order)
     const void* tc_b;     // tensor-core variant: B operand image (TcShape<P>::B_BYTES), or null

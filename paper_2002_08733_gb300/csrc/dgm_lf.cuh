@@ -1,4 +1,4 @@
-// Leapfrog half step of FP32 plans with receivers, on reference-frame traces.
+// Leapfrog half step of FP32 plans for receivers, on reference-frame traces.
 //
 // Those plans keep the rounding of stage_kernel (dgm_stage.cuh): receiver
 // records are FP64 results formed from FP32 fields.  So every value here is the

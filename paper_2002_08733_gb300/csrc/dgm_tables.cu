@@ -7,10 +7,11 @@
 // packed FP32x2 arithmetic, 4 = paired kernel with scalar arithmetic; at p = 2, 3
 // also 5 = tensor-core variant (64 columns x 512 threads, curl and lift on tcgen05).
 //
-// FP32 plans with receivers and without the penalty (prm.recorded) run stage_kernel
-// (dgm_stage.cuh) in the LSRK mode and lf_kernel (dgm_lf.cuh) in the leapfrog modes: receiver records and the adjoint's gradients are
-// FP64 results formed from FP32 fields, and what was recorded before stays
-// reproducible to FP64 accuracy only if the fields keep their rounding.  Its
+// FP32 plans created for receivers (max_receivers > 0) and without the penalty
+// (prm.recorded) run stage_kernel (dgm_stage.cuh) in the LSRK mode and lf_kernel
+// (dgm_lf.cuh) in the leapfrog modes: receiver records and the adjoint's gradients
+// are FP64 results formed from FP32 fields, and what was recorded before stays
+// reproducible to FP64 accuracy only if the fields keep their rounding.  stage_kernel's
 // variants: 0 = 32 columns x 384 threads, 1 = 32 x 192, 2 = 16 x 192, p >= 4:
 // 3 = 32 x 512.
 #include "dgm_internal.h"

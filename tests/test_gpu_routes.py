@@ -80,3 +80,95 @@ def test_penalty_plan_with_receivers_matches_oracle(D, p):
         for s in range(2):
             want[s, r] = plain.evaluate(got[T, s, 0:3].reshape(-1), T, x[None, :])[0]
     assert rel_err(rec, want) < 1e-6
+
+
+# -- the kernel is the plan's, not the receivers' ----------------------------------------
+
+PML = dict(lo=(-0.4,) * 3, hi=(0.4,) * 3, thickness=0.6, sigma_max=15.0, order=2)
+
+
+def _plan(D, n, p, integrator="lsrk4", flux="upwind", S=1, pml=True, max_receivers=1, prec="fp32", src=True,
+          nseed=0):
+    xyz, tets = W.kuhn_mesh(n, (-1, -1, -1), (1, 1, 1), jitter=0.1, seed=310 + n + nseed)
+    K = len(tets)
+    eps = W.lognormal_material(K, 1.5, 0.2, 311)
+    mu = W.lognormal_material(K, 1.0, 0.1, 312)
+    g = D.Solver(xyz, tets, eps, mu, p, prec, flux, integrator, W.stable_dt(2.0 / n, p) / 2, S=S,
+                 pml=PML if pml else None, max_receivers=max_receivers)
+    if src:
+        g.set_sources([W.dipole((0.11, -0.07, 0.05), 2.0, 0.2)] + [None] * (S - 1))
+    u = W.random_state(K, S, p, seed=313) * 1e-2
+    if g.npml:
+        g.set_state(u, (W.random_state(K, S, p, seed=314) * 1e-3)[g.pml_elements()])
+    else:
+        g.set_state(u)
+    if integrator == "leapfrog":
+        g.leapfrog_start(0.0)
+    return g
+
+
+def _result(g):
+    return g.state(), g.from_device(g.aux[g.current()]) if g.npml else np.zeros(1)
+
+
+def _same(a, b):
+    return all(np.array_equal(x, y) for x, y in zip(_result(a), _result(b)))
+
+
+POINT = np.array([[0.1, 0.2, -0.1]])
+
+
+@pytest.mark.parametrize("integrator,flux", [("lsrk4", "upwind"), ("leapfrog", "central")])
+@pytest.mark.parametrize("p", [2, 4])
+def test_setting_receivers_changes_no_bit_of_the_fields(D, p, integrator, flux):
+    a = _plan(D, 3, p, integrator, flux)
+    b = _plan(D, 3, p, integrator, flux)
+    b.set_receivers(POINT)
+    a.advance(2, 0.0)
+    b.advance(2, 0.0)
+    assert _same(a, b)
+    a.set_receivers(POINT)          # in the middle of a run
+    for g in (a, b):
+        g.advance(1, 2 * g.dt)
+    assert _same(a, b)
+
+
+@pytest.mark.parametrize("p", [2, 4])
+def test_batch_captured_before_the_receivers_are_set(D, p):
+    """The graph's two steps and the odd third step run the same kernel."""
+    import torch
+    a = _plan(D, 3, p, src=False)
+    b = _plan(D, 3, p, src=False)
+    batch = D.Batch([a])
+    a.set_receivers(POINT)
+    batch.advance(3)
+    torch.cuda.synchronize()
+    b.set_receivers(POINT)
+    b.advance(3, 0.0)
+    assert _same(a, b)
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("n,S,pml", [(1, 1, False), (2, 2, True), (2, 3, False), (3, 1, True), (4, 1, False)])
+@pytest.mark.parametrize("integrator,flux", [("leapfrog", "central"), ("lsrk4", "upwind")])
+def test_plans_for_receivers_agree_with_plans_without(D, p, n, S, pml, integrator, flux):
+    """The two kernels on one problem: to twice the FP32 tolerance of one of them against
+    the oracle (1e-5 of the max-norm)."""
+    r = []
+    for cap in (0, 1):
+        g = _plan(D, n, p, integrator, flux, S, pml, cap)
+        g.advance(3, 0.0)
+        g.status()
+        r.append(_result(g))
+    assert rel_err(r[0][0], r[1][0]) < 2e-5
+    assert not pml or rel_err(r[0][1], r[1][1]) < 2e-5
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("integrator,flux", [("leapfrog", "central"), ("lsrk4", "upwind")])
+def test_plans_without_receivers_64_bit_indices(D, p, integrator, flux):
+    a, b = (_plan(D, 2, p, integrator, flux, 3, True, 0) for _ in range(2))
+    b.set_index64()
+    for g in (a, b):
+        g.advance(2, 0.0)
+    assert _same(a, b)
