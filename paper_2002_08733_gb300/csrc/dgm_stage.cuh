@@ -746,7 +746,7 @@ stage_kernel(const StageParams prm) {
         const int fb = (grp / NP5) * 3, part = grp % NP5;
         const int lo = part * N / NP5, hi = (part + 1) * N / NP5;
         const bool load = active && coef(prm.a, prm.a_f) != R(0);
-        const R* __restrict__ res = static_cast<const R*>(prm.res);
+        const R* res = static_cast<const R*>(prm.res);
 #pragma unroll
         for (int k = 0; k < 3; ++k)
 #pragma unroll
@@ -982,10 +982,10 @@ stage_kernel(const StageParams prm) {
         const IX C2 = IX(prm.npml) * S;
         const IX acol = IX(pi) * S + s;
         R* uo = static_cast<R*>(prm.u_out);
-        R* __restrict__ res = static_cast<R*>(prm.res);
-        const R* __restrict__ aux = static_cast<const R*>(prm.aux);
-        R* __restrict__ auxo = static_cast<R*>(prm.aux_out);
-        R* __restrict__ auxr = static_cast<R*>(prm.aux_res);
+        R* res = static_cast<R*>(prm.res);
+        const R* aux = static_cast<const R*>(prm.aux);
+        R* auxo = static_cast<R*>(prm.aux_out);
+        R* auxr = static_cast<R*>(prm.aux_res);
         const R dt = coef(prm.dt, prm.dt_f), ca = coef(prm.a, prm.a_f), cb = coef(prm.b, prm.b_f);
         const int lo = part * N / NP5, hi = (part + 1) * N / NP5;
         const IX gb = IX(fb * N + lo) * C + col;          // (fb, lo) in the fields

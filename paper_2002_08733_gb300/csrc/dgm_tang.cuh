@@ -228,7 +228,7 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
     const bool active = id.active;
     const R ca = coef(prm.a, prm.a_f), cb = coef(prm.b, prm.b_f), dt = coef(prm.dt, prm.dt_f);
     const IX gb = IX(r0 + LO) * C + id.col;
-    const R* __restrict__ resi = static_cast<const R*>(prm.res);
+    const R* resi = static_cast<const R*>(prm.res);   // written below, by the same thread after it has read
     const bool ld = active && ca != R(0);
     R rv[EARLY ? NR : 1][3];
     if constexpr (EARLY) {
@@ -277,7 +277,7 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
             }
         }
     }
-    R* __restrict__ res = static_cast<R*>(prm.res);
+    R* res = static_cast<R*>(prm.res);
     R* uo = static_cast<R*>(prm.u_out);
     // the mass block; outside the right-hand-side mode scaled by the step
     const R sc = MODE == MODE_RHS ? im : im * dt;
@@ -409,8 +409,8 @@ __device__ __forceinline__ void tang_rows(const StageParams& prm, int F, const R
                 return;
             } else {
                 // (an auxiliary residual row is read before it is written, by the same thread)
-                const R* __restrict__ aux = static_cast<const R*>(prm.aux);
-                const R* __restrict__ auxi = static_cast<const R*>(prm.aux_res);
+                const R* aux = static_cast<const R*>(prm.aux);
+                const R* auxi = static_cast<const R*>(prm.aux_res);
                 R* auxo = static_cast<R*>(prm.aux_out);
                 R* auxr = static_cast<R*>(prm.aux_res);
                 // -eta, -Sigma, mat xi and -1/mat, times the step outside the right-hand-side mode
