@@ -152,11 +152,11 @@ int launch_mode(const StageParams& prm, cudaStream_t st) {
                                                : launch_lf_ix<MODE, int64_t>(q, grid, st);
 }
 #else
-template <typename IX>
+template <typename IX, bool PML>
 int launch_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
     constexpr size_t smem = stage_smem_bytes<kP, Real, kTE, kTC>();
     static bool configured = false;
-    auto k = stage_kernel<kP, Real, kTE, kNT, DGM_MODE, IX, kTC>;
+    auto k = stage_kernel<kP, Real, kTE, kNT, DGM_MODE, IX, kTC, PML>;
     if (kTC && q.tc_b == nullptr) return DGM_EUNSUP;   // no operator image for this plan
     if (!configured) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
@@ -199,7 +199,11 @@ int launch_mode(const StageParams& prm, cudaStream_t st) {
                  : (q.tm_fw != nullptr && q.u == q.tm_fw) ? TM_UW : -1;
     }
     if (q.hs != nullptr) return DGM_EUNSUP;   // the interior penalty: tang_kernel only
-    return i32 ? launch_ix<uint32_t>(q, grid, st) : launch_ix<int64_t>(q, grid, st);
+    // (64-bit indices, and the tensor-core variant: with the layer's terms)
+    if constexpr (DGM_MODE == MODE_LSRK && !kTC) {
+        if (i32 && q.pml == nullptr) return launch_ix<uint32_t, false>(q, grid, st);
+    }
+    return i32 ? launch_ix<uint32_t, true>(q, grid, st) : launch_ix<int64_t, true>(q, grid, st);
 }
 #endif
 

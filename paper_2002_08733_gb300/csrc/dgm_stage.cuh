@@ -474,7 +474,10 @@ __device__ __forceinline__ void rhs_part(int part, int comp, int c, const R* us,
 // tensor cores (dgm_tc.cuh, TcShape), with tensor-memory row (field, column);
 // phase 5 reads the pre-mass right-hand side from tensor memory.  The other
 // phases are shared with the SIMT kernel.
-template <int P, typename R, int TE, int NT, int MODE, typename IX = int64_t, bool TC = false>
+// PML: phase 5 has the layer's terms.  An instantiation without them serves the plans
+// without a layer, whose phase 5 the layer's chunked rows slow down (FP32 LSRK4 stage, us,
+// 16^3 grid, without the terms | with: p = 4 53.6 | 57.7; p = 5 135 | 150).
+template <int P, typename R, int TE, int NT, int MODE, typename IX = int64_t, bool TC = false, bool PML = true>
 __global__ void __launch_bounds__(NT, TC ? 1 : ((sizeof(R) == 8 || P <= 3) ? 2 : 1))
 stage_kernel(const StageParams prm) {
     static_assert(MODE == MODE_LSRK || MODE == MODE_RAW, "LSRK4 stages and the adjoint's forward quantities");
@@ -937,10 +940,10 @@ stage_kernel(const StageParams prm) {
             }
         // PML: (A^T D A^-T)[j][k] = sum_a A^T[j][a] D_a A^-T[a][k] for D = eta, Sigma, xi
         int32_t pi = -1;
-        if (prm.pml != nullptr) pi = prm.pml[e];
+        if (PML && prm.pml != nullptr) pi = prm.pml[e];
         R ETA[3][3], SIG[3][3], XI[3][3];
         R ait[9], AT[3][3], sg3[3], et3[3], xi3[3];   // PML: A^-T, A^T, sigma, eta, xi
-        if (pi >= 0) {
+        if (PML && pi >= 0) {
 #pragma unroll
             for (int k = 0; k < 9; ++k) ait[k] = eg[(G_AIT + k) * TE + c];
             // A^T = adj(A^-T) det A
@@ -1001,7 +1004,7 @@ stage_kernel(const StageParams prm) {
             for (int i = 0; i < CR; ++i)
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                    const bool ok = pi >= 0 && i0 + i < RP5 && (P5_EVEN || lo + i0 + i < hi);
+                    const bool ok = PML && pi >= 0 && i0 + i < RP5 && (P5_EVEN || lo + i0 + i < hi);
                     const IX aj = ab + IX(k * N + i0 + i) * C2;
                     av[i][k] = ok ? aux[aj] : R(0);
                     ar[i][k] = ok && ca != R(0) ? auxr[aj] : R(0);
@@ -1018,7 +1021,7 @@ stage_kernel(const StageParams prm) {
                 }
 #pragma unroll
                 for (int k = 0; k < 3; ++k) du[k] = B[k][0] * r[0] + B[k][1] * r[1] + B[k][2] * r[2];
-                if (pi >= 0) {
+                if (PML && pi >= 0) {
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         du[k] -= ETA[k][0] * uv[0] + ETA[k][1] * uv[1] + ETA[k][2] * uv[2] + av[i][k] * imat;

@@ -172,3 +172,15 @@ def test_plans_without_receivers_64_bit_indices(D, p, integrator, flux):
     for g in (a, b):
         g.advance(2, 0.0)
     assert _same(a, b)
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("n,S", [(1, 1), (2, 3), (3, 1)])
+def test_plans_for_receivers_without_a_layer(D, p, n, S):
+    """LSRK4 stages of plans without a PML have an instantiation of their own; the 64-bit one
+    serves both: the same bits."""
+    a, b = (_plan(D, n, p, "lsrk4", "upwind", S, False, 1) for _ in range(2))
+    b.set_index64()
+    for g in (a, b):
+        g.advance(2, 0.0)
+    assert _same(a, b)
