@@ -137,15 +137,15 @@ int launch_t_m4_f64_rhs(const StageParams&, void*);
 
 namespace {
 
-// No more tiles of 32 columns than SMs: a CTA has its SM to itself, and eight
-// threads per column fill it better than four, which win once several CTAs share
-// it.  us per FP32 LSRK4 stage, four | eight threads: 137 tiles p = 1 3.99 | 3.28,
-// p = 2 5.10 | 4.71 (PML 9.05 | 7.35), p = 3 9.26 | 7.86, p = 4 19.7 | 15.3; 324
-// tiles p = 1 4.06 | 4.24, p = 2 5.40 | 5.51, p = 4 19.0 | 23.9.  (The penalty and
-// p = 5 always run eight.)
-bool few_tiles(const StageParams& prm) {
+// FP32 LSRK4 stages of few tiles of 32 columns.  No more of them than SMs (p = 4: than two
+// per SM): the CTAs run side by side, and eight threads per column fill the SMs better than
+// four, which win once more CTAs queue.  us per stage, four | eight threads: 137 tiles p = 1
+// 3.99 | 3.28, p = 2 5.10 | 4.71 (PML 9.05 | 7.35), p = 3 9.26 | 7.86, p = 4 19.7 | 15.3;
+// 274 tiles p = 4 20.0 | 17.0 (PML 27.6 | 23.1); 324 tiles p = 1 4.06 | 4.24, p = 2
+// 5.40 | 5.51, p = 4 19.0 | 23.9.  (The penalty and p = 5 always run eight.)
+bool few_tiles(const StageParams& prm, int per_sm = 1) {
     constexpr int64_t kSMs = 152;
-    return prm.hs == nullptr && (prm.K_active * prm.S + 31) / 32 <= kSMs;
+    return prm.hs == nullptr && (prm.K_active * prm.S + 31) / 32 <= per_sm * kSMs;
 }
 
 int launch_p1_f32(const StageParams& prm, int mode, void* st) {
@@ -260,7 +260,7 @@ int launch_p4_f32(const StageParams& prm, int mode, void* st) {
                 case 3: return rec ? launch_p4_f32_lsrk_v3(prm, st) : launch_t_p4_f32_lsrk_v3(prm, st);
                 default:
                     return rec              ? launch_p4_f32_lsrk(prm, st)
-                           : few_tiles(prm) ? launch_t_p4_f32_lsrk_v3(prm, st)
+                           : few_tiles(prm, 2) ? launch_t_p4_f32_lsrk_v3(prm, st)
                                             : launch_t_p4_f32_lsrk(prm, st);
             }
         case MODE_LF_E: return rec ? launch_p4_f32_lfe(prm, st) : launch_t_p4_f32_lf(prm, st);

@@ -27,12 +27,14 @@ struct Shape {
 #else
     // FP32: four threads per column while a thread's rows (half of them) and a
     // trace's coefficients fit its registers, eight from p = 5 on, and at p = 4
-    // with the PML's matrices or the penalty's facet values besides.
+    // with the penalty's facet values besides.  (p = 4 with a PML, LSRK4, us, eight
+    // threads on 80 registers | four on 168: 250 tiles of 32 columns 47.4 | 27.9, 768 tiles
+    // 118 | 62.7; right-hand side of 999 tiles 110 | 64.7)
     // FP64 (bound by the FP64 pipe, which few warps saturate): full warps of 32
     // columns, so that no warp runs two faces or row parts in turn.
     static constexpr int TE = 32;
     static constexpr int NG = kLF ? (kF64 ? 4 : kP <= 4 ? 4 : 8)
-                                  : kF64 || SIP || kP == 5 || (kP == 4 && PML) ? 8 : 4;
+                                  : kF64 || SIP || kP == 5 ? 8 : 4;
     static constexpr int MINB =
         kF64 ? (kLF ? (kP <= 3 ? 2 : 1) : kP <= 3 ? 2 : 1)
         : SIP ? (kP <= 3 ? 3 : 2)
