@@ -607,13 +607,34 @@ __global__ void __launch_bounds__(CL > 1 ? TE * CLW : TE * NG, MINB) tang_kernel
 
     // The tile: one bulk tensor copy of its rows where the plan has a
     // map of u (aligned rows), issued first and waited for by thread 0; columns
-    // past the end arrive as zeros.  Otherwise every thread loads its rows.
+    // past the end arrive as zeros.
     const bool bulk = CL == 1 && prm.tm_u >= 0 && (tc::smem_addr(smem_raw) & 127u) == 0;
     if (bulk && threadIdx.x == 0) {
         static_assert(sizeof(R) * TE * ROWS < (1u << 20), "bytes of an mbarrier phase");
         tc::mbar_init(bar, 1);
         bulk::arrive_expect_tx(bar, uint32_t(sizeof(R)) * TE * ROWS);
         bulk::load_3d(us, static_cast<const char*>(prm.tmaps) + prm.tm_u * TMAP_BYTES, int(x0), 0, 0, bar);
+    }
+    // Otherwise every thread loads its rows: by asynchronous copies, all in flight at once,
+    // in a cluster (whose CTAs all take the whole tile) and in the shapes of few tiles, else
+    // in batches through registers, which follow one another, each a round trip, but
+    // leave the L1 to the gathers (us, batches | copies: right-hand side p = 4, 16 tiles
+    // 16.7 | 12.8; LSRK4 p = 5, 768 tiles in random order 203 | 222).  One of the two per
+    // instantiation: the choice at run time cost the p = 3 kernel 7 percent.
+    constexpr bool ASYNC = CL > 1 || (sizeof(R) == 4 && NG == 8 && TE == 32 && MINB <= 2 &&
+                                      (MINB == 1 || P == 3 || (P == 4 && !SIP)));
+    if (ASYNC && !bulk) {
+        constexpr int STEP = CL > 1 ? CLW : NG;
+        const int r0 = CL > 1 ? sub : grp;
+        if (active) {
+            const R* src = u + (IX(r0) * C + id.col);
+            uint32_t dst = tc::smem_addr(us + r0 * TE + c);
+#pragma unroll 8
+            for (int q = r0; q < ROWS; q += STEP, src += IX(STEP) * C, dst += STEP * TE * uint32_t(sizeof(R)))
+                asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" :: "r"(dst), "l"(src), "n"(sizeof(R)) : "memory");
+        } else {
+            for (int q = r0; q < ROWS; q += STEP) us[q * TE + c] = R(0);
+        }
     }
     // ---- phase A: jumps and fluxes of one face -----------------------------------
     const bool bad = code >= 0 && IX(code >> 2) >= K;
@@ -625,8 +646,11 @@ __global__ void __launch_bounds__(CL > 1 ? TE * CLW : TE * NG, MINB) tang_kernel
     constexpr int QF = MODE == MODE_LF_E ? 2 : 0;              // leapfrog: only the other field's jumps
     constexpr int QN = LF ? (NG == 4 ? 2 : 1) : (NG == 4 ? 4 : 2);
     const int q0 = QF + (NG == 4 ? 0 : half * QN);
-    constexpr bool AHEAD = P <= 3 || (P == 4 && PML);   // gathers of a slanted neighbour face in two register sets
-    R vn[N], vm[AHEAD ? N : 1];
+    // ALL: registers for the gathers of both items at once, one round trip instead of two
+    // to four (a slanted neighbour face's component 0 serves both)
+    constexpr bool ALL = sizeof(R) == 4 && NG == 8 && TE == 32 && MINB == 1;
+    constexpr bool AHEAD = ALL || P <= 3 || (P == 4 && PML);   // gathers of a slanted neighbour face in two register sets
+    R vn[N], vm[AHEAD ? N : 1], vx[ALL && QN == 2 ? N : 1];
     // first field row of component `comp` of a field
     auto row_of = [&](int fld, int comp) { return fld == 0 ? comp * N : 3 * N + comp * NH; };
     auto fetch = [&](int fld, int comp, R* v) {   // the neighbour's coefficients of one component
@@ -647,6 +671,9 @@ __global__ void __launch_bounds__(CL > 1 ? TE * CLW : TE * NG, MINB) tang_kernel
         }
     };
     gather(q0);
+    if constexpr (ALL && QN == 2) {
+        if (has) fetch(q0 >> 1, tang_comp(nf, 1), vx);
+    }
     if (bulk) {
         bool ok = true;
         if (threadIdx.x == 0) ok = tc::mbar_wait(bar, 0, 500000000ull);
@@ -660,19 +687,10 @@ __global__ void __launch_bounds__(CL > 1 ? TE * CLW : TE * NG, MINB) tang_kernel
             }
             return;
         }
-    } else if constexpr (CL > 1) {
-        // every CTA of the cluster holds the tile; asynchronous copies, all in flight
-        if (active) {
-#pragma unroll 4
-            for (int q = sub; q < ROWS; q += CLW)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;"
-                             :: "r"(tc::smem_addr(us + q * TE + c)), "l"(u + (IX(q) * C + id.col)) : "memory");
-            asm volatile("cp.async.wait_all;" ::: "memory");
-        } else {
-            for (int q = sub; q < ROWS; q += CLW) us[q * TE + c] = R(0);
-        }
+    } else if constexpr (ASYNC) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        if constexpr (CL > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     } else {
         constexpr int UR = (ROWS + NG - 1) / NG, BATCH = UR < 16 ? UR : 16;
 #pragma unroll 1
@@ -767,7 +785,12 @@ __global__ void __launch_bounds__(CL > 1 ? TE * CLW : TE * NG, MINB) tang_kernel
         } else {
             quarter(std::integral_constant<int, 0>{});
         }
-        if (k + 1 < QN) gather(q + 1);
+        if constexpr (ALL && QN == 2) {
+#pragma unroll
+            for (int l = 0; l < N; ++l) vn[l] = vx[l];
+        } else {
+            if (k + 1 < QN) gather(q + 1);
+        }
     }
     if constexpr (!LF) {
         // fluxes in place; with NG = 8 the face's two threads split the modes
@@ -877,13 +900,14 @@ __global__ void __launch_bounds__(CL > 1 ? TE * CLW : TE * NG, MINB) tang_kernel
 
     // ---- phase B: curl, lift, mass block, update ----------------------------------
     if constexpr (LF) {
-        // one field; NG = 8 would need eight row parts, its second half idles
+        // one field.  At p = 5 (eight groups) eight row parts with a layer, four without one,
+        // half of the groups idle: of eight every one repeats the curl's reads of the
+        // tile (us per half step, four | eight parts: 137 tiles with a PML 41.4 | 37.5; 999 tiles
+        // without 87 | 92).
         constexpr int F = MODE == MODE_LF_E ? 0 : 1;
-        if constexpr (CL > 1) {
-            constexpr int NPB = N < 16 ? N : 16;
-            if (const int part = sub * CL + grp; part < NPB)
-                tang_part<P, R, TE, MODE, IX, PML, MX, NPB>(prm, F, part, us + c, gs + c, id);
-        } else if (grp < 4) tang_part<P, R, TE, MODE, IX, PML, MX, 4>(prm, F, grp, us + c, gs + c, id);
+        constexpr int G = CL > 1 ? 16 : P == 5 && !PML ? 4 : NG, NPB = N < G ? N : G;
+        if (const int part = CL > 1 ? sub * CL + grp : grp; part < NPB)
+            tang_part<P, R, TE, MODE, IX, PML, MX, NPB>(prm, F, part, us + c, gs + c, id);
     } else if constexpr (CL > 1) {
         constexpr int NPB = N < 16 ? N : 16;
         if (const int part = sub * 4 + (grp >> 1); part < NPB)

@@ -43,35 +43,49 @@ struct Shape {
 #endif
 };
 
-// the interior penalty runs in the default shape
 #ifdef DGM_MIXED
 constexpr bool kMX = true;   // E of degree kP, H of degree kP - 1
 #else
 constexpr bool kMX = false;
 #endif
-#if !defined(DGM_TE) && !defined(DGM_MIXED)
-constexpr bool kSIP = true;
+// not an autotuner variant: all modes, the interior penalty, the rules for few tiles
+#ifdef DGM_TE
+constexpr bool kDefault = false;
 #else
-constexpr bool kSIP = false;
+constexpr bool kDefault = true;
 #endif
 
-// Most tiles (of 32 columns) for which the cluster form is taken: two of its CTAs per
-// SM (8 x 38 = 2 x 152; three would wait for one another's FP64 pipes).
-constexpr unsigned kClusterTiles = 38;
+// the tensor map of this stage's input for the tile's bulk copy (TmapIndex), or -1
+int tile_map(const StageParams& q) {
+    if (q.tmaps == nullptr) return -1;
+    return q.u == q.tm_f0 ? TM_U0 : q.u == q.tm_f1 ? TM_U1 : (q.tm_fw != nullptr && q.u == q.tm_fw) ? TM_UW : -1;
+}
 
-template <int MODE, typename IX, bool SIP, bool PML>
-int launch_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
-    using Sh = Shape<MODE, SIP, PML>;
-    constexpr size_t smem = tang_smem_bytes<kP, Real, Sh::TE, kMX>();
+template <int TE, int NG, int MODE, typename IX, bool SIP, bool PML, int MINB, int CL = 1>
+int launch_shape(StageParams& q, int64_t columns, cudaStream_t st) {
+    constexpr size_t smem = tang_smem_bytes<kP, Real, TE, kMX>();
     static bool configured = false;
-    auto k = tang_kernel<kP, Real, Sh::TE, Sh::NG, MODE, IX, SIP, PML, kMX, Sh::MINB>;
+    auto k = tang_kernel<kP, Real, TE, NG, MODE, IX, SIP, PML, kMX, MINB, CL>;
     if (!configured) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
             cudaSuccess)
             return DGM_ECUDA;
         configured = true;
     }
-    return launch_ex(k, grid, Sh::TE * Sh::NG, smem, st, q.pdl != 0, 1, q) == cudaSuccess ? DGM_OK : DGM_ECUDA;
+    // the plan's tensor-map set of this tile width
+    constexpr int kSet = TE == tmap_columns(0) ? 0 : 1;
+    static_assert(TE == tmap_columns(kSet), "a tensor-map set of this tile width");
+    q.tm_u = tile_map(q);
+    if (q.tm_u >= 0) q.tmaps = static_cast<const char*>(q.tmaps) + size_t(kSet) * TMAP_COUNT * TMAP_BYTES;
+    const unsigned tiles = unsigned((columns + TE - 1) / TE);
+    return launch_ex(k, CL * tiles, CL > 1 ? TE * CLW : TE * NG, smem, st, q.pdl != 0, CL, q) == cudaSuccess
+               ? DGM_OK : DGM_ECUDA;
+}
+
+template <int MODE, typename IX, bool SIP, bool PML>
+int launch_ix(StageParams& q, int64_t columns, cudaStream_t st) {
+    using Sh = Shape<MODE, SIP, PML>;
+    return launch_shape<Sh::TE, Sh::NG, MODE, IX, SIP, PML, Sh::MINB>(q, columns, st);
 }
 
 // true when every index the kernel forms for this plan is below 2^32: field
@@ -85,62 +99,81 @@ bool fits_32bit(const StageParams& p) {
            uint64_t(G_COUNT) * K < lim && uint64_t(TG_ROWS) * K < lim && 12 * NF * K < lim;
 }
 
-// FP64 meshes of few tiles: a cluster of eight CTAs per tile (see tang_kernel).
-// With a tile per CTA the launch takes as long as one SM's FP64 pipe needs for one
-// tile, however few there are; a cluster spreads a tile over eight SMs.  us per launch
-// of 12 tiles, one CTA | cluster: leapfrog p = 2 15.1 | 7.0; with clusters of
-// one-warp CTAs p = 3 37 | 23, LSRK4 p = 4 140 | 90, and from 65 tiles on no gain.
-template <int MODE>
-int launch_cluster(const StageParams& q, unsigned tiles, cudaStream_t st) {
-    constexpr size_t smem = tang_smem_bytes<kP, Real, 32, false>();
-    static bool configured = false;
-    auto k = tang_kernel<kP, Real, 32, 8, MODE, uint32_t, false, true, false, 1, 8>;
-    if (!configured) {
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
-            return DGM_ECUDA;
-        configured = true;
-    }
-    return launch_ex(k, 8 * tiles, 32 * CLW, smem, st, q.pdl != 0, 8, q) == cudaSuccess ? DGM_OK : DGM_ECUDA;
-}
+// Rules for few tiles (of 32 columns; one CTA of the ordinary shape works on each).
+//
+// FP64.  The launch takes as long as one SM's FP64 pipe needs for one tile, however few
+// there are.  LSRK4 and leapfrog up to kClusterTiles: a cluster of eight CTAs spreads a tile
+// over eight SMs (see tang_kernel; two of its CTAs per SM, 8 x 38 = 2 x 152; three would
+// wait for one another's FP64 pipes).  us per launch of 12 tiles, one CTA | cluster: leapfrog
+// p = 2 15.1 | 7.0; with clusters of one-warp CTAs p = 3 37 | 23, LSRK4 p = 4 140 | 90.
+// LSRK4 beyond and right-hand sides, up to kHalfTiles: tiles of 16 columns, which still find
+// an SM each.  65 tiles, 32 columns | 16: LSRK4 p = 1 10.0 | 7.3, with a PML 25.9 | 16.1, p = 4
+// with a PML 178 | 111; right-hand side p = 1 with a PML 25.2 | 16.7.  At 94 tiles 9.9 | 9.9
+// and 178 | 223.
+//
+// FP32 right-hand sides: eight threads per column instead of four while their CTAs run side
+// by side, at p = 3 up to one tile per SM, at p = 4 up to two (us, four | eight: p = 3 41 tiles
+// 8.8 | 8.2, 137 tiles 10.6 | 9.1, 375 tiles 10.9 | 15.5; p = 4 41 tiles 13.0 | 10.9, 137 tiles
+// 16.9 | 14.9, 274 tiles 18.7 | 16.7, 375 tiles 19.0 | 25.4).
+// FP32 leapfrog at p = 4, without a layer as the right-hand side (137 tiles 17.5 | 13.4, 274
+// tiles 18.5 | 14.5, 375 tiles 16.9 | 23.0), with one up to one tile per pair of SMs (41
+// tiles 15.2 | 14.1, 94 tiles 18.2 | 19.1).
+// FP32 at p = 5, penalty and right-hand side up to one tile per pair of SMs, the penalty on
+// rows without a bulk copy up to one per SM: 255 registers per thread instead of 128, and all
+// gathers in flight at once (penalty 41 tiles 27.5 | 20.7, 94 tiles 31.6 | 33.4, 137 tiles without
+// a bulk copy 41.7 | 35.2; right-hand side with a PML 41 tiles 25.1 | 23.2, 137 tiles 29.2 |
+// 28.9).  (The code exceeds the instruction cache, and from one tile per pair on the two SMs of
+// a pair share the way it comes.)
+constexpr int64_t kSMs = 152, kClusterTiles = kSMs / 4, kHalfTiles = kSMs / 2;
 
 template <int MODE>
 int launch_mode(const StageParams& prm, cudaStream_t st) {
     const int64_t C = prm.K_active * prm.S;   // columns updated
     if (C <= 0) return DGM_OK;
-    constexpr int kTE = Shape<MODE, false, false>::TE;   // (the same for every shape of a mode)
-    const unsigned grid = unsigned((C + kTE - 1) / kTE);
+    const int64_t tiles = (C + 31) / 32;
     StageParams q = prm;
     q.dt_f = float(prm.dt);
     q.a_f = float(prm.a);
     q.b_f = float(prm.b);
     const bool i32 = !q.force_index64 && fits_32bit(q);
-    // the tile's bulk copy: the plan's tensor-map set of this tile width and the
-    // map of this stage's input
-    q.tm_u = -1;
-    if (q.tmaps != nullptr) {
-        constexpr int kSet = kTE == tmap_columns(0) ? 0 : 1;
-        static_assert(kTE == tmap_columns(kSet), "a tensor-map set of this tile width");
-        q.tmaps = static_cast<const char*>(q.tmaps) + size_t(kSet) * TMAP_COUNT * TMAP_BYTES;
-        q.tm_u = q.u == q.tm_f0 ? TM_U0
-                 : q.u == q.tm_f1 ? TM_U1
-                 : (q.tm_fw != nullptr && q.u == q.tm_fw) ? TM_UW : -1;
-    }
+    const bool layer = q.pml != nullptr && q.npml > 0;
+    constexpr bool kLF = MODE == MODE_LF_E || MODE == MODE_LF_H;
     if (q.hs != nullptr) {   // interior penalty
-        if constexpr (kSIP && (MODE == MODE_LSRK || MODE == MODE_RHS)) {
-            return i32 ? launch_ix<MODE, uint32_t, true, false>(q, grid, st) : launch_ix<MODE, int64_t, true, false>(q, grid, st);
+        if constexpr (kDefault && !kMX && !kLF) {
+            if constexpr (sizeof(Real) == 4 && kP == 5) {
+                if (i32 && tiles <= (tile_map(q) < 0 ? kSMs : kSMs / 2))
+                    return launch_shape<32, 8, MODE, uint32_t, true, false, 1>(q, C, st);
+            }
+            return i32 ? launch_ix<MODE, uint32_t, true, false>(q, C, st) : launch_ix<MODE, int64_t, true, false>(q, C, st);
         } else {
             return DGM_EUNSUP;
         }
     }
-    if constexpr (sizeof(Real) == 8 && !kMX && MODE != MODE_RHS) {
-        if (i32 && grid <= kClusterTiles) return launch_cluster<MODE>(q, grid, st);
+    if constexpr (sizeof(Real) == 8 && !kMX) {
+        if constexpr (MODE != MODE_RHS) {
+            if (i32 && tiles <= kClusterTiles) return launch_shape<32, 8, MODE, uint32_t, false, true, 1, 8>(q, C, st);
+        }
+        if constexpr (!kLF) {
+            if (i32 && tiles <= kHalfTiles) return launch_shape<16, 8, MODE, uint32_t, false, true, 1>(q, C, st);
+        }
+    }
+    if constexpr (sizeof(Real) == 4 && !kMX && MODE == MODE_RHS && kP >= 3) {
+        constexpr int64_t kTiles = kP == 3 ? kSMs : kP == 4 ? 2 * kSMs : kSMs / 2;
+        constexpr int kMinB = kP == 5 ? 1 : 2;
+        if (i32 && tiles <= kTiles)
+            return layer ? launch_shape<32, 8, MODE, uint32_t, false, true, kMinB>(q, C, st)
+                         : launch_shape<32, 8, MODE, uint32_t, false, false, kMinB>(q, C, st);
+    }
+    if constexpr (sizeof(Real) == 4 && !kMX && kLF && kP == 4) {
+        if (i32 && !layer && tiles <= 2 * kSMs) return launch_shape<32, 8, MODE, uint32_t, false, false, 2>(q, C, st);
+        if (i32 && layer && tiles <= kSMs / 2) return launch_shape<32, 8, MODE, uint32_t, false, true, 2>(q, C, st);
     }
     // (64-bit indices: the PML instantiation serves plans without a layer too)
-    if (!i32) return launch_ix<MODE, int64_t, false, !kMX>(q, grid, st);
+    if (!i32) return launch_ix<MODE, int64_t, false, !kMX>(q, C, st);
     if constexpr (!kMX) {
-        if (q.pml != nullptr && q.npml > 0) return launch_ix<MODE, uint32_t, false, true>(q, grid, st);
+        if (layer) return launch_ix<MODE, uint32_t, false, true>(q, C, st);
     }
-    return launch_ix<MODE, uint32_t, false, false>(q, grid, st);
+    return launch_ix<MODE, uint32_t, false, false>(q, C, st);
 }
 
 }  // namespace
