@@ -9,6 +9,8 @@
 #include <string>
 #include <vector>
 
+#include "dgm_once.h"
+
 namespace dgm {
 
 constexpr int PMAX = 5;
@@ -139,6 +141,17 @@ struct StageParams {
     // plan's tables are read before that wait, so the first launch of a call is 0.
     int32_t pdl;
 };
+
+// Opt-in of kernel `k` to `smem` bytes of dynamic shared memory on the current device.
+template <typename K>
+inline bool opt_in_smem(K k, size_t smem, OncePerDevice& once) {
+    int device = -1;
+    const bool ok = cudaGetDevice(&device) == cudaSuccess && once.ensure(device, [&] {
+        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) == cudaSuccess;
+    });
+    if (!ok) cudaGetLastError();
+    return ok;
+}
 
 // Launch of `k` in clusters of `cluster` CTAs, with the programmatic-dependent-launch
 // attribute when pdl is set.

@@ -46,14 +46,9 @@ constexpr int kNTA = sizeof(Real) == 8 ? 192 : 384;
 template <typename IX>
 int launch_adj_ix(const AdjParams& prm, unsigned grid, cudaStream_t st) {
     constexpr size_t smem = adjoint_smem_bytes<kP, Real, kTEA, kNTA>();
-    static bool configured = false;
+    static OncePerDevice once;
     auto k = adjoint_kernel<kP, Real, kTEA, kNTA, IX>;
-    if (!configured) {
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
-            cudaSuccess)
-            return DGM_ECUDA;
-        configured = true;
-    }
+    if (!opt_in_smem(k, smem, once)) return DGM_ECUDA;
     k<<<grid, kNTA, smem, st>>>(prm);
     return cudaGetLastError() == cudaSuccess ? DGM_OK : DGM_ECUDA;
 }
@@ -83,14 +78,9 @@ template <typename IX>
 int launch_pair_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
     using Pair = DGM_PAIR;
     constexpr size_t smem = stage2_smem_bytes<kP, Pair>();
-    static bool configured = false;
+    static OncePerDevice once;
     auto k = stage2_kernel<kP, Pair, kNT, IX>;
-    if (!configured) {
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
-            cudaSuccess)
-            return DGM_ECUDA;
-        configured = true;
-    }
+    if (!opt_in_smem(k, smem, once)) return DGM_ECUDA;
     k<<<grid, kNT, smem, st>>>(q);
     return cudaGetLastError() == cudaSuccess ? DGM_OK : DGM_ECUDA;
 }
@@ -120,14 +110,9 @@ int launch_mode(const StageParams& prm, cudaStream_t st) {
 template <int MODE, typename IX>
 int launch_lf_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
     constexpr size_t smem = lf_smem_bytes<kP, Real, 32>();
-    static bool configured = false;
+    static OncePerDevice once;
     auto k = lf_kernel<kP, Real, 32, MODE, IX>;
-    if (!configured) {
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
-            cudaSuccess)
-            return DGM_ECUDA;
-        configured = true;
-    }
+    if (!opt_in_smem(k, smem, once)) return DGM_ECUDA;
     return launch_ex(k, grid, 32 * LF_NG, smem, st, q.pdl != 0, 1, q) == cudaSuccess ? DGM_OK : DGM_ECUDA;
 }
 
@@ -155,15 +140,10 @@ int launch_mode(const StageParams& prm, cudaStream_t st) {
 template <typename IX, bool PML>
 int launch_ix(const StageParams& q, unsigned grid, cudaStream_t st) {
     constexpr size_t smem = stage_smem_bytes<kP, Real, kTE, kTC>();
-    static bool configured = false;
+    static OncePerDevice once;
     auto k = stage_kernel<kP, Real, kTE, kNT, DGM_MODE, IX, kTC, PML>;
     if (kTC && q.tc_b == nullptr) return DGM_EUNSUP;   // no operator image for this plan
-    if (!configured) {
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
-            cudaSuccess)
-            return DGM_ECUDA;
-        configured = true;
-    }
+    if (!opt_in_smem(k, smem, once)) return DGM_ECUDA;
     k<<<grid, kNT, smem, st>>>(q);
     return cudaGetLastError() == cudaSuccess ? DGM_OK : DGM_ECUDA;
 }

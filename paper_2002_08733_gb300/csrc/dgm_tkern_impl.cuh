@@ -64,14 +64,9 @@ int tile_map(const StageParams& q) {
 template <int TE, int NG, int MODE, typename IX, bool SIP, bool PML, int MINB, int CL = 1>
 int launch_shape(StageParams& q, int64_t columns, cudaStream_t st) {
     constexpr size_t smem = tang_smem_bytes<kP, Real, TE, kMX>();
-    static bool configured = false;
+    static OncePerDevice once;
     auto k = tang_kernel<kP, Real, TE, NG, MODE, IX, SIP, PML, kMX, MINB, CL>;
-    if (!configured) {
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
-            cudaSuccess)
-            return DGM_ECUDA;
-        configured = true;
-    }
+    if (!opt_in_smem(k, smem, once)) return DGM_ECUDA;
     // the plan's tensor-map set of this tile width
     constexpr int kSet = TE == tmap_columns(0) ? 0 : 1;
     static_assert(TE == tmap_columns(kSet), "a tensor-map set of this tile width");

@@ -2,6 +2,7 @@
 import glob
 import os
 import re
+import subprocess
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2002_08733_gb300", "csrc")
 
@@ -17,3 +18,42 @@ def test_no_restrict_name_for_a_buffer_the_kernel_writes():
     for name, text in _sources(".cuh").items():
         bound = re.findall(r"__restrict__\s+\w+\s*=\s*static_cast<[^>]*>\(prm\.(\w+)\)", text)
         assert not bound, (name, bound)
+
+
+def test_launchers_opt_in_to_shared_memory_on_each_device(tmp_path):
+    """The opt-in to more than 48 KB of shared memory holds per device: a plan on a second device
+    needs it too (OncePerDevice), and no launcher remembers it in a plain flag."""
+    for name, text in _sources(".cuh", ".cu").items():
+        assert not re.search(r"static\s+bool\s+\w+\s*=", text), name
+        if "cudaFuncAttributeMaxDynamicSharedMemorySize" in text:
+            assert "OncePerDevice" in text, name
+    src = tmp_path / "once.cpp"
+    src.write_text("""
+#include <cstdio>
+#include <thread>
+#include <vector>
+#include "dgm_once.h"
+int main() {
+    dgm::OncePerDevice o;
+    int calls = 0;
+    auto ok = [&] { ++calls; return true; };
+    auto bad = [&] { ++calls; return false; };
+    if (!o.ensure(0, ok) || !o.ensure(0, ok) || calls != 1) return 1;
+    if (!o.ensure(1, ok) || calls != 2) return 2;                 // another device
+    if (o.ensure(2, bad) || !o.ensure(2, ok) || calls != 4) return 3;   // again after a failure
+    if (!o.ensure(64, ok) || !o.ensure(64, ok) || calls != 6) return 4;  // past what it remembers
+    if (!o.ensure(63, ok) || !o.ensure(63, ok) || calls != 7) return 5;
+    dgm::OncePerDevice m;
+    std::atomic<int> n{0};
+    std::vector<std::thread> t;
+    for (int i = 0; i < 8; ++i)
+        t.emplace_back([&, i] { for (int d = 0; d < 8; ++d) m.ensure((d + i) % 8, [&] { ++n; return true; }); });
+    for (auto& x : t) x.join();
+    const int first = n;
+    for (int d = 0; d < 8; ++d) m.ensure(d, [&] { ++n; return true; });
+    return n == first && first >= 8 ? 0 : 6;
+}
+""")
+    exe = str(tmp_path / "once")
+    subprocess.run(["g++", "-std=c++17", "-pthread", "-I", CSRC, str(src), "-o", exe], check=True)
+    assert subprocess.run([exe]).returncode == 0
