@@ -177,7 +177,11 @@ inline cudaError_t launch_ex(void (*k)(A...), dim3 grid, unsigned block, size_t 
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = n;
-    return cudaLaunchKernelEx(&cfg, k, args...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, args...);
+    // a refused launch also stays the thread's last error, which the next check of an
+    // unrelated call would report
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 // Tensor maps (CUtensorMap, 128 bytes each) of one tile width, all with the
