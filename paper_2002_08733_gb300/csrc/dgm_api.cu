@@ -176,7 +176,7 @@ struct dgm_plan {
     double sip_alpha = 0.0;          // 0: off
     int64_t n_facets = 0;            // interior facets
     size_t off_sfid = 0;             // [4][K] int32: (facet << 1) | owner, or -1
-    size_t off_fcp = 0;              // [FC_ROWS][K] precomputed face constants (plan precision)
+    size_t off_fcp = 0;              // [FC_ROWS][K] precomputed face constants (plan precision; none in mixed orders)
     size_t off_fct = 0;              // [TG_ROWS][K] tangential face constants (plan precision)
     std::vector<int32_t> sfid_host;
     void* hs[2] = {nullptr, nullptr};
@@ -469,8 +469,8 @@ static int plan_create(dgm_plan** out, int64_t nv, const double* xyz, int64_t nt
     P->nbr_plain = P->mesh.nbr;
     P->off_sfid = off;   // facet codes of the interior penalty
     off = align256(off + sizeof(int32_t) * 4 * K);
-    P->off_fcp = off;    // precomputed face constants of the stage kernels
-    off = align256(off + size_t(kt->real_size) * FC_ROWS * K);
+    P->off_fcp = off;    // precomputed face constants of the reference-frame kernels, or the penalty's
+    off = align256(off + (mixed ? 0 : size_t(kt->real_size) * FC_ROWS * K));
     P->off_fct = off;    // constants of the tangential-trace kernels
     off = align256(off + size_t(kt->real_size) * TG_ROWS * K);
     P->off_tmap = off;   // tensor maps of the phase-1 bulk copies
@@ -667,8 +667,10 @@ static int build_face_table(dgm_plan* P) {
     stage_params(P, prm);
     const bool sip = P->sip_alpha > 0.0;
     prm.sfid = sip ? reinterpret_cast<const int32_t*>(P->geom + P->off_sfid) : nullptr;
-    int rc = P->mixed ? DGM_OK : launch_face_consts(prm, P->kt->real_size, P->geom + P->off_fcp, P->stream);
-    if (!rc) rc = launch_tang_consts(prm, P->kt->real_size, sip, P->geom + P->off_fct, P->stream);
+    int rc = P->mixed || sip ? DGM_OK : launch_face_consts(prm, P->kt->real_size, P->geom + P->off_fcp, P->stream);
+    if (!rc)
+        rc = launch_tang_consts(prm, P->kt->real_size, P->geom + P->off_fct, sip ? P->geom + P->off_fcp : nullptr,
+                                P->stream);
     return rc ? fail(rc, "face constants") : DGM_OK;
 }
 

@@ -64,11 +64,10 @@ enum TangConst {
     TG_FACE = 8,                  // rows per face
     TG_METRIC = 4 * TG_FACE,      // A^T A: 00, 01, 02, 11, 12, 22
     TG_IE = TG_METRIC + 6,        // 1 / (eps det A)
-    TG_IH = TG_METRIC + 7,        // -1 / (mu det A)
-    TG_SIP = TG_METRIC + 8,       // interior penalty, per face: KS, A t_1 (3), A t_2 (3)
-    TG_SIPF = 7
+    TG_IH = TG_METRIC + 7         // -1 / (mu det A)
 };
-static_assert(TG_SIP + 4 * TG_SIPF == TG_ROWS, "rows of the tangential face-constant table");
+static_assert(TG_IH + 1 == TG_ROWS, "rows of the tangential face-constant table");
+// interior penalty, a table of its own, per face (TG_SIPF rows): KS, A t_1 (3), A t_2 (3)
 
 // component of tangent i of face f (face 0: minus component 0)
 __host__ __device__ constexpr int tang_comp(int f, int i) { return f == 2 ? 2 * i : (f == 3 ? i : 1 + i); }
@@ -76,7 +75,7 @@ __host__ __device__ constexpr int tang_comp(int f, int i) { return f == 2 ? 2 * 
 // One thread per element, from the FP64 geometry (once per plan, again when the
 // materials or the boundary codes change); rounded to the plan's precision last.
 template <typename R>
-__global__ void tang_consts_kernel(const StageParams prm, bool sip, R* __restrict__ out) {
+__global__ void tang_consts_kernel(const StageParams prm, R* __restrict__ out, R* __restrict__ sip_out) {
     const int64_t K = prm.K;
     const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (e >= K) return;
@@ -124,10 +123,10 @@ __global__ void tang_consts_kernel(const StageParams prm, bool sip, R* __restric
         const double v[TG_FACE] = {sg * ce, sg * ch, kb * be * t11, -kb * be * t12, kb * be * t22,
                                    -kb * bh * t11, kb * bh * t12, -kb * bh * t22};
         for (int k = 0; k < TG_FACE; ++k) out[int64_t(f * TG_FACE + k) * K + e] = R(v[k]);
-        if (sip) {
+        if (sip_out != nullptr) {
             const int32_t sf = prm.sfid[int64_t(f) * K + e];
             const double ks = (sf >= 0 && (sf & 1)) ? prm.sip_alpha / (0.5 * (mu + mun)) * kb : 0.0;
-            R* o = out + int64_t(TG_SIP + f * TG_SIPF) * K + e;
+            R* o = sip_out + int64_t(f * TG_SIPF) * K + e;
             o[0] = R(ks);
             for (int i = 0; i < 2; ++i)
                 for (int r = 0; r < 3; ++r) o[int64_t(1 + 3 * i + r) * K] = R(T[i][r]);
@@ -826,7 +825,7 @@ __global__ void __launch_bounds__(CL > 1 ? TE * CLW : TE * NG, MINB) tang_kernel
                     hsr = MODE == MODE_LSRK ? static_cast<R*>(prm.hs_res) + off : nullptr;
                 }
             }
-            const R* ts = static_cast<const R*>(prm.fct) + IX(TG_SIP + f * TG_SIPF) * K + id.e;
+            const R* ts = static_cast<const R*>(prm.fcp) + IX(f * TG_SIPF) * K + id.e;
             ks = ts[0];
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
