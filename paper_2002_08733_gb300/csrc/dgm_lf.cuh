@@ -4,7 +4,8 @@
 // records are FP64 results formed from FP32 fields.  So every value here is the
 // same chain of operations as in stage_kernel, with what a half step does not
 // need left out: it advances one field from the jumps of the other, the flux is
-// central, and the advanced field enters by its own rows only.
+// central, no face is incident (those need LSRK4), and the advanced field enters by its
+// own rows only.
 //
 // One CTA owns TE consecutive columns, NG = 12 threads per column:
 //   1  tile of the other field; neighbour trace of item (face, component);
@@ -123,10 +124,6 @@ __global__ void __launch_bounds__(TE * LF_NG, 2) lf_kernel(const StageParams prm
 
     // ---- phase 3: central flux g = +-c (m_f x jump of the other field) ------------
     {
-        // incident face (e+ = e- + 2 E_inc): the E jump is the incident term alone
-        const R* inc = (O == 0 && code <= -2 && prm.inc != nullptr && active)
-                           ? static_cast<const R*>(prm.inc) + IX(-code - 2) * NF * 3
-                           : nullptr;
         const R cs = F == 0 ? cc : -cc;
         const int ax = ff - 1;                   // axis of m_f = -e_A; -1 on the slanted face
         for (int m = ch * NF / 3; m < (ch + 1) * NF / 3; ++m) {
@@ -140,7 +137,6 @@ __global__ void __launch_bounds__(TE * LF_NG, 2) lf_kernel(const StageParams prm
                 d[r] = R(0);
                 if (r == ax) continue;
                 d[r] = q[3 * r] * tp[0] + q[3 * r + 1] * tp[1] + q[3 * r + 2] * tp[2] + na * own[r * NF * TE];
-                if (inc != nullptr) d[r] += inc[m * 3 + r];
             }
             // m_f = (1, 1, 1): m x y = (y2 - y1, y0 - y2, y1 - y0); m_f = -e_A:
             // (m x y)_A = 0 (not stored), (m x y)_B = y_CC, (m x y)_CC = -y_B, (A, B, CC) cyclic
