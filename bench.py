@@ -39,26 +39,30 @@ sys.path.insert(0, ROOT)
 import workloads as W  # noqa: E402
 
 METRIC = "DoF-updates/s"
-# FP32 LSRK stage-kernel variants in autotuner order (degree 3 instantiations)
-VARIANT_NAMES = ["32 cols x 384 thr", "32 cols x 192 thr", "16 cols x 192 thr",
+# FP32 LSRK stage-kernel variants in autotuner order (degree 3 instantiations, plans without
+# receivers): the tangential-trace kernel in three shapes, then the reference-frame kernels
+VARIANT_NAMES = ["tangential, 32 cols x 4 threads per column (8 up to 152 tiles)",
+                 "tangential, 32 cols x 8 threads per column", "tangential, 16 cols x 8 threads per column",
                  "64 cols paired x 384 thr, packed FP32x2", "64 cols paired x 384 thr, scalar",
                  "64 cols x 512 thr, curl and lift on tensor cores (tcgen05, 3xTF32)"]
-KERNEL_NAMES = ["stage_kernel<3,float,32,384,LSRK>", "stage_kernel<3,float,32,192,LSRK>",
-                "stage_kernel<3,float,16,192,LSRK>", "stage2_kernel<3,F2x,384>",
+KERNEL_NAMES = ["tang_kernel<3,float,32,4,LSRK>", "tang_kernel<3,float,32,8,LSRK>",
+                "tang_kernel<3,float,16,8,LSRK>", "stage2_kernel<3,F2x,384>",
                 "stage2_kernel<3,P2,384>", "stage_kernel<3,float,64,512,LSRK,TC>"]
 UNIT = "DoF-updates/s"
 
 
 def kernel_name(variant, K, N, S):
-    """The stage kernel a variant launches; single-column shapes use 32-bit index
-    arithmetic when every index fits (the library's own test: field and
-    face-jump rows x columns, geometry, per-face table below 2^32)."""
+    """The stage kernel a variant launches; the tangential-trace and the tensor-core kernel
+    use 32-bit index arithmetic when every index fits (the library's own tests: field rows x
+    columns, geometry, constant tables and, for the latter, face-jump rows below 2^32)."""
+    C = K * S
+    if variant == 0 and -(-C // 32) <= 152:
+        variant = 1
     name = KERNEL_NAMES[variant]
     if variant < 3 or variant == 5:
         NF = {4: 3, 10: 6, 20: 10, 35: 15, 56: 21}[N]
-        C = K * S
-        fits = max(6 * N * C, 24 * NF * C, 16 * K, 52 * K) < 2 ** 32
-        name = name[:-1] + (",unsigned int>" if fits else ",long>")
+        rows = [6 * N * C, 66 * K, 12 * NF * K] + ([24 * NF * C] if variant == 5 else [])
+        name = name[:-1] + (",unsigned int>" if max(rows) < 2 ** 32 else ",long>")
     return name
 
 
@@ -594,24 +598,26 @@ def run_adjoint(steps, n=24):
                 grad_eps_norm=float(eps.grad.norm()), grad_mu_norm=float(mu_p.grad.norm()))
 
 
-TRAFFIC_PROFILE = "stage_kernel_full_jittered_sphere_n28_p3_fp32.md"
+TRAFFIC_PROFILE = "tang_kernel_full_jittered_sphere_n28_p3_fp32.md"
 
 
-def profiled_traffic(path, variant, groups, columns, loads="bulk"):
+def profiled_traffic(path, variant, groups, columns, loads="bulk", kernel=None):
     """DRAM bytes of one stage launch from the committed ncu summary: its line
-    `traffic_bytes_per_element_stage variant=V tile_groups=G loads=L: B` for
-    the tile shape, tile order and phase-1 load path (bulk copies or
-    per-thread loads) this run uses, times the columns; None when the summary
-    has no line for them (counters of another kernel configuration say nothing
-    about this one)."""
+    `traffic_bytes_per_element_stage [kernel=NAME] variant=V tile_groups=G loads=L: B` for
+    the kernel (the name before its template arguments; not compared when `kernel` is
+    None), tile shape, tile order and phase-1 load path (bulk copies or per-thread loads)
+    this run uses, times the columns; None when the summary has no line for them
+    (counters of another kernel or configuration say nothing about this one)."""
     import re
     if not os.path.exists(path):
         return None
     txt = open(path).read()
-    for m in re.finditer(r"traffic_bytes_per_element_stage variant=(\d+) tile_groups=(\d+)"
+    for m in re.finditer(r"traffic_bytes_per_element_stage(?: kernel=(\w+))? variant=(\d+) tile_groups=(\d+)"
                          r" loads=(\w+):\s*(\d+)", txt):
-        if int(m.group(1)) == variant and int(m.group(2)) == groups and m.group(3) == loads:
-            return int(m.group(4)) * columns
+        if kernel is not None and m.group(1) != kernel.split("<")[0]:
+            continue
+        if int(m.group(2)) == variant and int(m.group(3)) == groups and m.group(4) == loads:
+            return int(m.group(5)) * columns
     return None
 
 
@@ -882,8 +888,9 @@ def main():
     chosen = (r32["tuned"] or {}).get("variant", 0)
     groups = (r32["tuned"] or {}).get("tile_groups", 1)
     loads = "bulk" if (r32["tuned"] or {}).get("bulk_tile_loads", False) else "per_thread"
+    kernel = kernel_name(chosen, r32["K"], r32["N"], r32["S"])
     traffic = profiled_traffic(os.path.join(ROOT, "profiles", TRAFFIC_PROFILE), chosen, groups,
-                               r32["K"] * r32["S"], loads)
+                               r32["K"] * r32["S"], loads, kernel)
     line = {
         "metric": METRIC, "value": r32["value"], "unit": UNIT, "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": r32["ms"] / args.steps,
@@ -892,7 +899,7 @@ def main():
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                      "frac": achieved / hbm, "traffic": traffic,
                      "peak_source": peak_src,
-                     "kernel": kernel_name(chosen, r32["K"], r32["N"], r32["S"]),
+                     "kernel": kernel,
                      "algorithmic_bytes_per_launch": bytes_step / 5},
         "fp64": {"value": r64["value"], "ms_per_step": r64["ms"] / r64["steps"],
                  "steps": r64["steps"], "dtype": "f64"},
@@ -928,8 +935,7 @@ def main():
     if not args.no_mixed and world == 1:
         line["mixed_orders"] = dict(
             workload="jittered sphere mesh (%d^3, %d tets), E of degree 3 and H of degree 2 "
-                     "(Sec. III), upwind, LSRK4, the same pulse; plain one-thread-per-column "
-                     "kernel with dense operators" % (args.n, w.K),
+                     "(Sec. III), upwind, LSRK4, the same pulse" % (args.n, w.K),
             fp32=run_mixed("fp32", args.mixed_steps, 2, n=args.n),
             fp64=run_mixed("fp64", min(args.mixed_steps, 3), 1, n=args.n))
     if not args.no_boundary and world == 1:

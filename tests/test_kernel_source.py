@@ -57,3 +57,22 @@ int main() {
     exe = str(tmp_path / "once")
     subprocess.run(["g++", "-std=c++17", "-pthread", "-I", CSRC, str(src), "-o", exe], check=True)
     assert subprocess.run([exe]).returncode == 0
+
+
+def test_bench_names_the_kernel_it_times(tmp_path):
+    """Counters of one kernel are not reported beside another."""
+    import sys
+    sys.path.insert(0, os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    import bench
+    name = bench.kernel_name(0, 196608, 20, 1)
+    assert name == "tang_kernel<3,float,32,4,LSRK,unsigned int>"
+    assert bench.kernel_name(0, 1296, 20, 1).startswith("tang_kernel<3,float,32,8,")
+    assert bench.kernel_name(5, 196608, 20, 1).startswith("stage_kernel<")
+    f = tmp_path / "p.md"
+    f.write_text("traffic_bytes_per_element_stage variant=0 tile_groups=6 loads=bulk: 2034\n"
+                 "traffic_bytes_per_element_stage kernel=tang_kernel variant=0 tile_groups=12 loads=bulk: 1800\n")
+    assert bench.profiled_traffic(str(f), 0, 6, 10, "bulk", name) is None
+    assert bench.profiled_traffic(str(f), 0, 12, 10, "bulk", name) == 18000
+    assert bench.profiled_traffic(str(f), 0, 12, 10, "bulk", "stage_kernel<3>") is None
+    committed = os.path.join(os.path.dirname(CSRC), "..", "profiles", bench.TRAFFIC_PROFILE)
+    assert bench.profiled_traffic(committed, 0, 6, 196608, "bulk", name) is not None
