@@ -249,13 +249,14 @@ int dgm_set_variant(dgm_plan* plan, int32_t variant);
  * always, to check that path on problems of any size.  Results are the same
  * either way.  DGM_EINVAL for other values. */
 int dgm_set_index64(dgm_plan* plan, int32_t force);
-/* How the single-column stage kernels bring a tile's coefficients, element
- * constants and face constants into shared memory.  Where the plan allows it
- * (one column per element, S = 1; rows of the field and table buffers on
- * 16-byte boundaries, i.e. K a multiple of 4 in FP32 and of 2 in FP64; the
- * stage reads one of the two bound field buffers) dgm_bind builds tensor maps
- * and phase 1 moves the tile with a few tiled bulk copies (TMA) issued by one
- * thread; otherwise every thread loads and stores its share of rows.
+/* How the single-column stage kernels bring a tile's coefficients (and the
+ * reference-frame kernel its element and face constants) into shared memory.
+ * Where the plan allows it (rows of the field and table buffers on 16-byte
+ * boundaries, i.e. K S a multiple of 4 in FP32 and of 2 in FP64, and with several
+ * columns per element S itself; the stage reads one of the two bound field
+ * buffers) dgm_bind builds tensor maps and the tile arrives by tiled bulk copies
+ * (TMA) issued by one thread; otherwise every thread brings its share of rows, as
+ * it also does where several thread blocks share a tile (small FP64 meshes).
  * per_thread = 1 forces the per-thread loads, 0 (the default) restores the
  * automatic choice; the results are the same bits either way.  DGM_EINVAL for
  * other values.  dgm_get_tile_loads sets *bulk to 1 when the next stages of a
@@ -270,7 +271,8 @@ int dgm_get_tile_loads(const dgm_plan* plan, int32_t* bulk);
  * neighbours' coefficients of meshes numbered in G blocks (e.g. a Kuhn grid
  * numbered by tetrahedron type) in L2; 1 = plain order.  Results do not
  * depend on it.  A new plan takes the order that brings most face neighbours
- * close together.  dgm_autotune picks it after the tile shape: the fastest of
+ * close together (with the penalty at p = 5 the
+ * plain one).  dgm_autotune picks it after the tile shape: the fastest of
  * 1, 2, 3, 4, 6, 8, 12, or 1 unless that is at least 1 % faster than the plain
  * order; DGM_EINVAL outside 1..64. */
 int dgm_set_tile_groups(dgm_plan* plan, int32_t groups);

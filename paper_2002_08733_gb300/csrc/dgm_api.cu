@@ -163,6 +163,8 @@ struct dgm_plan {
     int variant = 0;          // LSRK stage tile shape chosen by dgm_autotune
     int force_index64 = 0;    // dgm_set_index64
     int tile_groups = 1;      // tile visiting order (dgm_autotune, dgm_set_tile_groups)
+    int mesh_groups = 1;      // the order chosen from the mesh (choose_tile_groups)
+    bool own_groups = false;  // tile_groups is the caller's
     int64_t k_active = 0;     // elements updated (dgm_set_active); the rest are halo copies
     float variant_ms[8] = {0};
     // incident plane wave (dgm_set_incident)
@@ -477,8 +479,9 @@ static int plan_create(dgm_plan** out, int64_t nv, const double* xyz, int64_t nt
     off = align256(off + size_t(TMAP_SETS) * TMAP_COUNT * TMAP_BYTES);
     P->bytes_geom = off;
     P->k_active = K;
-    P->tile_groups = choose_tile_groups(P->mesh, opt->n_columns, kt->real_size,
-                                        size_t(opt->integrator == DGM_LEAPFROG ? 3 : 6) * P->N * K * Sc * kt->real_size);
+    P->tile_groups = P->mesh_groups =
+        choose_tile_groups(P->mesh, opt->n_columns, kt->real_size,
+                           size_t(opt->integrator == DGM_LEAPFROG ? 3 : 6) * P->N * K * Sc * kt->real_size);
     P->src_host.assign(size_t(Sc) * (SRC_HDR + 3 * P->N), 0.0);
     for (int s = 0; s < Sc; ++s) P->src_host[size_t(s) * (SRC_HDR + 3 * P->N)] = -1.0;
     *out = P;
@@ -1257,6 +1260,11 @@ int dgm_set_sip(dgm_plan* P, double alpha) {
     }
     const int64_t K = P->mesh.K;
     P->sip_alpha = alpha;
+    // At p = 5 with the penalty the plain order: the facets of a tile's elements are
+    // numbered side by side, and the interleaved order takes them from each other (us per
+    // stage, plain | six segments: 16^3, 8 columns 1031 | 1655, 22^3 370 | 509; p = 4, 12^3, 16
+    // columns 357 | 318, p = 3, 13^3, 16 columns 218 | 199).
+    if (!P->own_groups) P->tile_groups = alpha > 0.0 && P->opt.p == 5 ? 1 : P->mesh_groups;
     P->n_facets = 0;
     P->sfid_host.assign(size_t(4) * K, -1);
     if (alpha == 0.0) return DGM_OK;
@@ -2107,6 +2115,7 @@ extern "C" int dgm_set_tile_groups(dgm_plan* P, int32_t groups) {
     if (!P) return fail(DGM_EINVAL, "null plan");
     if (groups < 1 || groups > 64) return fail(DGM_EINVAL, "tile groups must be 1..64");
     P->tile_groups = groups;
+    P->own_groups = true;
     return DGM_OK;
 }
 
