@@ -140,7 +140,8 @@ __device__ __host__ constexpr size_t adjoint_smem_bytes() {
 // IX: index type (uint32_t when every index of the plan fits, else int64_t)
 // The stage also forms the next stage's residual (in another buffer: neighbours still
 // read this one), which as a pass of its own read both vectors again.
-// It is bound by latency: 24 warps per SM, 49 k thread instructions per column at p = 3.
+// It is bound by latency: 20.6 warps per SM, long-scoreboard stalls first, 61 k thread
+// instructions per column at p = 3 (12^3 grid with a PML, 8 columns).
 // Gradient of the 24^3 inverse problem with a PML, 8 columns, 4 steps: 98.0 ms with the
 // rows of phase 5 one by one and the residual as its own pass, 82.8 ms so.
 template <int P, typename R, int TE, int NT, typename IX = int64_t>

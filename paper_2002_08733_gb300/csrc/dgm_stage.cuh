@@ -523,7 +523,7 @@ stage_kernel(const StageParams prm) {
     const bool active = col < IX(prm.K_active) * IX(S);
     const IX e = active ? col / S : 0;
     const int s = active ? int(col - e * S) : 0;
-    const R* u = static_cast<const R*>(prm.u);   // may alias u_out (leapfrog)
+    const R* u = static_cast<const R*>(prm.u);
     const R* gr = static_cast<const R*>(prm.geo_r);
     // stage coefficients in the kernel's precision: FP32 kernels read the FP32
     // copies, so that no conversion runs on the FP64 pipe
@@ -600,8 +600,8 @@ stage_kernel(const StageParams prm) {
         request_nbr(grp, code0, vn);
         request_nbr(grp + NG, code1, vn1);
     } else {
-        // rows q: [0, 6N) coefficients, then EG element constants, 4 FGRT face
-        // constants, GM metric rows and (penalty) GA rows of A^T
+        // rows q: [0, 6N) coefficients, then EG element constants, 4 FGR face
+        // constants and GM metric rows
         constexpr int Q0 = 6 * N, Q1 = Q0 + EG, Q2 = Q1 + 4 * FGR, Q3 = Q2 + GM;
         constexpr int T1 = Q3;
         constexpr int UR = (T1 + NG - 1) / NG;          // rows per thread (at most)

@@ -34,7 +34,7 @@
 //     and the stage update, so the right-hand side never leaves the registers.
 // One barrier between the two (and one before phase A for the tile).
 //
-// What bounds it.  FP64: the FP64 pipe (88 % of its rate at 48,000 elements,
+// What bounds it.  FP64: the FP64 pipe (84 % of its rate at 48,000 elements,
 // p = 3); the tangential form needs 6.1 k operations per element-stage instead of
 // about 10 k, and with full warps of 32 columns no warp runs two row parts in
 // turn: 22.8 -> 11.9 ms per LSRK4 step of the 32^3 grid.  FP32: instruction issue

@@ -29,7 +29,7 @@ struct Shape {
     // trace's coefficients fit its registers, eight from p = 5 on, and at p = 4
     // with the penalty's facet values besides.  (p = 4 with a PML, LSRK4, us, eight
     // threads on 80 registers | four on 168: 250 tiles of 32 columns 47.4 | 27.9, 768 tiles
-    // 118 | 62.7; right-hand side of 999 tiles 110 | 64.7)
+    // 118 | 62.7, 12,000 tiles 2405 | 1079; right-hand side of 999 tiles 110 | 64.7)
     // FP64 (bound by the FP64 pipe, which few warps saturate): full warps of 32
     // columns, so that no warp runs two faces or row parts in turn.
     static constexpr int TE = 32;
