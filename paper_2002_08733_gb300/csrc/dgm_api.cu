@@ -671,9 +671,7 @@ static int build_face_table(dgm_plan* P) {
     const bool sip = P->sip_alpha > 0.0;
     prm.sfid = sip ? reinterpret_cast<const int32_t*>(P->geom + P->off_sfid) : nullptr;
     int rc = P->mixed || sip ? DGM_OK : launch_face_consts(prm, P->kt->real_size, P->geom + P->off_fcp, P->stream);
-    if (!rc)
-        rc = launch_tang_consts(prm, P->kt->real_size, P->geom + P->off_fct, sip ? P->geom + P->off_fcp : nullptr,
-                                P->stream);
+    if (!rc) rc = launch_tang_consts(prm, P->kt->real_size, sip, P->geom + P->off_fct, P->stream);
     return rc ? fail(rc, "face constants") : DGM_OK;
 }
 

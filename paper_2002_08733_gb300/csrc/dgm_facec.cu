@@ -19,12 +19,12 @@ int launch_face_consts(const StageParams& prm, int real_size, void* out, void* s
     return cudaGetLastError() == cudaSuccess ? DGM_OK : DGM_ECUDA;
 }
 
-int launch_tang_consts(const StageParams& prm, int real_size, void* out, void* sip_out, void* stream) {
+int launch_tang_consts(const StageParams& prm, int real_size, bool sip, void* out, void* stream) {
     if (prm.K <= 0) return DGM_OK;
     const unsigned grid = unsigned((prm.K + 127) / 128);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (real_size == 8) tang_consts_kernel<double><<<grid, 128, 0, st>>>(prm, static_cast<double*>(out), static_cast<double*>(sip_out));
-    else tang_consts_kernel<float><<<grid, 128, 0, st>>>(prm, static_cast<float*>(out), static_cast<float*>(sip_out));
+    if (real_size == 8) tang_consts_kernel<double><<<grid, 128, 0, st>>>(prm, sip, static_cast<double*>(out));
+    else tang_consts_kernel<float><<<grid, 128, 0, st>>>(prm, sip, static_cast<float*>(out));
     return cudaGetLastError() == cudaSuccess ? DGM_OK : DGM_ECUDA;
 }
 

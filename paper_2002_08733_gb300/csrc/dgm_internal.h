@@ -208,13 +208,13 @@ constexpr int FC_ROWS = 4 * 15 + 6;
 // Computes them for a plan (dgm_facec.cu); real_size 4 or 8.
 int launch_face_consts(const StageParams& prm, int real_size, void* out, void* stream);
 // Rows per element of the tangential face-constant table (dgm_tang.cuh): per face
-// 8, the metric A^T A (6), two mass factors; and its launcher.  The penalty's 4 x 7 rows
-// (sip_out, null without it) take the place of the face constants above, which only
-// the reference-frame kernels read and no plan with the penalty runs.
+// 8, the metric A^T A (6), two mass factors; and its launcher.  With the penalty (sip) its
+// 4 x 7 rows go to prm.fcp, in the place of the face constants above, which only the
+// reference-frame kernels read and no plan with the penalty runs.
 constexpr int TG_ROWS = 4 * 8 + 6 + 2;
 constexpr int TG_SIPF = 7;
 static_assert(4 * TG_SIPF <= FC_ROWS, "the penalty's rows fit the face-constant table");
-int launch_tang_consts(const StageParams& prm, int real_size, void* out, void* sip_out, void* stream);
+int launch_tang_consts(const StageParams& prm, int real_size, bool sip, void* out, void* stream);
 
 // One adjoint stage: lu += dt F_u^T lr, and the material-gradient terms
 // dt lr . (dF/d eps_T, dF/d mu_T) u at the stage input u (per column).

@@ -75,7 +75,7 @@ __host__ __device__ constexpr int tang_comp(int f, int i) { return f == 2 ? 2 * 
 // One thread per element, from the FP64 geometry (once per plan, again when the
 // materials or the boundary codes change); rounded to the plan's precision last.
 template <typename R>
-__global__ void tang_consts_kernel(const StageParams prm, R* __restrict__ out, R* __restrict__ sip_out) {
+__global__ void tang_consts_kernel(const StageParams prm, bool sip, R* __restrict__ out) {
     const int64_t K = prm.K;
     const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (e >= K) return;
@@ -123,10 +123,10 @@ __global__ void tang_consts_kernel(const StageParams prm, R* __restrict__ out, R
         const double v[TG_FACE] = {sg * ce, sg * ch, kb * be * t11, -kb * be * t12, kb * be * t22,
                                    -kb * bh * t11, kb * bh * t12, -kb * bh * t22};
         for (int k = 0; k < TG_FACE; ++k) out[int64_t(f * TG_FACE + k) * K + e] = R(v[k]);
-        if (sip_out != nullptr) {
+        if (sip) {
             const int32_t sf = prm.sfid[int64_t(f) * K + e];
             const double ks = (sf >= 0 && (sf & 1)) ? prm.sip_alpha / (0.5 * (mu + mun)) * kb : 0.0;
-            R* o = sip_out + int64_t(f * TG_SIPF) * K + e;
+            R* o = const_cast<R*>(static_cast<const R*>(prm.fcp)) + int64_t(f * TG_SIPF) * K + e;
             o[0] = R(ks);
             for (int i = 0; i < 2; ++i)
                 for (int r = 0; r < 3; ++r) o[int64_t(1 + 3 * i + r) * K] = R(T[i][r]);
