@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import concurrent.futures as cf
 import os
+import platform
 import shutil
 import subprocess
 import sys
@@ -17,7 +18,10 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
-GEN = os.path.join(BUILD, "gen")
+# The generated operators belong to the machine that generated them: the last bits of their
+# literals follow its compiler (whether products and sums are fused), so a tree that moves
+# to another architecture generates its own.
+GEN = os.path.join(BUILD, "gen_" + platform.machine())
 GEN_HEADER = os.path.join(GEN, "dgm_ops_gen.cuh")
 GENERATOR_SRC = ("dgm_refgen.cpp", "dgm_refmats.cpp")
 LIBDIR = os.path.join(PKG, "_lib")

@@ -76,3 +76,19 @@ def test_bench_names_the_kernel_it_times(tmp_path):
     assert bench.profiled_traffic(str(f), 0, 12, 10, "bulk", "stage_kernel<3>") is None
     committed = os.path.join(os.path.dirname(CSRC), "..", "profiles", bench.TRAFFIC_PROFILE)
     assert bench.profiled_traffic(committed, 0, 6, 196608, "bulk", name) is not None
+
+
+def test_generated_operators_belong_to_the_machine(monkeypatch):
+    """A header generated on one architecture is not taken on another, whose compiler rounds the
+    literals differently in the last bit."""
+    import importlib
+    import platform
+    from paper_2002_08733_gb300 import build as B
+    here = B.GEN_HEADER
+    try:
+        monkeypatch.setattr(platform, "machine", lambda: "another")
+        assert importlib.reload(B).GEN_HEADER != here
+    finally:
+        monkeypatch.undo()
+        importlib.reload(B)
+    assert B.GEN_HEADER == here
